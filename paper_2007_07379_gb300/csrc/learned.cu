@@ -84,12 +84,23 @@ __host__ __device__ inline int suffix_start(uint64_t seed, uint32_t move, int d)
 
 // The start of a move: unslice as above, and (thread 0) the suffix start k*
 // from the seed and the move count (SplitMix64, so that one captured graph
-// serves every move), and the proposal's log q sums cleared.
+// serves every move), and the proposal's log q sums cleared.  In a learned
+// run's device-side loop (hdr != nullptr) thread 0 also counts the loop's
+// period down and tells the graph's while node whether another follows (the
+// node looks when the whole body has run).
 __global__ void move_begin_kernel(const uint32_t* __restrict__ state, int n, int d, uint32_t groups,
                                   uint32_t* __restrict__ P, MhCounters* __restrict__ ctr, uint64_t seed,
-                                  float* __restrict__ lqf, uint32_t chains) {
+                                  float* __restrict__ lqf, uint32_t chains, WsHeader* hdr,
+                                  cudaGraphConditionalHandle loop) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0) ctr->k = suffix_start(seed, ctr->moves, d);
+  if (i == 0) {
+    ctr->k = suffix_start(seed, ctr->moves, d);
+    if (hdr) {
+      const uint32_t left = hdr->periods_left - 1u;
+      hdr->periods_left = left;
+      cudaGraphSetConditional(loop, left > 0u ? 1u : 0u);
+    }
+  }
   if (i < chains) lqf[i] = 0.f;
   const uint32_t w = i >> 5;
   const int lane = threadIdx.x & 31;
@@ -98,25 +109,6 @@ __global__ void move_begin_kernel(const uint32_t* __restrict__ state, int n, int
   const uint32_t x = lane < n ? state[((size_t)g * d + j) * n + lane] : 0u;
   const uint32_t y = warp_transpose(x, lane);
   P[(size_t)(g * 32 + lane) * d + j] = y;
-}
-
-// Per-chain words -> bit-sliced words for layers k..d (1-based), k read from
-// k_dev; one warp per (group, layer) over all d layers, the warps of layers
-// before k leave at once.
-__global__ void slice_kernel(const uint32_t* __restrict__ P, int n, int d, MhCounters* __restrict__ ctr,
-                             uint32_t groups, uint32_t* __restrict__ state) {
-  const uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  const int* k_dev = &ctr->k;
-  // the end of the move: its count (read by no kernel of this move after
-  // the acceptance, which ran before)
-  if (blockIdx.x == 0 && threadIdx.x == 0) ctr->moves += 1u;
-  if (w >= groups * (uint32_t)d) return;
-  const uint32_t g = w / d, j = w % d;
-  if ((int)j + 1 < *k_dev) return;  // the whole warp: layer j+1 is before the suffix
-  const uint32_t x = P[(size_t)(g * 32 + lane) * d + j];
-  const uint32_t y = warp_transpose(x, lane);
-  if (lane < n) state[((size_t)g * d + j) * n + lane] = y;
 }
 
 // Row x = [2 s_{j-1} - 1 (n), onehot(j-1) (d), 0...] in bf16, written in
@@ -215,57 +207,82 @@ __global__ void sample_kernel(const float* __restrict__ logits, int npad, int n,
 }
 
 // Violation counts of layers k..d for the current and proposed suffix, the
-// Metropolis-Hastings decision, and the accepted suffix copied into P.  One
+// Metropolis-Hastings decision, and the suffix that stands sliced back into
+// the chain words: the end of a move in one launch.  One CTA per group, one
 // warp per chain: lane l takes layers k + l, k + l + 32, ...; the warp sums
-// the counts and the log q terms (a fixed tree), lane 0 decides.
-__global__ void accept_kernel(uint32_t* __restrict__ P, const uint32_t* __restrict__ Pn,
-                              const LayerTab* __restrict__ tab, uint32_t beta, uint32_t nmask,
-                              int d, float J, const float* __restrict__ lq,
-                              const float* __restrict__ lqf, uint32_t chains, uint32_t k0,
-                              uint32_t k1, MhCounters* __restrict__ ctr, uint32_t group0) {
+// the counts and the log q terms (a fixed tree), lane 0 decides; the chains'
+// words meet in shared memory, and warp w transposes layers k + w, k + w +
+// 32, ...  The last CTA counts the move.
+constexpr int kMaxLayers = 64;
+__global__ void __launch_bounds__(1024) accept_slice_kernel(
+    const uint32_t* __restrict__ P, const uint32_t* __restrict__ Pn,
+    const LayerTab* __restrict__ tab, uint32_t beta, uint32_t nmask, int n, int d, float J,
+    const float* __restrict__ lq, const float* __restrict__ lqf, uint32_t chains, uint32_t k0,
+    uint32_t k1, MhCounters* __restrict__ ctr, uint32_t* __restrict__ ticket, uint32_t group0,
+    uint32_t* __restrict__ state) {
+  __shared__ uint32_t words[kMaxLayers][33];
   __shared__ uint32_t n_acc;
   if (threadIdx.x == 0) n_acc = 0u;
   __syncthreads();
-  const uint32_t c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t g = blockIdx.x, c = g * 32u + (uint32_t)warp;
   const bool in = c < chains;  // warp-uniform
   const uint32_t move = ctr->moves;
   const int k = ctr->k;
-  bool acc = false;
-  if (in) {
-    const uint32_t* cur = P + (size_t)c * d;
-    const uint32_t* prop = Pn + (size_t)c * d;
-    int v = 0, vn = 0;
-    float lrev = 0.f;
-    for (int j = k + lane; j <= d; j += 32) {
-      const LayerTab& L = tab[j - 1];
-      const uint32_t link = ~L.hmask & nmask;
-      const uint32_t pc = j == 1 ? beta : cur[j - 2];   // s_{j-1}
-      const uint32_t pn = j == k ? pc : prop[j - 2];    // s'_{j-1}, s'_{k-1} = s_{k-1}
-      v += __popc((cur[j - 1] ^ layer_map(L, pc)) & link);
-      vn += __popc((prop[j - 1] ^ layer_map(L, pn)) & link);
-      lrev += lq[(size_t)c * d + (j - 1)];
-    }
+  const uint32_t* cur = P + (size_t)c * d;
+  const uint32_t* prop = Pn + (size_t)c * d;
+  uint32_t sc[2] = {0u, 0u}, sp[2] = {0u, 0u};  // this lane's layers, current and proposed
+  int v = 0, vn = 0;
+  float lrev = 0.f;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      v += __shfl_xor_sync(0xffffffffu, v, off);
-      vn += __shfl_xor_sync(0xffffffffu, vn, off);
-      lrev += __shfl_xor_sync(0xffffffffu, lrev, off);
-    }
-    if (lane == 0) {
-      const float logA = -J * (float)(vn - v) + lrev - lqf[c];
-      const uint32_t gc = group0 * 32u + c;
-      const uint32_t u = philox4x32_10(make_uint4(gc, move, 0xFFFFu | (kTagMH << 16), 0u), k0, k1).x;
-      const float uf = ((float)(u >> 8) + 0.5f) * (1.f / 16777216.f);
-      acc = logf(uf) < logA;
-      if (acc) atomicAdd(&n_acc, 1u);
-    }
-    acc = __shfl_sync(0xffffffffu, acc, 0);
-    if (acc)
-      for (int j = k + lane; j <= d; j += 32) P[(size_t)c * d + (j - 1)] = prop[j - 1];
+  for (int h = 0; h < 2; ++h) {
+    const int j = k + lane + 32 * h;
+    if (j > d) continue;
+    sc[h] = cur[j - 1];
+    if (!in) continue;
+    sp[h] = prop[j - 1];
+    const LayerTab& L = tab[j - 1];
+    const uint32_t link = ~L.hmask & nmask;
+    const uint32_t pc = j == 1 ? beta : cur[j - 2];   // s_{j-1}
+    const uint32_t pn = j == k ? pc : prop[j - 2];    // s'_{j-1}, s'_{k-1} = s_{k-1}
+    v += __popc((sc[h] ^ layer_map(L, pc)) & link);
+    vn += __popc((sp[h] ^ layer_map(L, pn)) & link);
+    lrev += lq[(size_t)c * d + (j - 1)];
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    v += __shfl_xor_sync(0xffffffffu, v, off);
+    vn += __shfl_xor_sync(0xffffffffu, vn, off);
+    lrev += __shfl_xor_sync(0xffffffffu, lrev, off);
+  }
+  bool acc = false;
+  if (in && lane == 0) {
+    const float logA = -J * (float)(vn - v) + lrev - lqf[c];
+    const uint32_t gc = group0 * 32u + c;
+    const uint32_t u = philox4x32_10(make_uint4(gc, move, 0xFFFFu | (kTagMH << 16), 0u), k0, k1).x;
+    const float uf = ((float)(u >> 8) + 0.5f) * (1.f / 16777216.f);
+    acc = logf(uf) < logA;
+    if (acc) atomicAdd(&n_acc, 1u);
+  }
+  acc = __shfl_sync(0xffffffffu, acc, 0);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int j = k + lane + 32 * h;
+    if (j <= d) words[j - 1][warp] = acc ? sp[h] : sc[h];
   }
   __syncthreads();
-  if (threadIdx.x == 0 && n_acc) atomicAdd(&ctr->accepted, (unsigned long long)n_acc);
+  for (int j = k + warp; j <= d; j += 32) {
+    const uint32_t y = warp_transpose(words[j - 1][lane], lane);
+    if (lane < n) state[((size_t)g * d + (j - 1)) * n + lane] = y;
+  }
+  if (threadIdx.x == 0) {
+    if (n_acc) atomicAdd(&ctr->accepted, (unsigned long long)n_acc);
+    // every CTA has read the counters before it counts itself
+    if (atomicAdd(ticket, 1u) == gridDim.x - 1u) {
+      *ticket = 0u;
+      ctr->moves = move + 1u;
+    }
+  }
 }
 
 // A host-drawn k* (networks that do not fit the fused kernel).
@@ -395,6 +412,7 @@ MhLayout mh_layout(int d, uint32_t groups) {
 // The pieces of a move region.
 struct MhPtrs {
   MhCounters* ctr;
+  uint32_t* ticket;  // CTAs of the acceptance that have finished (behind the counters)
   const LayerTab* tab;
   uint32_t *P, *Pn;
   float *lq, *lqf;
@@ -403,6 +421,8 @@ MhPtrs mh_ptrs(const MhCtx& c) {
   const MhLayout L = mh_layout(c.model->d, c.groups);
   MhPtrs q;
   q.ctr = reinterpret_cast<MhCounters*>(c.ws + L.ctr);
+  q.ticket = reinterpret_cast<uint32_t*>(q.ctr + 1);
+  static_assert(sizeof(MhCounters) + 4 <= 256, "the next piece starts at 256");
   q.tab = reinterpret_cast<const LayerTab*>(c.ws + L.tab);
   q.P = reinterpret_cast<uint32_t*>(c.ws + L.P);
   q.Pn = reinterpret_cast<uint32_t*>(c.ws + L.Pn);
@@ -414,14 +434,10 @@ MhPtrs mh_ptrs(const MhCtx& c) {
 // Acceptance, slicing back and the move counter: the end of every move.
 cudaError_t finish_move(const MhCtx& c, const MhPtrs& q, cudaStream_t st) {
   const pb_model& m = *c.model;
-  const int n = m.n, d = m.d, T = 256;
-  const uint32_t nmask = n == 32 ? 0xFFFFFFFFu : ((1u << n) - 1u);
-  const uint32_t k0 = (uint32_t)c.seed, k1 = (uint32_t)(c.seed >> 32);
-  accept_kernel<<<(c.chains * 32 + T - 1) / T, T, 0, st>>>(q.P, q.Pn, q.tab, m.beta, nmask, d, (float)m.J,
-                                                           q.lq, q.lqf, c.chains, k0, k1, q.ctr, c.group0);
-  // slicing back also counts the move
-  const uint32_t sw = c.groups * (uint32_t)d;
-  slice_kernel<<<(sw * 32 + T - 1) / T, T, 0, st>>>(q.P, n, d, q.ctr, c.groups, c.state);
+  const uint32_t nmask = m.n == 32 ? 0xFFFFFFFFu : ((1u << m.n) - 1u);
+  accept_slice_kernel<<<c.groups, 1024, 0, st>>>(
+      q.P, q.Pn, q.tab, m.beta, nmask, m.n, m.d, (float)m.J, q.lq, q.lqf, c.chains,
+      (uint32_t)c.seed, (uint32_t)(c.seed >> 32), q.ctr, q.ticket, c.group0, c.state);
   return cudaGetLastError();
 }
 
@@ -486,7 +502,8 @@ cudaError_t mh_region_init(const MhCtx& c, cudaStream_t st) {
 // One move (fused networks): unslice, draw k*, log q of the current suffix,
 // the proposal layer by layer, acceptance, slice back; no host value depends
 // on k*, so the sequence is captured once.
-cudaError_t mh_enqueue_move_dev(const MhCtx& c, cudaStream_t st) {
+cudaError_t mh_enqueue_move_dev(const MhCtx& c, cudaStream_t st, WsHeader* hdr,
+                                cudaGraphConditionalHandle loop) {
   const pb_model& m = *c.model;
   const MhPtrs q = mh_ptrs(c);
   const int n = m.n, d = m.d, T = 256;
@@ -494,7 +511,7 @@ cudaError_t mh_enqueue_move_dev(const MhCtx& c, cudaStream_t st) {
   const uint32_t k0 = (uint32_t)c.seed, k1 = (uint32_t)(c.seed >> 32);
   const uint32_t warps = c.groups * (uint32_t)d;
   move_begin_kernel<<<(warps * 32 + T - 1) / T, T, 0, st>>>(c.state, n, d, c.groups, q.P, q.ctr, c.seed,
-                                                            q.lqf, C);
+                                                            q.lqf, C, hdr, loop);
   // the proposal (sequential over the suffix layers, one CTA per 128
   // chains) first on st; log q of the current suffix (one CTA per tile and
   // layer) beside it on the side stream; both read P and k only

@@ -318,7 +318,9 @@ bool mh_fused(const pb_mlp* mlp);
 cudaError_t mh_region_init(const MhCtx& c, cudaStream_t st);
 // Enqueues one move with its suffix start drawn on the device from the seed
 // and the move counter (fused networks; capturable, no host synchronisation).
-cudaError_t mh_enqueue_move_dev(const MhCtx& c, cudaStream_t st);
+// hdr != nullptr: the move also counts down a period of the graph loop `loop`.
+cudaError_t mh_enqueue_move_dev(const MhCtx& c, cudaStream_t st, WsHeader* hdr = nullptr,
+                                cudaGraphConditionalHandle loop = 0);
 
 // What the learned-proposal code needs to know about one model of a run.
 struct RunView {

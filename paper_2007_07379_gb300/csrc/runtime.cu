@@ -942,14 +942,9 @@ namespace {
 int cuda_status(cudaError_t e) { return e == cudaSuccess ? PB_OK : PB_ECUDA; }
 
 // The device-side loop of a learned run's launch: the count of move periods
-// is set at the start, and the last kernel of each period counts down and
-// tells the graph's while node whether to run another.
+// is set at the start; the first kernel of each period counts down and tells
+// the graph's while node whether to run another.
 __global__ void periods_init_kernel(WsHeader* hdr, uint32_t periods) { hdr->periods_left = periods; }
-__global__ void periods_step_kernel(WsHeader* hdr, cudaGraphConditionalHandle loop) {
-  const uint32_t left = hdr->periods_left - 1u;
-  hdr->periods_left = left;
-  cudaGraphSetConditional(loop, left > 0u ? 1u : 0u);
-}
 
 // The launches of n sweeps of every model (no moves), in stream order.
 cudaError_t enqueue_sweeps(pb_run* r, uint32_t n_sweeps, cudaStream_t st) {
@@ -1002,13 +997,13 @@ cudaError_t build_learned_graph(pb_run* r, uint32_t n_sweeps, cudaStream_t cap, 
     cudaGraph_t body = cp.conditional.phGraph_out[0];
     if ((e = cudaStreamBeginCaptureToGraph(cap, body, nullptr, nullptr, 0, mode)) != cudaSuccess)
       return fail(e);
+    WsHeader* hdr = r->hdr();  // the first model's move counts the period
     for (const MhCtx& x : r->mh)
-      if (x.mlp && e == cudaSuccess) e = mh_enqueue_move_dev(x, cap);
+      if (x.mlp && e == cudaSuccess) {
+        e = mh_enqueue_move_dev(x, cap, hdr, loop);
+        hdr = nullptr;
+      }
     if (e == cudaSuccess) e = enqueue_sweeps(r, r->mh_every, cap);
-    if (e == cudaSuccess) {
-      periods_step_kernel<<<1, 1, 0, cap>>>(r->hdr(), loop);
-      e = cudaGetLastError();
-    }
     e2 = cudaStreamEndCapture(cap, &body);
     if (e != cudaSuccess || e2 != cudaSuccess) return fail(e != cudaSuccess ? e : e2);
     last = cond;
