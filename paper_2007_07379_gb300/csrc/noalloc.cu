@@ -18,13 +18,10 @@ namespace pb {
 cudaError_t launch_init(const RunModelDev* d_rm, int n_models, uint32_t total_groups,
                         const uint32_t* const* d_init_tabs, size_t smem_bytes, WsHeader* hdr,
                         cudaStream_t st);
-cudaError_t launch_sweeps(const RunModelDev* d_rm, int n_models, uint32_t total_groups,
-                          uint32_t n_sweeps, int cons, int prod, int max_col, int nc,
-                          size_t smem_bytes, WsHeader* hdr, cudaStream_t st, bool wgt = false,
-                          bool ext = false, bool bal = false, bool dec = false);
-size_t sweep_smem_bytes(int n, int d, int cons, int max_col, uint32_t hist_bins,
-                        bool wgt = false, bool bal = false);
-cudaError_t sweep_prepare();
+cudaError_t launch_sweeps_plain(const RunModelDev* d_rm, int n_models, uint32_t total_groups,
+                                uint32_t n_sweeps, int cons, int prod, int units, int max_col, int nc,
+                                size_t smem_bytes, WsHeader* hdr, cudaStream_t st);
+cudaError_t sweep_plain_prepare();
 }  // namespace pb
 
 using namespace pb;
@@ -53,7 +50,7 @@ int scratch_address(void** out) {
   if (!g_scratch_addr[dev]) {
     void* p = nullptr;
     if (cudaGetSymbolAddress(&p, g_pb_scratch) != cudaSuccess || p == nullptr) return PB_ECUDA;
-    if (sweep_prepare() != cudaSuccess) return PB_ECUDA;
+    if (sweep_plain_prepare() != cudaSuccess) return PB_ECUDA;
     g_scratch_addr[dev] = p;
   }
   *out = g_scratch_addr[dev];
@@ -112,23 +109,22 @@ extern "C" PB_API int pb_gibbs_run_noalloc(const pb_model* m, const pb_run_cfg* 
     maxcol = std::max(maxcol, m->col_off[c + 1] - m->col_off[c]);
     if (m->col_off[c + 1] > m->col_off[c]) nc = std::max(nc, c + 1);
   }
-  auto up32 = [](int x) { return ((x + 31) / 32) * 32; };
-  const int cons = std::max(32, std::min(224, up32(maxcol)));
-  int prod = std::max(32, std::min(kProducersMax, up32(sweep_producers_wanted(*m, nc, false))));
-  // histogram placement and plane buffers: the rules of a single-model run
-  // (shared memory when its u32 counters take at most 128 KiB and the CTA
-  // still fits; 16 planes ahead in three buffers when that fits with the
-  // same placement)
-  auto hist_fits = [&](bool bal) {
-    const size_t smem0 = sweep_smem_bytes(n, d, cons, maxcol, 0, false, bal);
-    return (size_t)bins * 32 <= (128u << 10) && smem0 + (size_t)bins * 32 <= kSweepSmemMax;
+  // histogram placement: the rule of a single-model run (shared memory for
+  // up to 4096 bins when the CTA still fits)
+  auto hist_fits = [&](int units) {
+    return bins <= 4096u && plain_smem_bytes(n, d, bins, units) <= kSweepSmemMax;
   };
-  const bool hist_smem = hist_fits(false);
-  const bool bal = hist_fits(true) == hist_smem &&
-                   sweep_smem_bytes(n, d, cons, maxcol, hist_smem ? bins : 0, false, true) <= kSweepSmemMax;
-  const size_t smem = sweep_smem_bytes(n, d, cons, maxcol, hist_smem ? bins : 0, false, bal);
+  auto smem_for = [&](int units) {
+    return plain_smem_bytes(n, d, hist_fits(units) ? bins : 0, units);
+  };
+  int dev = 0, sms = 1;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return PB_ECUDA;
+  const PlainDefault ps = plain_shape(n * d, maxcol, groups, sms, smem_for);
+  const bool hist_smem = hist_fits(ps.units);
+  const size_t smem = smem_for(ps.units);
   if (smem > kSweepSmemMax) return PB_ERANGE;
-  if (bal) prod = std::min(prod, kProducersBalanced);  // cons + prod + 32 <= kSweepThreadsBal
 
   ModelDev md{};
   md.n = n;
@@ -139,9 +135,11 @@ extern "C" PB_API int pb_gibbs_run_noalloc(const pb_model* m, const pb_run_cfg* 
   for (int k = 0; k < 4; ++k) md.thr[k] = m->thr[k];
   for (int k = 0; k < 5; ++k) md.col_off[k] = m->col_off[k];
   md.max_col = maxcol;
+  for (int k = 0; k < 4; ++k) md.n_rec[k] = m->n_rec[k];
 
   RunModelDev r{};
   r.model = reinterpret_cast<const ModelDev*>(base + o_md);
+  r.md = md;
   r.desc = reinterpret_cast<const Desc*>(base + o_desc);
   r.rec = reinterpret_cast<const Rec*>(base + o_rec);
   r.state = reinterpret_cast<uint32_t*>(base + o_state);
@@ -183,8 +181,8 @@ extern "C" PB_API int pb_gibbs_run_noalloc(const pb_model* m, const pb_run_cfg* 
                        (size_t)n_words(n, d) * 4, hdr, st)) != cudaSuccess)
     return PB_ECUDA;
   if (n_sweeps > 0 &&
-      (e = launch_sweeps(d_rm, 1, groups, n_sweeps, cons, prod, maxcol, nc, smem, hdr, st, false,
-                         false, bal, bal && maxcol > cons)) != cudaSuccess)
+      (e = launch_sweeps_plain(d_rm, 1, groups, n_sweeps, ps.cons, ps.prod, ps.units,
+                               maxcol, nc, smem, hdr, st)) != cudaSuccess)
     return PB_ECUDA;
   if ((e = cudaMemcpyAsync(d_counts, base + o_hist, (size_t)bins * 8 * 8, cudaMemcpyDeviceToDevice, st)) != cudaSuccess ||
       (e = cudaMemcpyAsync(d_totals, base + o_cnt, 2 * 8, cudaMemcpyDeviceToDevice, st)) != cudaSuccess)

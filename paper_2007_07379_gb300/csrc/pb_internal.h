@@ -37,12 +37,15 @@ static_assert(sizeof(Desc) == 16, "Desc must be 16 bytes");
 // Record term of one p-bit (16 bytes): violation word W[vd]^W[va]^W[vb]
 // (all ZERO when the p-bit has no own link; general-gate runs read
 // W[vd]^W[va]^(W[vb]&W[vc]), vc = ONES except on a Toffoli target) and phase
-// term w * (W[pa] & W[pb]) with w in {0, 1, 2, 4} units of pi/4.
+// term w * (W[pa] & W[pb]) with w (bits 0-2) in {0, 1, 2, 4} units of pi/4.
+// Plain runs keep the terms in lists: `slot` is the index among the
+// violation terms (0xFFFF: none), bits 3-15 of w the index among the phase
+// terms of that weight.
 struct Rec {
   uint16_t vd, va, vb;
   uint16_t pa, pb;
   uint16_t w;
-  uint16_t vc, pad;
+  uint16_t vc, slot;
 };
 static_assert(sizeof(Rec) == 16, "Rec must be 16 bytes");
 
@@ -119,6 +122,7 @@ struct ModelDev {
   int32_t n_ug;            // PB_U gates (UPh entries)
   int32_t n_tr;            // two-qubit table gates (TRec entries)
   double log2z;            // log2 of the estimator scale
+  int32_t n_rec[4];        // record terms: own links, phases of weight 1, 2, 4
 };
 
 // Per-model run entry (device), one per model of a run.
@@ -159,6 +163,7 @@ struct RunModelDev {
   const GLink* glk;        // models with Toffoli gates, else nullptr
   const TAcc* tacc;        // models with two-qubit table gates, else nullptr
   const TRec* trec;
+  ModelDev md;             // copy of *model
 };
 
 // Workspace header at offset 0.
@@ -167,7 +172,8 @@ struct WsHeader {
   uint32_t work_next;      // persistent scheduler counter
   uint32_t sweep0;         // absolute index of the next sweep
   uint32_t periods_left;   // learned runs: move periods still to run in a launch
-  uint32_t pad[60];
+  uint32_t ctas_done;      // CTAs of the current plain launch counted so far
+  uint32_t pad[59];
 };
 
 // Dynamic shared memory the sweep and exact-sampler kernels may use per CTA
@@ -176,10 +182,29 @@ constexpr size_t kSweepSmemMax = 226 * 1024;
 // Threads per sweep CTA in a run with general one-qubit gates (the general
 // instantiation is compiled for at most this many).
 constexpr int kSweepThreadsWgt = 512;
-// Plain runs with the three-buffer production: at most 512 threads a CTA,
-// so that the kernel gets up to 128 registers a thread (larger shapes take
-// the two-buffer form, 608 threads and 96 registers).
-constexpr int kSweepThreadsBal = 512;
+// Bound on the threads of a plain run's sweep CTA (224 consumers, 352
+// producers and one more warp at most): up to 88 registers a thread, so that
+// two CTAs of the default 352 threads share an SM.
+constexpr int kSweepThreadsPlain = 736;
+
+// Plain runs work in periods of plain_period sweeps: about `units` p-bit
+// updates (1 sweep at least, 16 at most, an even number above 1 because
+// sweeps are recorded in pairs).
+constexpr __host__ __device__ int plain_period(int npb, int units) {
+  const int ps = units / npb;
+  return ps < 2 ? 1 : (ps > 16 ? 16 : ps & ~1);
+}
+// Shared memory of a CTA: the group image, the snapshots of two periods,
+// consumer entries, three periods of comparison words, record lists, the
+// period's units, Philox and threshold words, undecided masks, an optional
+// histogram.
+inline size_t plain_smem_bytes(int n, int d, uint32_t hist_bins, int period_units) {
+  const size_t npb = (size_t)n * d, ps = (size_t)plain_period((int)npb, period_units), psp = (ps + 1) & ~(size_t)1;
+  const size_t units = (ps * npb + 63) & ~(size_t)63, npad = (npb + 31) & ~(size_t)31;
+  const size_t iw = ((size_t)n_words(n, d) + 1 + 3) & ~(size_t)3;
+  return (1 + 2 * psp) * iw * 4 + npb * 32 + (3 * units + npad) * 8 +
+         (npad + 96 + units) * 4 + (28 + 144 + 4) * 4 + 2 * (units >> 5) * 4 + (size_t)hist_bins * 32;
+}
 
 constexpr uint32_t kTagSweep = 0;
 constexpr uint32_t kTagInit = 1;
@@ -202,6 +227,7 @@ struct pb_model {
   std::vector<int32_t> colour;        // [d][n]
   std::vector<pb::Desc> desc;         // colour-ordered
   std::vector<pb::Rec> rec;           // by p = (k-1) n + q
+  int32_t n_rec[4] = {0, 0, 0, 0};    // lengths of the record lists (ModelDev::n_rec)
   std::vector<uint32_t> init;         // by p: 0xFFFFFFFF = free output, else a | b << 16
   std::vector<pb_gate> gates;
   // general one-qubit gates
@@ -218,29 +244,39 @@ struct pb_model {
 };
 
 namespace pb {
-// Philox calls the producers of a sweep launch make in one colour step for
-// model m, nc colour steps per sweep: 3 per p-bit of the next class in one
-// step (12 planes ahead, two buffers: general-gate runs, and plain runs
-// whose tables leave no room for more), or 4 per p-bit spread evenly over
-// the steps (16 planes ahead, three buffers: other plain runs); the larger
-// of the two for plain runs, which take either.
-inline int sweep_producers_wanted(const pb_model& m, int nc, bool wgt) {
+// Philox calls the producers of a general-gate launch make in one colour
+// step: 3 per p-bit of the next class (12 planes ahead, two buffers).
+inline int sweep_producers_wanted(const pb_model& m) {
   int maxcol = 1;
   for (int c = 0; c < 4; ++c) maxcol = std::max(maxcol, m.col_off[c + 1] - m.col_off[c]);
-  if (wgt) return 3 * maxcol;
-  return std::max(3 * maxcol, (4 * m.col_off[4] + nc - 1) / std::max(1, nc));
+  return 3 * maxcol;
 }
-// Default producer count caps: 352, and 224 for plain runs with the three-
-// buffer production (seven producer warps: with four consumer warps and the
-// recorder, three warps per scheduler; measured 6 % faster than 352 on the
-// mid workload, 2-4 % on the learned and large ones).
 constexpr int kProducersMax = 352;
-constexpr int kProducersBalanced = 224;
-template <class Models>  // a container of pointers to models
-inline int sweep_producers_wanted(const Models& ms, int nc, bool wgt) {
-  int p = 32;
-  for (auto& m : ms) p = std::max(p, sweep_producers_wanted(*m, nc, wgt));
-  return p;
+// Plain runs: default CTA shape and period for `groups` chain groups of
+// models of up to npb p-bits (largest colour class maxcol) on a GPU of `sms`
+// SMs; smem(units): shared memory of a CTA with that period.
+// Two CTAs an SM where there are groups for them and they fit: the roles of
+// one hide the other's latencies (large workload, ms per 1e3 sweeps: 64
+// consumers + 256 producers, two CTAs, 17.2; 64 + 352, one CTA, 21.8).
+// Otherwise one CTA an SM with a consumer per p-bit of the largest class, as
+// many producers as a period has tasks for and a longer period, whose tasks
+// spread more evenly over the warps (mid, ms per 1e4 sweeps: 4096 units
+// 4.73, 2048 4.89; learned 7.00 and 7.90).
+struct PlainDefault {
+  int cons, prod, units;
+};
+constexpr int kPlainUnitsOne = 4096, kPlainUnitsTwo = 2048;
+template <class Smem>
+inline PlainDefault plain_shape(int npb, int maxcol, uint32_t groups, int sms, Smem smem) {
+  auto up32 = [](int x) { return ((x + 31) / 32) * 32; };
+  PlainDefault s;
+  const bool two = groups > (uint32_t)sms && 2 * smem(kPlainUnitsTwo) <= kSweepSmemMax;
+  s.units = two || smem(kPlainUnitsOne) > kSweepSmemMax ? kPlainUnitsTwo : kPlainUnitsOne;
+  s.cons = std::max(32, std::min(two ? 64 : 224, up32(maxcol)));
+  const int ps = plain_period(npb, s.units);
+  const int tasks = (ps * npb + 63) / 64 + (ps * npb + 255) / 256 + (ps + 1) / 2;
+  s.prod = std::max(32, std::min(two ? 256 : 352, 32 * ((tasks + 1) / 2)));
+  return s;
 }
 }  // namespace pb
 

@@ -21,12 +21,17 @@ cudaError_t launch_init(const RunModelDev* d_rm, int n_models, uint32_t total_gr
                         cudaStream_t st);
 cudaError_t launch_sweeps(const RunModelDev* d_rm, int n_models, uint32_t total_groups,
                           uint32_t n_sweeps, int cons, int prod, int max_col, int nc,
-                          size_t smem_bytes, WsHeader* hdr, cudaStream_t st, bool wgt = false,
-                          bool ext = false, bool bal = false, bool dec = false);
-cudaError_t launch_sweeps_persistent(const RunModelDev* d_rm, int n_models, const uint32_t* d_work,
-                                     uint32_t n_work, uint32_t n_sweeps, int cons, int prod,
-                                     int max_col, int nc, int grid, size_t smem_bytes,
-                                     WsHeader* hdr, cudaStream_t st, bool bal);
+                          size_t smem_bytes, WsHeader* hdr, cudaStream_t st, bool ext);
+cudaError_t launch_sweeps_plain(const RunModelDev* d_rm, int n_models, uint32_t total_groups,
+                                uint32_t n_sweeps, int cons, int prod, int units, int max_col, int nc,
+                                size_t smem_bytes, WsHeader* hdr, cudaStream_t st);
+cudaError_t launch_sweeps_plain_persistent(const RunModelDev* d_rm, int n_models,
+                                           const uint32_t* d_work, uint32_t n_work,
+                                           uint32_t n_sweeps, int cons, int prod, int units,
+                                           int max_col, int nc, int grid, size_t smem_bytes,
+                                           WsHeader* hdr, cudaStream_t st);
+cudaError_t sweep_plain_prepare();
+int sweep_plain_blocks_per_sm(int max_col, int cons, int nc, int threads, size_t smem);
 cudaError_t launch_elim(const RunModelDev* d_rm, int n_models, uint32_t total_groups,
                         const uint32_t* const* d_init_tabs, uint32_t n_sweeps, size_t smem_bytes,
                         WsHeader* hdr, cudaStream_t st, bool wgt, int warps);
@@ -35,10 +40,8 @@ cudaError_t launch_amplitudes(const RunModelDev* d_rm, int model, uint32_t bins,
                               cudaStream_t st);
 cudaError_t launch_philox_fill(const uint32_t* ctr, uint32_t k0, uint32_t k1, uint32_t count,
                                uint32_t* out, cudaStream_t st);
-size_t sweep_smem_bytes(int n, int d, int cons, int max_col, uint32_t hist_bins,
-                        bool wgt = false, bool bal = false);
+size_t sweep_smem_bytes(int n, int d, int cons, int max_col, uint32_t hist_bins);
 cudaError_t sweep_prepare();
-int sweep_max_blocks_per_sm(int threads, size_t smem, bool bal);
 }  // namespace pb
 
 using namespace pb;
@@ -502,6 +505,9 @@ PB_API int pb_compile_g(int n, int d, const pb_gate* gates, int n_gates, const d
           break;
         default: break;
       }
+      // slots in the record lists of plain runs
+      R.slot = R.vd != R.va || R.vb != Z ? (uint16_t)m->n_rec[0]++ : (uint16_t)0xFFFF;
+      if (R.w) R.w |= (uint16_t)(m->n_rec[R.w == 1 ? 1 : (R.w == 2 ? 2 : 3)]++ << 3);
       m->rec[p] = R;
     }
   }
@@ -905,12 +911,11 @@ struct pb_run {
   uint32_t total_groups = 0;
   int threads = 32;
   int cons = 32, prod = 32, max_col = 1, blocks_per_sm = 0;
+  int units = 0;           // plain runs: units of a period
   size_t smem = 0;
   bool persistent = false;
   bool wgt = false;        // some model has PB_U gates (the general-gate kernels)
   bool ext = false;        // some model has Toffoli links or two-qubit tables
-  bool bal = false;        // plain run with 16 planes ahead, produced evenly over the steps
-  bool dec = false;        // (with bal) the recorder outside the colour steps' barriers
   int nc = 2;              // colour steps per sweep (largest over the models)
   bool elim = false;       // exact-sampler run: i.i.d. paths instead of sweeps
   size_t elim_smem = 0;
@@ -952,12 +957,15 @@ cudaError_t enqueue_sweeps(pb_run* r, uint32_t n_sweeps, cudaStream_t st) {
     return launch_elim(r->d_rm(), r->nm, r->total_groups,
                        reinterpret_cast<const uint32_t* const*>(r->ws + r->L.init_ptrs), n_sweeps,
                        r->elim_smem, r->hdr(), st, r->wgt, r->elim_warps);
+  if (r->wgt)
+    return launch_sweeps(r->d_rm(), r->nm, r->total_groups, n_sweeps, r->cons, r->prod, r->max_col,
+                         r->nc, r->smem, r->hdr(), st, r->ext);
   if (r->persistent)
-    return launch_sweeps_persistent(r->d_rm(), r->nm, reinterpret_cast<const uint32_t*>(r->ws + r->L.work),
-                                    r->total_groups, n_sweeps, r->cons, r->prod, r->max_col, r->nc,
-                                    r->grid, r->smem, r->hdr(), st, r->bal);
-  return launch_sweeps(r->d_rm(), r->nm, r->total_groups, n_sweeps, r->cons, r->prod, r->max_col,
-                       r->nc, r->smem, r->hdr(), st, r->wgt, r->ext, r->bal, r->dec);
+    return launch_sweeps_plain_persistent(
+        r->d_rm(), r->nm, reinterpret_cast<const uint32_t*>(r->ws + r->L.work), r->total_groups,
+        n_sweeps, r->cons, r->prod, r->units, r->max_col, r->nc, r->grid, r->smem, r->hdr(), st);
+  return launch_sweeps_plain(r->d_rm(), r->nm, r->total_groups, n_sweeps, r->cons, r->prod, r->units,
+                             r->max_col, r->nc, r->smem, r->hdr(), st);
 }
 
 // Graph of n sweeps of a learned run (Fig. 2 Step 1 with the network as the
@@ -1020,6 +1028,30 @@ cudaError_t build_learned_graph(pb_run* r, uint32_t n_sweeps, cudaStream_t cap, 
   return cudaSuccess;
 }
 
+// Shared memory of a sweep CTA with the run's consumers and a period of
+// `units`, and which models count in shared memory.  Shared-memory
+// histograms are counted per CTA and added to the global counters once per
+// launch; used when the bins fit (up to 4096 bins for one circuit, 1024 per
+// circuit in a batch so that several CTAs share an SM; 32 bytes a bin, 40
+// with general gates); otherwise the record adds to global memory directly.
+size_t plan_smem(const pb_run* r, int units, std::vector<char>* use) {
+  const size_t cap_bins = r->nm == 1 ? 4096u : 1024u;
+  size_t smem = 0;
+  if (use) use->assign(r->nm, 0);
+  for (int i = 0; i < r->nm; ++i) {
+    const pb_model& m = *r->models[i];
+    auto bytes = [&](uint32_t bins) {
+      return r->wgt ? sweep_smem_bytes(m.n, m.d, r->cons, r->max_col, bins)
+                    : plain_smem_bytes(m.n, m.d, bins, units);
+    };
+    const uint32_t bins = r->L.ms[i].bins;
+    const bool in = bins <= cap_bins && bytes(bins) <= kSweepSmemMax;
+    if (use) (*use)[i] = in;
+    smem = std::max(smem, bytes(in ? bins : 0));
+  }
+  return smem;
+}
+
 // Applies a CTA shape (consumer and producer threads, multiples of 32) to
 // the run: shared-memory size, histogram placement and the persistent grid.
 void apply_shape(pb_run* r, int cons, int prod, int blocks_per_sm) {
@@ -1030,56 +1062,18 @@ void apply_shape(pb_run* r, int cons, int prod, int blocks_per_sm) {
   r->prod = prod;
   r->max_col = maxcol;
   r->threads = cons + prod + 32;
-  // Shared-memory histograms: counted per CTA, added to the global counters
-  // once per launch.  Used when the bins fit (up to 4096 bins for one
-  // circuit, 1024 per circuit in a batch so that several CTAs share an SM;
-  // 32 bytes a bin, 40 with general gates); otherwise the record adds to
-  // global memory directly.
-  const size_t cap_bins = r->nm == 1 ? 4096u : 1024u;
-  auto layout = [&](bool bal, std::vector<char>& use) {
-    size_t smem = 0;
-    use.assign(r->nm, 0);
-    for (int i = 0; i < r->nm; ++i) {
-      const pb_model& m = *r->models[i];
-      const uint32_t bins = r->L.ms[i].bins;
-      use[i] = bins <= cap_bins &&
-               sweep_smem_bytes(m.n, m.d, cons, maxcol, bins, r->wgt, bal) <= kSweepSmemMax;
-      smem = std::max(smem, sweep_smem_bytes(m.n, m.d, cons, maxcol, use[i] ? bins : 0, r->wgt, bal));
-    }
-    return smem;
-  };
+  std::vector<char> use;
+  r->smem = plan_smem(r, r->units, &use);
+  for (int i = 0; i < r->nm; ++i) r->rm[i].hist_smem = use[i] ? 1u : 0u;
   r->persistent = r->nm > 1;
   if (const char* e = std::getenv("PB_PERSISTENT")) r->persistent = std::atoi(e) != 0;
   if (r->wgt) r->persistent = false;  // general-gate sweeps: one CTA per group
-  // Plain runs take the balanced production (16 planes ahead, three plane
-  // buffers) when its tables fit with the same histogram placement and, on
-  // a persistent grid, the same CTAs per SM; otherwise 12 planes in two.
-  std::vector<char> use_s, use_b;
-  const size_t smem_s = layout(false, use_s);
-  bool bal = false;
-  size_t smem_b = 0;
-  if (!r->wgt) {
-    smem_b = layout(true, use_b);
-    bal = smem_b <= kSweepSmemMax && use_b == use_s && r->threads <= kSweepThreadsBal;
-    if (bal && r->persistent)
-      bal = sweep_max_blocks_per_sm(r->threads, smem_b, true) >=
-            sweep_max_blocks_per_sm(r->threads, smem_s, false);
-    if (const char* e = std::getenv("PB_BALANCED")) bal = bal && std::atoi(e) != 0;
-  }
-  const std::vector<char>& use = bal ? use_b : use_s;
-  for (int i = 0; i < r->nm; ++i) r->rm[i].hist_smem = use[i] ? 1u : 0u;
-  const size_t smem = bal ? smem_b : smem_s;
-  r->bal = bal;
-  // the recorder outside the colour steps' barriers where some class takes
-  // more than one consumer pass (single-grid plain runs)
-  r->dec = bal && !r->wgt && !r->persistent && maxcol > cons;
-  r->smem = smem;
   r->grid = 0;
   if (r->persistent) {
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int per_sm = sweep_max_blocks_per_sm(r->threads, smem, r->bal);
+    int per_sm = sweep_plain_blocks_per_sm(maxcol, cons, r->nc, r->threads, r->smem);
     if (blocks_per_sm > 0) per_sm = std::min(per_sm, blocks_per_sm);
     r->grid = std::max(1, sms * std::max(1, per_sm));
     r->grid = (int)std::min<uint32_t>((uint32_t)r->grid, r->total_groups);
@@ -1087,40 +1081,43 @@ void apply_shape(pb_run* r, int cons, int prod, int blocks_per_sm) {
   r->blocks_per_sm = blocks_per_sm;
 }
 
-// Default launch shape: consumers = the largest colour class rounded up to
-// a warp (one p-bit per consumer per class), capped at 224; producers = one
-// per Philox call of a colour step (sweep_producers_wanted), capped at 352,
-// or at 224 when the run takes the three-buffer production; plus one
-// recorder warp.  Environment overrides PB_CONS, PB_PROD (multiples of 32).
+// Default launch shape.  Plain runs: plain_shape.  General-gate runs:
+// consumers = the largest colour class rounded up to a warp (one p-bit per
+// consumer per class), capped at 224; producers = one per Philox call of a
+// colour step, capped so that the CTA keeps 512 threads; plus one recorder
+// warp.  Environment overrides PB_CONS, PB_PROD (multiples of 32).
 void choose_shape(pb_run* r) {
-  int maxcol = 1;
-  for (auto& m : r->models)
+  int maxcol = 1, npb = 1, want = 32;
+  for (auto& m : r->models) {
     for (int c = 0; c < 4; ++c) maxcol = std::max(maxcol, m->col_off[c + 1] - m->col_off[c]);
+    npb = std::max(npb, m->n * m->d);
+    want = std::max(want, sweep_producers_wanted(*m));
+  }
   auto up32 = [](int x) { return ((x + 31) / 32) * 32; };
   int cons = std::max(32, std::min(224, up32(maxcol)));
-  const int want = up32(sweep_producers_wanted(r->models, r->nc, r->wgt));
-  int prod = std::max(32, std::min(kProducersMax, want));
+  int prod = std::min(kProducersMax, up32(want));
+  if (!r->wgt) {
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const PlainDefault ps = plain_shape(npb, maxcol, r->total_groups, sms,
+                                        [&](int units) { return plan_smem(r, units, nullptr); });
+    cons = ps.cons;
+    prod = ps.prod;
+    r->units = ps.units;
+  }
   if (const char* e = std::getenv("PB_CONS")) {
     int v = std::atoi(e);
     if (v >= 32 && v <= 224 && v % 32 == 0) cons = v;
   }
-  bool fixed_prod = false;
   if (const char* e = std::getenv("PB_PROD")) {
     int v = std::atoi(e);
-    if (v >= 32 && v <= 352 && v % 32 == 0) { prod = v; fixed_prod = true; }
+    if (v >= 32 && v <= 352 && v % 32 == 0) prod = v;
   }
   if (r->wgt) prod = std::max(32, std::min(prod, kSweepThreadsWgt - 32 - cons));
-  if (!r->wgt && !fixed_prod && prod > kProducersBalanced) {
-    // the three-buffer form with its producer count where it applies, else
-    // the two-buffer form with the larger one
-    apply_shape(r, cons, kProducersBalanced, 0);
-    if (r->bal) prod = kProducersBalanced;
-    else apply_shape(r, cons, prod, 0);
-  } else {
-    apply_shape(r, cons, prod, 0);
-  }
-  // a shape whose tables do not fit: fewer consumers (their class table and
-  // acceptance planes shrink; the class runs in more passes)
+  apply_shape(r, cons, prod, 0);
+  // a shape whose tables do not fit (general gates): fewer consumers (their
+  // class table and acceptance planes shrink; the class runs in more passes)
   while (r->smem > kSweepSmemMax && cons > 32) {
     cons -= 32;
     apply_shape(r, cons, prod, 0);
@@ -1198,6 +1195,7 @@ PB_API int pb_run_create(pb_model* const* models, const pb_run_cfg* cfgs, int n_
     md.max_col = 0;
     for (int k = 0; k < 4; ++k) md.max_col = std::max(md.max_col, m.col_off[k + 1] - m.col_off[k]);
     md.wgt = m.wgt ? 1 : 0;
+    for (int k = 0; k < 4; ++k) md.n_rec[k] = m.n_rec[k];
     md.n_ug = (int32_t)m.uph.size();
     md.n_tr = (int32_t)m.trec.size();
     md.log2z = m.n_tab ? 0.0 : m.log2z;  // tables: unit scale, read L2-normalised
@@ -1239,6 +1237,7 @@ PB_API int pb_run_create(pb_model* const* models, const pb_run_cfg* cfgs, int n_
     RunModelDev& d = r->rm[i];
     std::memset(&d, 0, sizeof d);
     d.model = reinterpret_cast<const ModelDev*>(ws + s.model_dev);
+    d.md = md;
     d.desc = reinterpret_cast<const Desc*>(ws + s.desc);
     d.rec = reinterpret_cast<const Rec*>(ws + s.rec);
     d.state = reinterpret_cast<uint32_t*>(ws + s.state);
@@ -1328,7 +1327,7 @@ PB_API int pb_run_create(pb_model* const* models, const pb_run_cfg* cfgs, int n_
                      return a.first > b.first;
                    });
   for (auto& c : cost) work.push_back(c.second);
-  if (sweep_prepare() != cudaSuccess) return PB_ECUDA;
+  if (sweep_prepare() != cudaSuccess || sweep_plain_prepare() != cudaSuccess) return PB_ECUDA;
   choose_shape(r.get());
   if (r->smem > kSweepSmemMax || r->elim_smem > kSweepSmemMax) return PB_ERANGE;
   if ((e = cudaMemcpyAsync(ws + r->L.rm, r->rm.data(), sizeof(RunModelDev) * n_models,
@@ -1620,8 +1619,12 @@ PB_API int pb_run_tune(pb_run* r, uint32_t trial_sweeps, const char* cache_path,
   std::vector<int> cons_c, prod_c, bpsm_c = {0};
   for (int c : {64, 128, 224})
     if (c <= std::max(64, up)) cons_c.push_back(c);
-  const int pw = sweep_producers_wanted(r->models, r->nc, r->wgt);
-  for (int p : {96, 192, 224, 352})
+  int pw = 352;
+  if (r->wgt) {
+    pw = 32;
+    for (auto& m : r->models) pw = std::max(pw, sweep_producers_wanted(*m));
+  }
+  for (int p : {96, 192, 256, 352})
     if (p <= std::max(96, ((pw + 31) / 32) * 32)) prod_c.push_back(p);
   if (r->nm > 1) bpsm_c = {1, 2, 0};
   double best = 1e30;

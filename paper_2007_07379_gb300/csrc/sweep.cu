@@ -1,4 +1,5 @@
-// Gibbs sweep, record and amplitude kernels (sm_103a).
+// General-gate Gibbs sweeps, initial paths, exact sampler and amplitude kernels
+// (sm_103a); sweep_plain.cu holds the plain (Clifford+T) sweeps.
 //
 // Layout: 32 chains are bit-sliced into one 32-bit word per p-bit (bit c =
 // chain 32 g + c of group g).  A CTA owns one group at a time and keeps the
@@ -20,6 +21,7 @@
 
 #include "pb_internal.h"
 #include "philox.cuh"
+#include "sweep_common.cuh"
 
 namespace pb {
 
@@ -50,16 +52,6 @@ __device__ __forceinline__ void compare4(uint32_t& lt, uint32_t& eq, const HbCla
   }
 }
 
-// Barrier `id` over the first `threads` threads of the CTA (whole warps).
-__device__ __forceinline__ void bar_sync_first(uint32_t id, uint32_t threads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-
-// Out-of-line Philox for the rarely taken paths (keeps the hot loop small).
-__device__ __noinline__ uint4 philox_cold(uint4 c, uint32_t k0, uint32_t k1) {
-  return philox4x32_10(c, k0, k1);
-}
-
 // Planes beyond the precomputed ones (rare): Philox calls grp0 .. 7.
 __device__ __forceinline__ void compare_tail(uint32_t& lt, uint32_t& eq, const HbClass& k,
                                              uint32_t grp0, uint32_t g, uint32_t sweep, uint32_t p,
@@ -69,30 +61,17 @@ __device__ __forceinline__ void compare_tail(uint32_t& lt, uint32_t& eq, const H
     compare4(lt, eq, k, philox_cold(make_uint4(g, sweep, p, grp), k0, k1), grp);
 }
 
-// Number of Philox calls computed ahead of a colour class: 12 planes for
-// general-gate runs, 16 for plain runs (whose producers spread the work over
-// the colour steps and have room for the fourth).
+// Philox calls computed ahead of a colour class: 12 planes.
 constexpr int kPre = 3;
-constexpr int kPrePlain = 4;
 // General-gate runs: Philox calls of the Metropolis acceptance draw (tag 6)
 // computed ahead (12 planes) for the coupled p-bits among the first
 // `consumers` of a class (the rest draw their own, out of line).
 constexpr int kPreC = 3;
 
-// Threshold pair of a p-bit with m links: tA for the lanes in `sel` (all
-// links agree), tB for the others (see the consumer table set-up).
-__device__ __forceinline__ uint32_t thr_a(int m, uint32_t t0, uint32_t t1, uint32_t t2, uint32_t t3) {
-  return m == 0 ? t0 : (m == 1 ? t1 : (m == 2 ? t2 : t3));
-}
-__device__ __forceinline__ uint32_t thr_b(int m, uint32_t t0, uint32_t t1) {
-  return (m == 0 || m == 2) ? t0 : t1;
-}
-
 // Comparison of the precomputed planes for any thresholds (small J), and
 // the planes beyond them; out of line: taken rarely.
-// np: the precomputed outputs R0 .. R{np-1} (3 or 4; R3 unused when 3).
 __device__ __noinline__ uint32_t heat_bath_general(const HbClass k, uint4 R0, uint4 R1, uint4 R2,
-                                                   uint4 R3, int np, uint32_t lt, uint32_t eq,
+                                                   uint32_t lt, uint32_t eq,
                                                    bool pre, uint32_t g, uint32_t sweep,
                                                    uint32_t pidx, uint32_t k0, uint32_t k1) {
   if (pre) {
@@ -102,9 +81,8 @@ __device__ __noinline__ uint32_t heat_bath_general(const HbClass k, uint4 R0, ui
     eq &= ~k.tail0;
     compare4(lt, eq, k, R1, 1u);
     compare4(lt, eq, k, R2, 2u);
-    if (np > 3) compare4(lt, eq, k, R3, 3u);
   }
-  compare_tail(lt, eq, k, (uint32_t)np, g, sweep, pidx, k0, k1);
+  compare_tail(lt, eq, k, (uint32_t)kPre, g, sweep, pidx, k0, k1);
   return lt;
 }
 
@@ -126,20 +104,16 @@ __device__ __forceinline__ FastThr fast_thresholds(uint32_t thr1, uint32_t thr2)
 
 // New value of the 32 chains of one p-bit (Fig. 2 Steps 1-2) from its link
 // demands r0..r2 (three-link form: m=0: 0,0,0  m=1: r0,r0,0  m=2: r0,r1,0
-// m=3: r0,r1,r2), its masks Mk = [m == k] and its NP precomputed Philox
+// m=3: r0,r1,r2), its masks Mk = [m == k] and its kPre precomputed Philox
 // outputs R.  Short form (F.on): plane 0 decides the t0 lanes (u < 2^31 iff
 // its top bit is 0); on planes 1..7 every other threshold bit is 0, so a
 // lane stays equal only while it draws zeros; on planes 8..11 the lanes
 // compared with thr1 (L1) meet thr1's bits and the thr2 / thr3 lanes zeros.
-// A lane is still equal after plane 11 with probability 2^-12, so about one
-// p-bit in 128 (32 lanes) needs more: with NP = 4 the fourth output gives
-// planes 12..15 inline (general comparison, no Philox call).  Lanes still
-// equal after the precomputed planes, and every lane when the thresholds do
-// not have that form, go to heat_bath_general.
-template <int NP>
+// Lanes still equal after the precomputed planes (one p-bit in 128), and every
+// lane when the thresholds do not have that form, go to heat_bath_general.
 __device__ __forceinline__ uint32_t heat_bath_links(uint32_t r0, uint32_t r1, uint32_t r2, int m,
                                                     uint32_t M0, uint32_t M1, uint32_t M2,
-                                                    uint32_t M3, const uint4 (&R)[NP],
+                                                    uint32_t M3, const uint4 (&R)[kPre],
                                                     const FastThr& F, uint32_t thr0,
                                                     uint32_t thr1, uint32_t thr2, uint32_t thr3,
                                                     uint32_t g, uint32_t sweep, uint32_t pidx,
@@ -161,19 +135,12 @@ __device__ __forceinline__ uint32_t heat_bath_links(uint32_t r0, uint32_t r1, ui
       lt |= eq & ~P[w] & A;
       eq &= ~(P[w] ^ A);
     }
-    if constexpr (NP > 3) {
-      if (eq != 0u) {
-        k.tA = thr_a(m, thr0, thr1, thr2, thr3);
-        k.tB = thr_b(m, thr0, thr1);
-        compare4(lt, eq, k, R[3], 3u);
-      }
-    }
     general = eq != 0u;
   }
   if (general) {
     k.tA = thr_a(m, thr0, thr1, thr2, thr3);
     k.tB = thr_b(m, thr0, thr1);
-    lt = heat_bath_general(k, R[0], R[1], R[2], R[NP > 3 ? 3 : 2], NP, lt, eq, !F.on, g, sweep,
+    lt = heat_bath_general(k, R[0], R[1], R[2], lt, eq, !F.on, g, sweep,
                            pidx, k0, k1);
   }
   return k.neg ^ lt;
@@ -314,29 +281,6 @@ __device__ __noinline__ uint32_t table_accept(const uint32_t* W, const TAcc* tp,
   return old ^ (flip & acc);
 }
 
-__device__ __forceinline__ void add3(uint32_t& f0, uint32_t& f1, uint32_t& f2, uint32_t x0,
-                                     uint32_t x1, uint32_t x2) {
-  const uint32_t c0 = f0 & x0;
-  f0 ^= x0;
-  const uint32_t t = f1 ^ x1;
-  const uint32_t c1 = (f1 & x1) | (c0 & t);
-  f1 = t ^ c0;
-  f2 ^= x2 ^ c1;
-}
-
-__device__ __forceinline__ int find_model(const RunModelDev* rm, int n_models, uint32_t flat) {
-  int lo = 0, hi = n_models - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (rm[mid].group_base <= flat) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
-__device__ __forceinline__ void set_status(WsHeader* hdr, int code) {
-  if (hdr) atomicCAS(&hdr->status, 0u, (uint32_t)code);
-}
-
 // Compensated FP64 accumulation of the phase sums: *s += x by an atomic add,
 // whose old value gives the exact rounding error of fl(old + x) (Knuth's
 // two-sum), and that error (plus `carry`, a compensation brought along) is
@@ -370,36 +314,14 @@ static_assert(sizeof(ClassEnt) == 48, "ClassEnt must be 48 bytes");
 
 // Shared-memory image of one group: words (image_words) and two snapshots,
 // descriptors, record terms, an optional histogram of hist_bins x 8 u32
-// counters, the consumers' class table and the plane buffers: three of
-// kPrePlain x max_col Philox outputs (plain runs), or two of kPre x max_col
-// plus kPreC x cons acceptance outputs (general-gate runs).  The image holds the (d+1) n layer words,
-// ZERO, ONES and one scratch word (the store target of consumers without a
-// p-bit in a colour class), rounded up to 16 bytes.
-__host__ __device__ inline int image_words(int n, int d) { return (n_words(n, d) + 1 + 3) & ~3; }
-
+// counters, the consumers' class table and two plane buffers, each of kPre x
+// max_col Philox outputs and kPreC x cons acceptance outputs.
 __host__ __device__ inline size_t group_smem_bytes(int n, int d, int cons, int max_col,
-                                                   uint32_t hist_bins, bool wgt = false,
-                                                   bool bal = false) {
+                                                   uint32_t hist_bins) {
   return (size_t)3 * image_words(n, d) * 4 + (size_t)n * d * sizeof(Desc) +
-         (size_t)n * d * sizeof(Rec) + (((size_t)hist_bins * (wgt ? 10 : 8) + 3) & ~(size_t)3) * 4 +
+         (size_t)n * d * sizeof(Rec) + (((size_t)hist_bins * 10 + 3) & ~(size_t)3) * 4 +
          (size_t)4 * cons * sizeof(ClassEnt) +
-         (wgt ? (size_t)2 * ((size_t)kPre * max_col + (size_t)kPreC * cons)
-              : bal ? (size_t)3 * kPrePlain * max_col : (size_t)2 * kPre * max_col) * sizeof(uint4);
-}
-
-// 32 x 32 bit transpose across a warp: on entry lane r holds row r; on
-// return lane c holds column c (bit r = bit c of row r).  Five butterfly
-// steps, each swapping the off-diagonal blocks of the current block size.
-__device__ __forceinline__ uint32_t warp_transpose32(uint32_t x, int lane) {
-  const uint32_t masks[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
-#pragma unroll
-  for (int k = 0; k < 5; ++k) {
-    const int j = 16 >> k;
-    const uint32_t M = masks[k];
-    const uint32_t y = __shfl_xor_sync(0xffffffffu, x, j);
-    x = (lane & j) ? ((x & ~M) | ((y & ~M) >> j)) : ((x & M) | ((y & M) << j));
-  }
-  return x;
+         (size_t)2 * ((size_t)kPre * max_col + (size_t)kPreC * cons) * sizeof(uint4);
 }
 
 // Record of one sweep (Fig. 2 Step 3), computed by the recorder warp from a
@@ -607,26 +529,24 @@ struct Recorder {
 };
 
 // p-bits lo + first, lo + first + stride, ... < hi of a colour class from
-// their descriptors (a class larger than the consumers; rare).  cpl: the
-// coupling table of a general-gate model, else nullptr.  Output j of the
-// class's k-th p-bit is cur[k NP + j] (pst = 1) or cur[j pst + k] (pst > 1:
-// plane-major buffers).
-template <int NP>
-__device__ __forceinline__ void redraw_body(uint32_t* W, uint32_t* S, const Desc* sdesc,
-                                            const uint4* cur, int pst, int lo, int first,
-                                            int hi, int stride, int n, FastThr fast, uint32_t thr0,
-                                            uint32_t thr1, uint32_t thr2, uint32_t thr3,
-                                            uint32_t g, uint32_t sweep, uint32_t k0, uint32_t k1,
-                                            const Cpl* cpl, const GLink* glk, const TAcc* tacc) {
+// their descriptors (a class larger than the consumers; rare).  Output j of
+// the class's k-th p-bit is cur[k kPre + j].
+__device__ __noinline__ void redraw_extra_coupled(uint32_t* W, uint32_t* S, const Desc* sdesc,
+                                                  const uint4* cur, int lo, int first, int hi,
+                                                  int stride, int n, FastThr fast, uint32_t thr0,
+                                                  uint32_t thr1, uint32_t thr2, uint32_t thr3,
+                                                  uint32_t g, uint32_t sweep, uint32_t k0,
+                                                  uint32_t k1, const Cpl* cpl, const GLink* glk,
+                                                  const TAcc* tacc) {
   for (int i = lo + first; i < hi; i += stride) {
     Desc D = sdesc[i];
     if (D.mflag & 0x80) continue;
     const int m = D.mflag & 3;
     if (m == 1) { D.a[1] = D.a[0]; D.b[1] = D.b[0]; }
-    const uint4* rp = cur + (i - lo) * (pst == 1 ? NP : 1);
-    uint4 R[NP];
+    const uint4* rp = cur + (i - lo) * kPre;
+    uint4 R[kPre];
 #pragma unroll
-    for (int j = 0; j < NP; ++j) R[j] = rp[j * pst];
+    for (int j = 0; j < kPre; ++j) R[j] = rp[j];
     const uint32_t r0 = W[D.a[0]] ^ W[D.b[0]];
     const uint32_t r1 = W[D.a[1]] ^ W[D.b[1]];
     const uint32_t r2 = W[D.a[2]] ^ W[D.b[2]];
@@ -634,7 +554,7 @@ __device__ __forceinline__ void redraw_body(uint32_t* W, uint32_t* S, const Desc
     uint32_t v = (glk && (D.mflag & 0x10))
                      ? glink_heat_bath(W, glk + (D.dst - n), rp, thr0, thr1, thr2, thr3, g, sweep,
                                        pidx, k0, k1)
-                     : heat_bath_links<NP>(r0, r1, r2, m, m == 0 ? ~0u : 0u, m == 1 ? ~0u : 0u,
+                     : heat_bath_links(r0, r1, r2, m, m == 0 ? ~0u : 0u, m == 1 ? ~0u : 0u,
                                        m == 2 ? ~0u : 0u, m == 3 ? ~0u : 0u, R, fast, thr0, thr1,
                                        thr2, thr3, g, sweep, pidx, k0, k1);
     if (cpl && (D.mflag & 8)) {
@@ -650,40 +570,15 @@ __device__ __forceinline__ void redraw_body(uint32_t* W, uint32_t* S, const Desc
   }
 }
 
-// Out-of-line entries (the plain one keeps the hot kernel's call site small:
-// one argument more there costs register spills).  NP: Philox outputs
-// computed ahead per p-bit.
-template <int NP>
-__device__ __noinline__ void redraw_extra(uint32_t* W, uint32_t* S, const Desc* sdesc,
-                                          const uint4* cur, int pst, int lo, int first, int hi,
-                                          int stride, int n, FastThr fast, uint32_t thr0,
-                                          uint32_t thr1, uint32_t thr2, uint32_t thr3, uint32_t g,
-                                          uint32_t sweep, uint32_t k0, uint32_t k1) {
-  redraw_body<NP>(W, S, sdesc, cur, pst, lo, first, hi, stride, n, fast, thr0, thr1, thr2, thr3,
-                  g, sweep, k0, k1, nullptr, nullptr, nullptr);
-}
-__device__ __noinline__ void redraw_extra_coupled(uint32_t* W, uint32_t* S, const Desc* sdesc,
-                                                  const uint4* cur, int lo, int first, int hi,
-                                                  int stride, int n, FastThr fast, uint32_t thr0,
-                                                  uint32_t thr1, uint32_t thr2, uint32_t thr3,
-                                                  uint32_t g, uint32_t sweep, uint32_t k0,
-                                                  uint32_t k1, const Cpl* cpl, const GLink* glk,
-                                                  const TAcc* tacc) {
-  redraw_body<kPre>(W, S, sdesc, cur, 1, lo, first, hi, stride, n, fast, thr0, thr1, thr2, thr3,
-                    g, sweep, k0, k1, cpl, glk, tacc);
-}
-
 // Runs `n_sweeps` sweeps (absolute indices sweep0...) of one chain group.
 // NC = colour steps per sweep (2..4; the model's classes NC.. are empty).
-// WGT: the instantiation for runs with general-gate models (coupled p-bits
+// The kernel of runs with general-gate models (coupled p-bits
 // get the Metropolis acceptance, records add FP64 phases); plain models run
-// through it unchanged.  EXT (with WGT): some model also has Toffoli links
-// or two-qubit tables; without them those paths are compiled out, so the
-// coupled-gate consumers and the recorder keep their shorter code.  BAL
-// (plain runs whose tables leave room): 16 planes computed ahead per p-bit
-// in three buffers, produced evenly over the colour steps; otherwise 12
-// planes in two buffers, each class's produced during the step before.
-template <int NC, bool WGT, bool EXT, bool BAL, bool DEC = false>
+// through it unchanged.  EXT: some model also has Toffoli links or two-qubit
+// tables; without them those paths are compiled out, so the coupled-gate
+// consumers and the recorder keep their shorter code.  12 planes are computed
+// ahead per p-bit, each class's during the step before.
+template <int NC, bool EXT>
 __device__ void run_group(const RunModelDev& rm_g, uint32_t g, uint32_t sweep0, uint32_t n_sweeps,
                           Shape sh, int max_col_all, uint32_t* smem, WsHeader* hdr) {
   // run and model constants held in registers for the whole launch
@@ -698,7 +593,7 @@ __device__ void run_group(const RunModelDev& rm_g, uint32_t g, uint32_t sweep0, 
   const bool producer = !consumer && !recorder;
   const int ptid = tid - sh.cons;
 
-  const bool wgt_m = WGT && rm.cpl != nullptr;
+  const bool wgt_m = rm.cpl != nullptr;
   const int nug = md.n_ug;
   const int iw = image_words(n, d);
   uint32_t* W = smem;
@@ -712,20 +607,11 @@ __device__ void run_group(const RunModelDev& rm_g, uint32_t g, uint32_t sweep0, 
   // (rounded up to 16 bytes: the class table and the plane buffers follow)
   const uint32_t hist_words = (rm.bins * (wgt_m ? 10u : 8u) + 3u) & ~3u;
   ClassEnt* sclass = reinterpret_cast<ClassEnt*>(after_rec + (rm.hist_smem ? hist_words : 0u));
-  // plane buffers, each [max_col][KP] sweep-draw outputs, then (general-
-  // gate runs) [cons][kPreC] acceptance outputs of the class's first cons
-  // p-bits: three with BAL (producers up to two steps ahead), else two (one
-  // step ahead)
+  // two plane buffers, each [max_col][kPre] sweep-draw outputs, then
+  // [cons][kPreC] acceptance outputs of the class's first cons p-bits
   uint4* planes = reinterpret_cast<uint4*>(sclass + 4 * sh.cons);
-  static_assert(!(WGT && BAL), "balanced production: plain runs only");
-  constexpr int KP = BAL ? kPrePlain : kPre;  // Philox outputs computed ahead per p-bit
-  // Output j of a class's k-th p-bit: [k KP + j] (48-byte rows, conflict-free
-  // for 16-byte loads across a warp), or with BAL [j max_col + k] (plane-
-  // major: 64-byte rows would put 16 lanes on the same four banks).
-  const int pst = BAL ? max_col_all : 1;
-  auto pidx_of = [&](int k, int j) { return BAL ? j * max_col_all + k : k * KP + j; };
-  const int acc_off = max_col_all * KP;
-  const int pbuf = acc_off + (WGT ? sh.cons * kPreC : 0);
+  const int acc_off = max_col_all * kPre;
+  const int pbuf = acc_off + sh.cons * kPreC;
 
   // ---- load the group image and the tables
   const uint32_t* gstate = rm.state + (size_t)g * npb;
@@ -752,7 +638,7 @@ __device__ void run_group(const RunModelDev& rm_g, uint32_t g, uint32_t sweep0, 
     }
     sdesc[i] = D;
     Rec R = rm.rec[i];
-    if (R.vd >= nw || R.va >= nw || R.vb >= nw || R.pa >= nw || R.pb >= nw || (WGT && R.vc >= nw)) {
+    if (R.vd >= nw || R.va >= nw || R.vb >= nw || R.pa >= nw || R.pb >= nw || R.vc >= nw) {
       set_status(hdr, PB_EINVAL);
       R.vd = R.va = R.vb = R.pa = R.pb = (uint16_t)zero_idx(n, d);
       R.vc = (uint16_t)ones_idx(n, d);
@@ -824,13 +710,11 @@ __device__ void run_group(const RunModelDev& rm_g, uint32_t g, uint32_t sweep0, 
       const int m = D.mflag & 3;
       if (m == 1) { D.a[1] = D.a[0]; D.b[1] = D.b[0]; }
       ClassEnt E;
-      // plain runs: link words as shared-window addresses (no add per load)
-      const uint32_t lbase = WGT ? 0u : (uint32_t)__cvta_generic_to_shared(W);
 #pragma unroll
-      for (int l = 0; l < 3; ++l) { E.la[l] = lbase + 4u * D.a[l]; E.lb[l] = lbase + 4u * D.b[l]; }
+      for (int l = 0; l < 3; ++l) { E.la[l] = 4u * D.a[l]; E.lb[l] = 4u * D.b[l]; }
       E.dst = 4u * D.dst;
       E.m = (uint32_t)m;
-      if (WGT && (D.mflag & 8)) E.m |= 0x100u;     // coupled: Metropolis acceptance
+      if (D.mflag & 8) E.m |= 0x100u;     // coupled: Metropolis acceptance
       if (EXT && (D.mflag & 0x10)) E.m |= 0x200u;  // general links (Toffoli)
       if (EXT && (D.mflag & 0x20)) E.m |= 0x400u;  // table acceptance
       E.M0 = m == 0 ? ~0u : 0u;
@@ -840,21 +724,18 @@ __device__ void run_group(const RunModelDev& rm_g, uint32_t g, uint32_t sweep0, 
       sclass[c * sh.cons + tid] = E;
     }
   }
-  // Producers: the Philox outputs of class C at sweep `sw` into `buf`
-  // (three-buffer runs: with the group's round keys computed once).
-  [[maybe_unused]] PhiloxGroup pg;
-  if constexpr (BAL) pg = philox_group(gglob, k0, k1);
+  // Producers: the Philox outputs of class C at sweep `sw` into `buf`.
   auto produce = [&](auto cc, uint32_t sw, uint4* buf) {
     constexpr int C = decltype(cc)::value;
     const int lo = col_lo[C], K = col_hi[C] - lo;
-    const int nsw = K * KP;
-    const int nacc = WGT ? (K < sh.cons ? K : sh.cons) * kPreC : 0;
+    const int nsw = K * kPre;
+    const int nacc = (K < sh.cons ? K : sh.cons) * kPreC;
 #pragma unroll 1
     for (int u = ptid; u < nsw + nacc; u += sh.prod) {
-      if (!WGT || u < nsw) {
-        const int i = u / KP, j = u - i * KP;
+      if (u < nsw) {
+        const int i = u / kPre, j = u - i * kPre;
         const uint32_t p = (uint32_t)(sdesc[lo + i].dst - n) | (kTagSweep << 16);
-        buf[pidx_of(i, j)] = philox4x32_10(make_uint4(gglob, sw, p, (uint32_t)j), k0, k1);
+        buf[i * kPre + j] = philox4x32_10(make_uint4(gglob, sw, p, (uint32_t)j), k0, k1);
       } else {  // acceptance draws: coupled p-bits only
         const int a = u - nsw, i = a / kPreC, j = a - i * kPreC;
         const Desc& D = sdesc[lo + i];
@@ -867,19 +748,6 @@ __device__ void run_group(const RunModelDev& rm_g, uint32_t g, uint32_t sweep0, 
   if (producer && n_sweeps > 0u) produce(std::integral_constant<int, 0>{}, sweep0, planes);
   __syncthreads();
 
-  // BAL: production spread evenly over the colour steps.  The units
-  // of a sweep are its U Philox outputs (KP a p-bit) in step order; step t
-  // needs its own before it starts, and the three buffers hold steps t (being
-  // read), t + 1 and t + 2.  During step t the producers take the next units
-  // of the stream up to max(D(t + 2), pp + B) and at most D(t + 3), B = U /
-  // NC a step (D(t): units of the steps before t; pp: units produced so
-  // far, kept relative to the current sweep's first unit).  With classes of
-  // 116, 91 and 33 p-bits this is 320 outputs a step instead of 364, 132 and
-  // 464 for the next step alone.
-  [[maybe_unused]] const uint32_t U = (uint32_t)(KP * col_hi[NC - 1]);  // every p-bit is in one class
-  [[maybe_unused]] const uint32_t B = (U + NC - 1) / NC;
-  [[maybe_unused]] uint32_t pp = (uint32_t)(KP * col_hi[0]);  // units of step 0, produced above
-
   const FastThr fast = fast_thresholds(thr1, thr2);
   Recorder rec;
   unsigned long long n_valid = 0ull, n_samples = 0ull;  // recorder warp only
@@ -890,130 +758,81 @@ __device__ void run_group(const RunModelDev& rm_g, uint32_t g, uint32_t sweep0, 
   // One colour class C of sweep sweep0 + s: consumers redraw it from plane
   // buffer C & 1, producers fill the other buffer for the next class, the
   // recorder works on the previous sweep's snapshot; then one barrier.
-  [[maybe_unused]] ClassEnt En{};  // DEC consumers: the coming step's table entry
-  if (DEC && consumer) En = sclass[tid];
   auto step = [&](auto cc, uint32_t s) {
     constexpr int C = decltype(cc)::value;
     const uint32_t sweep = sweep0 + s;
     uint32_t* S = smem + iw * (1 + (s & 1u));
     // plane buffer of global step s NC + C
     const uint32_t gstep = s * (uint32_t)NC + (uint32_t)C;
-    // (with three colour steps a sweep, step C's buffer is C)
-    const uint32_t cslot = BAL ? (NC == 3 ? (uint32_t)C : gstep % 3u) : (gstep & 1u);
+    const uint32_t cslot = gstep & 1u;
     const uint4* cur = planes + cslot * pbuf;
     if (consumer) {
       const int lo = col_lo[C], hi = col_hi[C], K = hi - lo;
       // the first p-bit of every consumer from its table entry; warps with no
       // p-bit in this class skip it (their entries are dummies)
       if (warp * 32 < K) {
-        const ClassEnt E = DEC ? En : sclass[C * sh.cons + tid];
-        const uint4* rp = cur + pidx_of(tid < K ? tid : 0, 0);  // dummies: any planes
-        uint4 R[KP];
+        const ClassEnt E = sclass[C * sh.cons + tid];
+        const uint4* rp = cur + (tid < K ? tid : 0) * kPre;  // dummies: any planes
+        uint4 R[kPre];
 #pragma unroll
-        for (int j = 0; j < KP; ++j) R[j] = rp[j * pst];
+        for (int j = 0; j < kPre; ++j) R[j] = rp[j];
         const char* Wb = reinterpret_cast<const char*>(W);
         auto word = [&](uint32_t off) { return *reinterpret_cast<const uint32_t*>(Wb + off); };
-        auto link = [&](uint32_t a) {  // plain runs: a is a shared-window address
-          if constexpr (WGT) return word(a);
-          uint32_t x;
-          asm volatile("ld.shared.u32 %0, [%1];" : "=r"(x) : "r"(a));
-          return x;
-        };
-        const uint32_t r0 = link(E.la[0]) ^ link(E.lb[0]);
-        const uint32_t r1 = link(E.la[1]) ^ link(E.lb[1]);
-        const uint32_t r2 = link(E.la[2]) ^ link(E.lb[2]);
+        const uint32_t r0 = word(E.la[0]) ^ word(E.lb[0]);
+        const uint32_t r1 = word(E.la[1]) ^ word(E.lb[1]);
+        const uint32_t r2 = word(E.la[2]) ^ word(E.lb[2]);
         const uint32_t pidx = (E.dst / 4u - (uint32_t)n) | (kTagSweep << 16);
         // coupled p-bit: its coupling entry and neighbour words, loaded
         // ahead so that their latency overlaps the heat-bath draw
-        [[maybe_unused]] Cpl Cp{};
-        [[maybe_unused]] uint32_t old_w = 0u, win_w = 0u, wout_w = 0u;
-        if constexpr (WGT) {
-          if (E.m & 0x100u) {
-            Cp = rm.cpl[E.dst / 4u - (uint32_t)n];
-            old_w = word(E.dst);
-            win_w = W[Cp.win];
-            wout_w = W[Cp.wout];
-          }
+        Cpl Cp{};
+        uint32_t old_w = 0u, win_w = 0u, wout_w = 0u;
+        if (E.m & 0x100u) {
+          Cp = rm.cpl[E.dst / 4u - (uint32_t)n];
+          old_w = word(E.dst);
+          win_w = W[Cp.win];
+          wout_w = W[Cp.wout];
         }
         uint32_t v;
         if (EXT && (E.m & 0x200u))
           v = glink_heat_bath(W, rm.glk + (E.dst / 4u - (uint32_t)n), rp, thr0, thr1, thr2, thr3,
                               gglob, sweep, pidx, k0, k1);
         else
-          v = heat_bath_links<KP>(r0, r1, r2, (int)(WGT ? (E.m & 3u) : E.m), E.M0, E.M1, E.M2, E.M3, R,
+          v = heat_bath_links(r0, r1, r2, (int)(E.m & 3u), E.M0, E.M1, E.M2, E.M3, R,
                               fast, thr0, thr1, thr2, thr3, gglob, sweep, pidx, k0, k1);
-        if constexpr (WGT) {
-          if (E.m & 0x100u) {
-            const uint32_t p = E.dst / 4u - (uint32_t)n;
-            v = couple_accept_body(Cp, win_w, wout_w, old_w, v, cur + acc_off + tid * kPreC,
-                                   gglob, sweep, p, k0, k1);
-          }
-          if (EXT && (E.m & 0x400u)) {  // a second acceptance factor: the tables' energy
-            const uint32_t p = E.dst / 4u - (uint32_t)n;
-            v = table_accept(W, rm.tacc + p, word(E.dst), v, gglob, sweep, p, k0, k1);
-          }
+        if (E.m & 0x100u) {
+          const uint32_t p = E.dst / 4u - (uint32_t)n;
+          v = couple_accept_body(Cp, win_w, wout_w, old_w, v, cur + acc_off + tid * kPreC, gglob,
+                                 sweep, p, k0, k1);
+        }
+        if (EXT && (E.m & 0x400u)) {  // a second acceptance factor: the tables' energy
+          const uint32_t p = E.dst / 4u - (uint32_t)n;
+          v = table_accept(W, rm.tacc + p, word(E.dst), v, gglob, sweep, p, k0, k1);
         }
         *reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(W) + E.dst) = v;
         *reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(S) + E.dst) = v;
       }
       // further p-bits (a class larger than the consumers) from the descriptors
       if (K > sh.cons) {
-        if constexpr (WGT)
-          redraw_extra_coupled(W, S, sdesc, cur, lo, tid + sh.cons, hi, sh.cons, n, fast, thr0,
-                               thr1, thr2, thr3, gglob, sweep, k0, k1, rm.cpl,
-                               EXT ? rm.glk : nullptr, EXT ? rm.tacc : nullptr);
-        else
-          redraw_extra<KP>(W, S, sdesc, cur, pst, lo, tid + sh.cons, hi, sh.cons, n, fast, thr0, thr1, thr2,
-                       thr3, gglob, sweep, k0, k1);
+        redraw_extra_coupled(W, S, sdesc, cur, lo, tid + sh.cons, hi, sh.cons, n, fast, thr0, thr1,
+                             thr2, thr3, gglob, sweep, k0, k1, rm.cpl, EXT ? rm.glk : nullptr,
+                             EXT ? rm.tacc : nullptr);
       }
-      // DEC: the next step's table entry, loaded before the barrier so that
-      // the step after it starts with the link loads
-      if constexpr (DEC) En = sclass[((C + 1) % NC) * sh.cons + tid];
     } else if (producer) {
-      if constexpr (!BAL) {
-        // the next step: class C + 1 of this sweep, or class 0 of the next one
-        const uint32_t nxt = gstep + 1u;
-        if constexpr (C + 1 < NC) {
-          produce(std::integral_constant<int, C + 1>{}, sweep, planes + (nxt & 1u) * pbuf);
-        } else {
-          if (s + 1u < n_sweeps)
-            produce(std::integral_constant<int, 0>{}, sweep + 1u, planes + (nxt & 1u) * pbuf);
-        }
+      // the next step: class C + 1 of this sweep, or class 0 of the next one
+      const uint32_t nxt = gstep + 1u;
+      if constexpr (C + 1 < NC) {
+        produce(std::integral_constant<int, C + 1>{}, sweep, planes + (nxt & 1u) * pbuf);
       } else {
-        // steps gstep + 1 and gstep + 2: classes C1, C2 of sweeps s + c1, s + c2
-        constexpr int C1 = (C + 1) % NC, C2 = (C + 2) % NC, C3 = (C + 3) % NC;
-        constexpr uint32_t c1 = (C + 1) / NC, c2 = (C + 2) / NC, c3 = (C + 3) / NC;
-        const uint32_t d1 = c1 * U + (uint32_t)(KP * col_lo[C1]);  // D(t + k) - D(sweep s)
-        const uint32_t d2 = c2 * U + (uint32_t)(KP * col_lo[C2]);
-        uint32_t lim = c3 * U + (uint32_t)(KP * col_lo[C3]);
-        if (s + 1u >= n_sweeps && lim > U) lim = U;  // no unit past the launch
-        uint32_t tgt = pp + B > d2 ? pp + B : d2;
-        if (tgt > lim) tgt = lim;
-#pragma unroll 1
-        for (uint32_t u = pp + (uint32_t)ptid; u < tgt; u += (uint32_t)sh.prod) {
-          const bool second = u >= d2;
-          const uint32_t r = u - (second ? d2 : d1);  // unit within its step
-          const uint32_t i = r / (uint32_t)KP, j = r - i * (uint32_t)KP;
-          const int lo = second ? col_lo[C2] : col_lo[C1];
-          const uint32_t sw = sweep + (second ? c2 : c1);
-          const uint32_t slot = NC == 3 ? (second ? (uint32_t)((C + 2) % 3) : (uint32_t)((C + 1) % 3))
-                                        : (gstep + (second ? 2u : 1u)) % 3u;
-          const uint32_t p = (uint32_t)(sdesc[lo + (int)i].dst - n) | (kTagSweep << 16);
-          planes[slot * (uint32_t)pbuf + j * (uint32_t)max_col_all + i] =
-              philox4x32_10_group(pg, sw, p, j);
-        }
-        pp = tgt;
+        if (s + 1u < n_sweeps)
+          produce(std::integral_constant<int, 0>{}, sweep + 1u, planes + (nxt & 1u) * pbuf);
       }
     } else {
       // records run one sweep behind: the record of sweep s-1 reads its
       // snapshot in NC-1 parts (steps 0..NC-2 of sweep s), then reduces and
-      // bins (step NC-1).  General-gate runs, and plain runs with DEC: the
-      // recorder takes no part in the colour steps' barriers, only in the
-      // sweep's last one (it reads the previous sweep's snapshot, which no
-      // consumer writes during this sweep, at its own pace; measured 3-4 %
-      // faster on general_mid and on the large workload, whose classes take
-      // two consumer passes, and slower on the plain mid circuit, whose
-      // steps it then crowds).
+      // bins (step NC-1).  The recorder takes no part in the colour steps'
+      // barriers, only in the sweep's last one (it reads the previous sweep's
+      // snapshot, which no consumer writes during this sweep, at its own
+      // pace; measured 3-4 % faster on general_mid).
       if (s > 0u && recorded(sweep - 1u)) {
         const uint32_t* Sp = smem + iw * (1 + ((s + 1u) & 1u));
         if constexpr (C == 0) rec.clear();
@@ -1026,11 +845,11 @@ __device__ void run_group(const RunModelDev& rm_g, uint32_t g, uint32_t sweep0, 
           if (EXT && rm.trec) rec.read_t(Sp, rm.trec, B0 * md.n_tr / D, B1 * md.n_tr / D, lane);
         } else {
           rec.reduce(Sp, n, d, lane);
-          rec.bin<WGT>(rm_g, g, batch, lane, shist, n_valid, n_samples);
+          rec.bin<true>(rm_g, g, batch, lane, shist, n_valid, n_samples);
         }
       }
     }
-    if constexpr ((WGT || DEC) && C + 1 < NC) {
+    if constexpr (C + 1 < NC) {
       if (!recorder) bar_sync_first(1u, (uint32_t)(sh.cons + sh.prod));
     } else {
       __syncthreads();  // (the sweep's end: snapshots change parity)
@@ -1042,7 +861,6 @@ __device__ void run_group(const RunModelDev& rm_g, uint32_t g, uint32_t sweep0, 
     step(std::integral_constant<int, 1>{}, s);
     if constexpr (NC > 2) step(std::integral_constant<int, 2>{}, s);
     if constexpr (NC > 3) step(std::integral_constant<int, 3>{}, s);
-    if constexpr (BAL) pp -= U;  // production pointer relative to the next sweep
   }
   // the record still in flight: the last sweep's
   if (recorder) {
@@ -1053,7 +871,7 @@ __device__ void run_group(const RunModelDev& rm_g, uint32_t g, uint32_t sweep0, 
       if (wgt_m) rec.read_u(Sl, rm.uph, 0, nug, lane);
       if (EXT && rm.trec) rec.read_t(Sl, rm.trec, 0, md.n_tr, lane);
       rec.reduce(Sl, n, d, lane);
-      rec.bin<WGT>(rm_g, g, batch, lane, shist, n_valid, n_samples);
+      rec.bin<true>(rm_g, g, batch, lane, shist, n_valid, n_samples);
     }
   }
   __syncthreads();
@@ -1088,13 +906,8 @@ __device__ void run_group(const RunModelDev& rm_g, uint32_t g, uint32_t sweep0, 
 }
 
 // One CTA per chain group of every model of the run (flat group index).
-constexpr int kMaxThreads = 608;  // 224 consumers + 352 producers + 1 recorder warp
-// General-gate runs: at most 512 threads, so that the longer consumer and
-// recorder paths get 128 registers.
-constexpr int kMaxThreadsWgt = 512;
-
-template <int NC, bool WGT, bool EXT, bool BAL, bool DEC = false>
-__global__ void __launch_bounds__(WGT ? kMaxThreadsWgt : (BAL ? kSweepThreadsBal : kMaxThreads)) sweep_kernel(const RunModelDev* __restrict__ rm,
+template <int NC, bool EXT>
+__global__ void __launch_bounds__(kSweepThreadsWgt) sweep_kernel(const RunModelDev* __restrict__ rm,
                                                      int n_models, uint32_t total_groups,
                                                      uint32_t n_sweeps, Shape sh, int max_col,
                                                      WsHeader* hdr) {
@@ -1106,30 +919,7 @@ __global__ void __launch_bounds__(WGT ? kMaxThreadsWgt : (BAL ? kSweepThreadsBal
   const RunModelDev& r = rm[mi];
   const uint32_t g = flat - r.group_base;
   if (g >= r.groups) return;
-  run_group<NC, WGT, EXT, BAL, DEC>(r, g, sweep0, n_sweeps, sh, max_col, smem, hdr);
-}
-
-// Persistent form: a fixed grid pops (model, group) items from a
-// cost-ordered work list with one atomic counter.  No CTA waits on another.
-template <int NC, bool BAL>
-__global__ void __launch_bounds__(BAL ? kSweepThreadsBal : kMaxThreads) sweep_persistent_kernel(
-    const RunModelDev* __restrict__ rm, int n_models, const uint32_t* __restrict__ work,
-    uint32_t n_work, uint32_t n_sweeps, Shape sh, int max_col, WsHeader* hdr) {
-  extern __shared__ __align__(16) uint32_t smem[];
-  const uint32_t sweep0 = hdr->sweep0;
-  __shared__ uint32_t item;
-  for (;;) {
-    if (threadIdx.x == 0) item = atomicAdd(&hdr->work_next, 1u);
-    __syncthreads();
-    const uint32_t it = item;
-    __syncthreads();
-    if (it >= n_work) break;
-    const uint32_t flat = work[it];
-    const int mi = find_model(rm, n_models, flat);
-    const RunModelDev& r = rm[mi];
-    const uint32_t g = flat - r.group_base;
-    if (g < r.groups) run_group<NC, false, false, BAL>(r, g, sweep0, n_sweeps, sh, max_col, smem, hdr);
-  }
+  run_group<NC, EXT>(r, g, sweep0, n_sweeps, sh, max_col, smem, hdr);
 }
 
 // ---------------------------------------------------------------------------
@@ -1522,67 +1312,27 @@ cudaError_t launch_init(const RunModelDev* d_rm, int n_models, uint32_t total_gr
 // Sweep index advance after a launch (the sweep kernels read hdr->sweep0, so
 // one captured graph replays correctly any number of times).
 __global__ void advance_kernel(WsHeader* hdr, uint32_t n_sweeps) { hdr->sweep0 += n_sweeps; }
-__global__ void reset_work_kernel(WsHeader* hdr) { hdr->work_next = 0u; }
 
 // nc: colour steps per sweep (the largest over the launch's models; 2..4).
-// wgt: some model has general gates (the WGT instantiation); ext: some model
+// ext: some model
 // has Toffoli links or two-qubit tables (EXT).
 cudaError_t launch_sweeps(const RunModelDev* d_rm, int n_models, uint32_t total_groups,
                           uint32_t n_sweeps, int cons, int prod, int max_col, int nc,
-                          size_t smem_bytes, WsHeader* hdr, cudaStream_t st, bool wgt, bool ext,
-                          bool bal, bool dec) {
+                          size_t smem_bytes, WsHeader* hdr, cudaStream_t st, bool ext) {
   const int threads = cons + prod + 32;
   const Shape sh{cons, prod};
   auto go = [&](auto kern) {
     kern<<<total_groups, threads, smem_bytes, st>>>(d_rm, n_models, total_groups, n_sweeps, sh,
                                                     max_col, hdr);
   };
-  if (wgt && ext) {
-    if (nc <= 2) go(sweep_kernel<2, true, true, false>);
-    else if (nc == 3) go(sweep_kernel<3, true, true, false>);
-    else go(sweep_kernel<4, true, true, false>);
-  } else if (wgt) {
-    if (nc <= 2) go(sweep_kernel<2, true, false, false>);
-    else if (nc == 3) go(sweep_kernel<3, true, false, false>);
-    else go(sweep_kernel<4, true, false, false>);
-  } else if (bal && dec) {
-    if (nc <= 2) go(sweep_kernel<2, false, false, true, true>);
-    else if (nc == 3) go(sweep_kernel<3, false, false, true, true>);
-    else go(sweep_kernel<4, false, false, true, true>);
-  } else if (bal) {
-    if (nc <= 2) go(sweep_kernel<2, false, false, true>);
-    else if (nc == 3) go(sweep_kernel<3, false, false, true>);
-    else go(sweep_kernel<4, false, false, true>);
+  if (ext) {
+    if (nc <= 2) go(sweep_kernel<2, true>);
+    else if (nc == 3) go(sweep_kernel<3, true>);
+    else go(sweep_kernel<4, true>);
   } else {
-    if (nc <= 2) go(sweep_kernel<2, false, false, false>);
-    else if (nc == 3) go(sweep_kernel<3, false, false, false>);
-    else go(sweep_kernel<4, false, false, false>);
-  }
-  advance_kernel<<<1, 1, 0, st>>>(hdr, n_sweeps);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_sweeps_persistent(const RunModelDev* d_rm, int n_models, const uint32_t* d_work,
-                                     uint32_t n_work, uint32_t n_sweeps, int cons, int prod,
-                                     int max_col, int nc, int grid, size_t smem_bytes,
-                                     WsHeader* hdr, cudaStream_t st, bool bal) {
-  const int threads = cons + prod + 32;
-  // the work counter is cleared by a kernel (a graph may hold this launch
-  // inside a device-side loop, whose body takes kernels)
-  reset_work_kernel<<<1, 1, 0, st>>>(hdr);
-  const Shape sh{cons, prod};
-  auto go = [&](auto kern) {
-    kern<<<grid, threads, smem_bytes, st>>>(d_rm, n_models, d_work, n_work, n_sweeps, sh, max_col,
-                                            hdr);
-  };
-  if (bal) {
-    if (nc <= 2) go(sweep_persistent_kernel<2, true>);
-    else if (nc == 3) go(sweep_persistent_kernel<3, true>);
-    else go(sweep_persistent_kernel<4, true>);
-  } else {
-    if (nc <= 2) go(sweep_persistent_kernel<2, false>);
-    else if (nc == 3) go(sweep_persistent_kernel<3, false>);
-    else go(sweep_persistent_kernel<4, false>);
+    if (nc <= 2) go(sweep_kernel<2, false>);
+    else if (nc == 3) go(sweep_kernel<3, false>);
+    else go(sweep_kernel<4, false>);
   }
   advance_kernel<<<1, 1, 0, st>>>(hdr, n_sweeps);
   return cudaGetLastError();
@@ -1633,9 +1383,8 @@ cudaError_t launch_philox_fill(const uint32_t* ctr, uint32_t k0, uint32_t k1, ui
   return cudaGetLastError();
 }
 
-size_t sweep_smem_bytes(int n, int d, int cons, int max_col, uint32_t hist_bins, bool wgt,
-                        bool bal) {
-  return group_smem_bytes(n, d, cons, max_col, hist_bins, wgt && !bal, bal && !wgt);
+size_t sweep_smem_bytes(int n, int d, int cons, int max_col, uint32_t hist_bins) {
+  return group_smem_bytes(n, d, cons, max_col, hist_bins);
 }
 
 // Opt the sweep kernels into large dynamic shared memory (called once per
@@ -1644,27 +1393,12 @@ cudaError_t sweep_prepare() {
   const int big = (int)kSweepSmemMax;
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(sweep_kernel<2, false, false, false>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_kernel<3, false, false, false>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_kernel<4, false, false, false>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_kernel<2, false, false, true>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_kernel<3, false, false, true>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_kernel<4, false, false, true>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_kernel<2, false, false, true, true>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_kernel<3, false, false, true, true>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_kernel<4, false, false, true, true>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_kernel<2, true, false, false>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_kernel<3, true, false, false>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_kernel<4, true, false, false>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_kernel<2, true, true, false>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_kernel<3, true, true, false>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_kernel<4, true, true, false>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_persistent_kernel<2, false>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_persistent_kernel<3, false>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_persistent_kernel<4, false>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_persistent_kernel<2, true>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_persistent_kernel<3, true>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_persistent_kernel<4, true>, a, big)) != cudaSuccess)
+  if ((e = cudaFuncSetAttribute(sweep_kernel<2, false>, a, big)) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(sweep_kernel<3, false>, a, big)) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(sweep_kernel<4, false>, a, big)) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(sweep_kernel<2, true>, a, big)) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(sweep_kernel<3, true>, a, big)) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(sweep_kernel<4, true>, a, big)) != cudaSuccess)
     return e;
   if ((e = cudaFuncSetAttribute(elim_kernel<false, 8>, a, big)) != cudaSuccess ||
       (e = cudaFuncSetAttribute(elim_kernel<false, 16>, a, big)) != cudaSuccess ||
@@ -1673,16 +1407,6 @@ cudaError_t sweep_prepare() {
       (e = cudaFuncSetAttribute(elim_kernel<true, 16>, a, big)) != cudaSuccess)
     return e;
   return cudaFuncSetAttribute(elim_kernel<true, 32>, a, big);
-}
-
-int sweep_max_blocks_per_sm(int threads, size_t smem, bool bal) {
-  int blocks = 0;
-  const cudaError_t e =
-      bal ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, sweep_persistent_kernel<4, true>,
-                                                          threads, smem)
-          : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, sweep_persistent_kernel<4, false>,
-                                                          threads, smem);
-  return e == cudaSuccess ? blocks : 1;
 }
 
 }  // namespace pb
