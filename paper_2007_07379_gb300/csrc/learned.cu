@@ -344,12 +344,13 @@ __global__ void __launch_bounds__(1024) collect_kernel(const uint32_t* __restric
   if (tid == 0) *count = base;
 }
 
-// Training rows from collected paths: row r takes path i and layer j drawn
+// Training rows (and their transpose, [kin x rows]) from collected paths: row r takes path i and layer j drawn
 // from Philox (key = seed, counter (r, step, 3 << 16, 0)); input s_{j-1},
 // target bits s_j.
 __global__ void train_rows_kernel(const uint32_t* __restrict__ paths, unsigned long long n_paths,
                                   uint32_t beta, int n, int d, int kin, int rows, uint32_t k0,
-                                  uint32_t k1, uint32_t step, __nv_bfloat16* X, float* target) {
+                                  uint32_t k1, uint32_t step, __nv_bfloat16* X,
+                                  __nv_bfloat16* Xt, float* target) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= rows) return;
   const uint4 u = philox4x32_10(make_uint4((uint32_t)r, step, 3u << 16, 0u), k0, k1);
@@ -359,6 +360,10 @@ __global__ void train_rows_kernel(const uint32_t* __restrict__ paths, unsigned l
   const uint32_t* p = paths + i * d;
   const uint32_t prev = j == 1 ? beta : p[j - 2];
   write_row(X, kin, n, d, r, prev, j);
+  const __nv_bfloat16 one = __float2bfloat16(1.f), mone = __float2bfloat16(-1.f),
+                      zero = __float2bfloat16(0.f);
+  for (int i = 0; i < kin; ++i)  // the row as a column of the transpose
+    Xt[(size_t)i * rows + r] = i < n ? (((prev >> i) & 1u) ? one : mone) : (i == n + j - 1 ? one : zero);
   const uint32_t nxt = p[j - 1];
   for (int q = 0; q < n; ++q) target[(size_t)r * n + q] = (float)((nxt >> q) & 1u);
 }
@@ -715,9 +720,8 @@ PB_API int pb_mlp_train_paths(pb_mlp* mlp, const uint32_t* d_paths, uint64_t n_p
   for (int s = 0; s < steps && e == cudaSuccess; ++s) {
     train_rows_kernel<<<(rows + T - 1) / T, T, 0, mlp->st>>>(d_paths, n_paths, beta, mlp->n, mlp->d,
                                                              mlp->kin, rows, k0, k1, (uint32_t)s,
-                                                             mlp->X, mlp->target);
-    if ((e = mlp_forward_rows(mlp, rows)) != cudaSuccess) break;
-    if ((e = mlp_backward_rows(mlp, rows)) != cudaSuccess) break;
+                                                             mlp->X, mlp->Xt, mlp->target);
+    if ((e = mlp_gradient_rows(mlp, rows)) != cudaSuccess) break;
     if (d_losses) cudaMemcpyAsync(d_losses + s, mlp->loss, 4, cudaMemcpyDeviceToDevice, mlp->st);
     e = mlp_adam_step(mlp, lr);
   }

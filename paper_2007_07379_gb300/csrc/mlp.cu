@@ -1,12 +1,19 @@
 // BF16 tensor-core GEMM on tcgen05 (sm_103a) and the small kernels around
 // it that the learned proposal's MLP needs (forward, backward, Adam).
 //
-// gemm_bf16_tn: D[M x N] = epilogue(alpha * A[M x K] * B[N x K]^T), A and B
-// bf16 row-major with K contiguous ("TN"), accumulation in fp32 in TMEM.
-// One CTA of 4 warps computes a 128 x BN tile (BN <= 256): K is staged in
-// chunks of 64 into shared memory in the canonical K-major layout, one
-// thread issues the MMAs and commits them to an mbarrier, all threads wait
-// (bounded), and the four warps read their 32 TMEM lanes for the epilogue.
+// gemm_tile: D[M x N] = epilogue(alpha * A[M x K] * B[N x K]^T), A and B bf16
+// row-major with K contiguous ("TN"), accumulation in fp32 in TMEM.  One CTA
+// of 4 warps computes a TM x BN tile (TM 64 or 128, BN <= 256): K passes
+// through shared memory in chunks of 128 (canonical K-major layout) in up to
+// four stages filled by cp.async while earlier chunks multiply; one thread
+// issues the MMAs of a chunk and commits them to the stage's mbarrier, all
+// threads wait (bounded) before the stage is filled again, and the warps read
+// their TMEM lanes for the epilogue.  What bounds it at the network's sizes
+// (256 x 256 weights, 4096 rows) is latency, not rate: a launch of a few
+// hundred tiles with one to 32 chunks each.  Small tiles where the rows
+// leave SMs idle, and the stages, are for that: the weight gradients (K =
+// 4096 rows) took 64 chunks one after the other, load, multiply, wait, 350 of
+// a training step's 583 us.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -26,6 +33,7 @@ enum : int {
   kEpiOutBf16 = 2,  // store bf16 (else fp32)
   kEpiAccum = 4,    // fp32 output: D += x
   kEpiMask = 8,     // x *= (mask[row, col] > 0)   (ReLU derivative)
+  kEpiBce = 16,     // fp32 logits: also the cross-entropy's gradient and terms
 };
 
 struct GemmArgs {
@@ -39,17 +47,38 @@ struct GemmArgs {
   int flags;
   float alpha;
   uint32_t* status;  // set to PB_ETIMEOUT when a bounded wait expires
+  __nv_bfloat16* Dt;  // when set: the result transposed, bf16 [N x ldt]
+  int ldt;
+  // kEpiBce (fp32 logits, N = npad >= n): the gradient of the binary cross-
+  // entropy against target [M x n], dY = (sigmoid(l) - t) / M, bf16 in D2 and
+  // Dt, and the loss terms (fp32 [M x n])
+  const float* target;
+  __nv_bfloat16* D2;
+  float* terms;
+  int n;
+  int tm, bn;  // tile (gemm_tiles)
 };
 
-// Tile width: N rounded up to 16, at most 256, narrowed to 128 or 64 when
-// the row tiles alone would leave most of the 152 SMs idle.
-__host__ __device__ inline int gemm_tile_n(int M, int N) {
-  int bn = ((N + 15) / 16) * 16;
+constexpr int kGemmK = 128;          // K elements of a stage
+constexpr size_t kGemmSmemMax = 200 * 1024;
+__host__ __device__ inline size_t gemm_stage_bytes(int tm, int bn) {
+  return (size_t)(tm + bn) * kGemmK * 2;
+}
+__host__ __device__ inline int gemm_stages(int tm, int bn) {
+  return 4 * gemm_stage_bytes(tm, bn) <= kGemmSmemMax ? 4 : 2;
+}
+// Tile: 128 rows and N rounded up to 16, at most 256, narrowed step by step to
+// 64 x 32 while the tiles would leave most of the 152 SMs idle.
+inline void gemm_tiles(GemmArgs& g) {
+  int bn = ((g.N + 15) / 16) * 16, tm = 128;
   if (bn > 256) bn = 256;
-  const int mt = (M + 127) / 128;
-  if (bn > 128 && mt * ((N + bn - 1) / bn) < 120) bn = 128;
-  if (bn > 64 && mt * ((N + bn - 1) / bn) < 120) bn = 64;
-  return bn;
+  auto tiles = [&] { return ((g.M + tm - 1) / tm) * ((g.N + bn - 1) / bn); };
+  if (bn > 128 && tiles() < 120) bn = 128;
+  if (bn > 64 && tiles() < 120) bn = 64;
+  if (tiles() < 120) tm = 64;
+  if (bn > 32 && tiles() < 120) bn = 32;
+  g.tm = tm;
+  g.bn = bn;
 }
 __host__ __device__ inline uint32_t tmem_cols(int bn) {
   uint32_t c = 32;
@@ -57,114 +86,216 @@ __host__ __device__ inline uint32_t tmem_cols(int bn) {
   return c;
 }
 
-__global__ void __launch_bounds__(128) gemm_bf16_tn_kernel(GemmArgs g) {
-  extern __shared__ __align__(1024) uint8_t sm[];
-  __shared__ uint64_t mbar;
-  __shared__ uint32_t tmem_base;
-  const int BN = gemm_tile_n(g.M, g.N);
-  uint8_t* sA = sm;            // 128 x 64 bf16 (16 KiB)
-  uint8_t* sB = sm + 16384;    // BN x 64 bf16 (<= 32 KiB)
+// dY element and loss term of one logit (rows B).
+__device__ __forceinline__ float bce_grad(float l, float t, int B) {
+  return (1.f / (1.f + __expf(-l)) - t) / (float)B;
+}
+__device__ __forceinline__ float bce_term(float l, float t, int B) {
+  return (fmaxf(l, 0.f) + log1pf(__expf(-fabsf(l))) - t * l) / (float)B;
+}
+
+// One tile (m0, n0) by the CTA's 128 threads; S stages of dynamic shared
+// memory at sm.
+template <int S>
+__device__ __forceinline__ void gemm_tile(const GemmArgs& g, int m0, int n0, uint8_t* sm,
+                                          uint64_t* mbar, uint32_t* tmem_base) {
+  const int TM = g.tm, BN = g.bn;
+  const uint32_t a_bytes = (uint32_t)TM * kGemmK * 2, stage = (uint32_t)gemm_stage_bytes(TM, BN);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int m0 = blockIdx.x * 128, n0 = blockIdx.y * BN;
   const uint32_t ncols = tmem_cols(BN);
 
-  if (warp == 0) tc::tmem_alloc(&tmem_base, ncols);
+  if (warp == 0) tc::tmem_alloc(tmem_base, ncols);
   if (tid == 0) {
-    tc::mbar_init(&mbar, 1);
+    for (int s = 0; s < S; ++s) tc::mbar_init(&mbar[s], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  // chunk c (K elements 128 c ..) into its stage: two 64-wide halves, each in
+  // the canonical layout; one 16-byte vector = 8 K elements
+  const int nch = (g.K + kGemmK - 1) / kGemmK;
+  auto load = [&](int c) {
+    if (c < nch) {
+      uint8_t* base = sm + (uint32_t)(c % S) * stage;
+      for (int v = tid; v < (TM + BN) * 16; v += 128) {
+        const bool isA = v < TM * 16;
+        const int u = isA ? v : v - TM * 16;
+        const int r = u >> 4, kk = (u & 15) * 8, k = c * kGemmK + kk;
+        const int row = (isA ? m0 : n0) + r;
+        const bool in = row < (isA ? g.M : g.N) && k < g.K;
+        const __nv_bfloat16* p = isA ? g.A : g.B;
+        uint8_t* dst = base + (isA ? 0u : a_bytes) + (uint32_t)(kk >> 6) * (isA ? TM : BN) * 128u +
+                       tc::chunk_offset(r, kk & 63);
+        tc::cp_async16(dst, in ? (const void*)(p + (size_t)row * (isA ? g.lda : g.ldb) + k) : (const void*)p,
+                       in ? 16u : 0u);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+#pragma unroll
+  for (int c = 0; c < S - 1; ++c) load(c);
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  const uint32_t tbase = tmem_base;
-  const uint32_t idesc = tc::idesc_bf16_f32(128, BN);
-  uint32_t phase = 0;
+  const uint32_t tbase = *tmem_base;
+  const uint32_t idesc = tc::idesc_bf16_f32(TM, BN);
   bool ok = true;
 
-  for (int k0 = 0; k0 < g.K; k0 += tc::kChunkK) {
-    // stage A (128 x 64) and B (BN x 64): one 16-byte vector = 8 K-elements
-    for (int v = tid; v < 128 * 8; v += 128) {
-      const int r = v >> 3, c = v & 7, k = k0 + c * 8, row = m0 + r;
-      const bool in = row < g.M && k < g.K;
-      tc::cp_async16(sA + tc::chunk_offset(r, c * 8),
-                     in ? (const void*)(g.A + (size_t)row * g.lda + k) : (const void*)g.A, in ? 16u : 0u);
-    }
-    for (int v = tid; v < BN * 8; v += 128) {
-      const int r = v >> 3, c = v & 7, k = k0 + c * 8, row = n0 + r;
-      const bool in = row < g.N && k < g.K;
-      tc::cp_async16(sB + tc::chunk_offset(r, c * 8),
-                     in ? (const void*)(g.B + (size_t)row * g.ldb + k) : (const void*)g.B, in ? 16u : 0u);
-    }
-    tc::cp_async_wait_all();
+  for (int c = 0; c < nch; ++c) {
+    // the stage of chunk c - 1 is filled again: its MMAs must be done
+    if (c > 0) ok = tc::mbar_wait(&mbar[(c - 1) % S], (uint32_t)((c - 1) / S) & 1u);
+    load(c + S - 1);
+    asm volatile("cp.async.wait_group %0;" ::"n"(S - 1) : "memory");
     tc::fence_proxy_async_smem();
-    __syncthreads();
-    if (tid == 0) {
-      tc::fence_after_sync();
-      const uint32_t a0 = tc::smem_u32(sA), b0 = tc::smem_u32(sB);
-#pragma unroll
-      for (int s = 0; s < tc::kChunkK / 16; ++s) {
-        if (k0 + 16 * s >= g.K) break;
-        // K-step s covers the K-chunks 2s, 2s+1 (LBO apart)
-        const uint64_t ad = tc::smem_desc(a0 + s * 2 * tc::kLBO, tc::kLBO, tc::kSBO);
-        const uint64_t bd = tc::smem_desc(b0 + s * 2 * tc::kLBO, tc::kLBO, tc::kSBO);
-        tc::mma_bf16(tbase, ad, bd, idesc, (k0 > 0) || (s > 0));
-      }
-      tc::mma_commit(&mbar);
-    }
     // one decision for the whole CTA: a thread that gave up and one that saw
     // the commit must take the same branch (the loop has barriers)
-    ok = __syncthreads_and(tc::mbar_wait(&mbar, phase)) != 0;
-    phase ^= 1u;
+    ok = __syncthreads_and(ok) != 0;
     if (!ok) {
       if (tid == 0 && g.status) atomicCAS(g.status, 0u, (uint32_t)PB_ETIMEOUT);
+      if (tid == 0) tc::mbar_wait(&mbar[(c - 1) % S], (uint32_t)((c - 1) / S) & 1u);  // drain (bounded)
       break;
     }
-    tc::fence_after_sync();
-    __syncthreads();  // shared operands may be overwritten now
+    if (tid == 0) {
+      tc::fence_after_sync();
+      const uint32_t a0 = tc::smem_u32(sm + (uint32_t)(c % S) * stage), b0 = a0 + a_bytes;
+#pragma unroll
+      for (int s = 0; s < kGemmK / 16; ++s) {
+        if (c * kGemmK + 16 * s >= g.K) break;
+        // K-step s covers two 8-wide K columns (LBO apart) of half s / 4
+        const uint32_t ao = (uint32_t)(s >> 2) * TM * 128u + (uint32_t)(s & 3) * 2u * tc::kLBO;
+        const uint32_t bo = (uint32_t)(s >> 2) * BN * 128u + (uint32_t)(s & 3) * 2u * tc::kLBO;
+        const uint64_t ad = tc::smem_desc(a0 + ao, tc::kLBO, tc::kSBO);
+        const uint64_t bd = tc::smem_desc(b0 + bo, tc::kLBO, tc::kSBO);
+        tc::mma_bf16(tbase, ad, bd, idesc, (c > 0) || (s > 0));
+      }
+      tc::mma_commit(&mbar[c % S]);
+    }
   }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  if (ok) {
+    const bool done = tc::mbar_wait(&mbar[(nch - 1) % S], (uint32_t)((nch - 1) / S) & 1u);
+    ok = __syncthreads_and(done) != 0;
+    if (!ok && tid == 0) {
+      if (g.status) atomicCAS(g.status, 0u, (uint32_t)PB_ETIMEOUT);
+      tc::mbar_wait(&mbar[(nch - 1) % S], (uint32_t)((nch - 1) / S) & 1u);
+    }
+  }
+  tc::fence_after_sync();
 
   if (ok) {
-    const int row = m0 + warp * 32 + lane;
+    // accumulator rows: TM = 128: TMEM lane = row; TM = 64: row r at lane
+    // 32 (r / 16) + r % 16
+    const int row = m0 + (TM == 128 ? warp * 32 + lane : warp * 16 + lane);
+    const bool live = row < g.M && (TM == 128 || lane < 16);
     for (int c0 = 0; c0 < BN; c0 += 16) {
       float v[16];
       tc::tmem_ld16(tbase + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
-      if (row >= g.M) continue;
+      if (!live) continue;
+      const int col0 = n0 + c0;
+      const bool full = col0 + 16 <= g.N;
+      __align__(16) __nv_bfloat16 mk[16];
+      if ((g.flags & kEpiMask) && full && (g.ldm & 7) == 0 && ((uintptr_t)g.mask & 15) == 0) {
+        const uint4* src = reinterpret_cast<const uint4*>(g.mask + (size_t)row * g.ldm + col0);
+        reinterpret_cast<uint4*>(mk)[0] = src[0];
+        reinterpret_cast<uint4*>(mk)[1] = src[1];
+      } else if (g.flags & kEpiMask) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+          mk[i] = col0 + i < g.N ? g.mask[(size_t)row * g.ldm + col0 + i] : __float2bfloat16(0.f);
+      }
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
-        const int col = n0 + c0 + i;
+        const int col = col0 + i;
         if (col >= g.N) continue;
         float x = g.alpha * v[i];
         if (g.bias) x += g.bias[col];
         if (g.flags & kEpiRelu) x = fmaxf(x, 0.f);
-        if (g.flags & kEpiMask)
-          x = (__bfloat162float(g.mask[(size_t)row * g.ldm + col]) > 0.f) ? x : 0.f;
-        if (g.flags & kEpiOutBf16) {
-          reinterpret_cast<__nv_bfloat16*>(g.D)[(size_t)row * g.ldd + col] = __float2bfloat16(x);
+        if (g.flags & kEpiMask) x = (__bfloat162float(mk[i]) > 0.f) ? x : 0.f;
+        v[i] = x;
+      }
+      if (g.flags & kEpiBce) {
+        __align__(16) __nv_bfloat16 gb[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          const int col = col0 + i;
+          float d = 0.f;
+          if (col < g.n) {
+            const float t = g.target[(size_t)row * g.n + col];
+            d = bce_grad(v[i], t, g.M);
+            g.terms[(size_t)row * g.n + col] = bce_term(v[i], t, g.M);
+          }
+          gb[i] = __float2bfloat16(d);
+          if (col < g.N) g.Dt[(size_t)col * g.ldt + row] = gb[i];
+        }
+        // (rows of npad elements, a multiple of 16)
+        uint4* dst = reinterpret_cast<uint4*>(g.D2 + (size_t)row * g.N + col0);
+        dst[0] = reinterpret_cast<const uint4*>(gb)[0];
+        dst[1] = reinterpret_cast<const uint4*>(gb)[1];
+      }
+      if (g.flags & kEpiOutBf16) {
+        __align__(16) __nv_bfloat16 o[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) o[i] = __float2bfloat16(v[i]);
+        __nv_bfloat16* d = reinterpret_cast<__nv_bfloat16*>(g.D);
+        if (d) {
+          d += (size_t)row * g.ldd + col0;
+          if (full && (g.ldd & 7) == 0 && ((uintptr_t)g.D & 15) == 0) {
+            reinterpret_cast<uint4*>(d)[0] = reinterpret_cast<const uint4*>(o)[0];
+            reinterpret_cast<uint4*>(d)[1] = reinterpret_cast<const uint4*>(o)[1];
+          } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+              if (col0 + i < g.N) d[i] = o[i];
+          }
+        }
+        if (g.Dt) {
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            if (col0 + i < g.N) g.Dt[(size_t)(col0 + i) * g.ldt + row] = o[i];
+        }
+      } else {
+        float* d = reinterpret_cast<float*>(g.D) + (size_t)row * g.ldd + col0;
+        if (full && !(g.flags & kEpiAccum) && (g.ldd & 3) == 0 && ((uintptr_t)g.D & 15) == 0) {
+#pragma unroll
+          for (int i = 0; i < 16; i += 4)
+            *reinterpret_cast<float4*>(d + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
         } else {
-          float* d = reinterpret_cast<float*>(g.D) + (size_t)row * g.ldd + col;
-          *d = (g.flags & kEpiAccum) ? *d + x : x;
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            if (col0 + i < g.N) d[i] = (g.flags & kEpiAccum) ? d[i] + v[i] : v[i];
         }
       }
     }
   }
-  if (!ok && tid == 0) tc::mbar_wait(&mbar, phase ^ 1u);  // let MMAs in flight drain (bounded)
   tc::fence_before_sync();
   __syncthreads();
   if (warp == 0) tc::tmem_dealloc(tbase, ncols);
 }
 
+template <int S>
+__global__ void __launch_bounds__(128) gemm_bf16_tn_kernel(GemmArgs g) {
+  extern __shared__ __align__(1024) uint8_t sm[];
+  __shared__ uint64_t mbar[S];
+  __shared__ uint32_t tmem_base;
+  gemm_tile<S>(g, blockIdx.x * g.tm, blockIdx.y * g.bn, sm, mbar, &tmem_base);
+}
+
 // One-time set-up outside any stream capture (shared-memory opt-in).
 cudaError_t mlp_fused_prepare();
+cudaError_t grads_prepare();
 cudaError_t mlp_prepare() {
-  cudaError_t e = cudaFuncSetAttribute(gemm_bf16_tn_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, 48 * 1024);
+  const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e = cudaFuncSetAttribute(gemm_bf16_tn_kernel<2>, a, (int)kGemmSmemMax);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_bf16_tn_kernel<4>, a, (int)kGemmSmemMax);
+  if (e == cudaSuccess) e = grads_prepare();
   return e == cudaSuccess ? mlp_fused_prepare() : e;
 }
 
-cudaError_t launch_gemm_bf16(const GemmArgs& g, cudaStream_t st) {
-  const int BN = gemm_tile_n(g.M, g.N);
-  dim3 grid((g.M + 127) / 128, (g.N + BN - 1) / BN);
-  gemm_bf16_tn_kernel<<<grid, 128, 16384 + BN * 64 * 2, st>>>(g);
+cudaError_t launch_gemm_bf16(GemmArgs g, cudaStream_t st) {
+  gemm_tiles(g);
+  dim3 grid((g.M + g.tm - 1) / g.tm, (g.N + g.bn - 1) / g.bn);
+  const int S = gemm_stages(g.tm, g.bn);
+  const size_t smem = (size_t)S * gemm_stage_bytes(g.tm, g.bn);
+  if (S == 4) gemm_bf16_tn_kernel<4><<<grid, 128, smem, st>>>(g);
+  else gemm_bf16_tn_kernel<2><<<grid, 128, smem, st>>>(g);
   return cudaGetLastError();
 }
 
@@ -269,108 +400,150 @@ cudaError_t transpose_bf16(const __nv_bfloat16* src, int R, int C, __nv_bfloat16
   return cudaGetLastError();
 }
 
-// fp32 [R x C] -> bf16 [R x C] and, when dst_t is given, bf16 [C x R].
-__global__ void to_bf16_kernel(const float* __restrict__ src, int R, int C,
-                               __nv_bfloat16* __restrict__ dst, __nv_bfloat16* __restrict__ dst_t) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (size_t)R * C) return;
-  const __nv_bfloat16 v = __float2bfloat16(src[i]);
-  dst[i] = v;
-  if (dst_t) {
-    const size_t r = i / C, c = i % C;
-    dst_t[c * R + r] = v;
+// Every parameter's bf16 copies from one fp32 weight (index i of the flat
+// block): the row-major copy, the transpose the backward pass reads, and the
+// canonical K-major image the fused kernels load: core matrices of 8 rows x
+// 8 elements (128 bytes), K-adjacent ones 128 bytes apart, 8-row groups
+// 16 K bytes apart (W2 in K-chunks of 64).
+struct Bf16Views {
+  __nv_bfloat16 *W1, *W2, *W3, *W2t, *W3t, *W1p, *W2p, *W3p;
+  int kin, H, npad, n;
+};
+__device__ __forceinline__ uint32_t canonical_index(int r, int c, int K) {
+  return (uint32_t)((r >> 3) * (K * 8) + (c >> 3) * 64 + (r & 7) * 8 + (c & 7));
+}
+__device__ __forceinline__ void write_bf16(const Bf16Views& b, uint32_t i, float w) {
+  const uint32_t n1 = (uint32_t)(b.H * b.kin), n2 = (uint32_t)(b.H * b.H), n3 = (uint32_t)(b.npad * b.H);
+  const uint32_t H = (uint32_t)b.H;
+  const __nv_bfloat16 v = __float2bfloat16(w);
+  if (i < n1) {  // W1 [H x kin]
+    b.W1[i] = v;
+    const uint32_t r = i / (uint32_t)b.kin;
+    b.W1p[canonical_index((int)r, (int)(i - r * (uint32_t)b.kin), b.kin)] = v;
+    return;
+  }
+  i -= n1;
+  if (i < H) return;  // b1
+  i -= H;
+  if (i < n2) {  // W2 [H x H]
+    b.W2[i] = v;
+    const uint32_t r = i / H, c = i - r * H;
+    b.W2t[c * H + r] = v;
+    const uint32_t k0 = c & ~63u;
+    b.W2p[H * k0 + canonical_index((int)r, (int)(c - k0), (int)min(64u, H - k0))] = v;
+    return;
+  }
+  i -= n2;
+  if (i < H) return;  // b2
+  i -= H;
+  if (i < n3) {  // W3 [npad x H]
+    b.W3[i] = v;
+    const uint32_t r = i / H, c = i - r * H;
+    b.W3t[c * (uint32_t)b.npad + r] = v;
+    b.W3p[canonical_index((int)r, (int)c, b.H)] = v;
   }
 }
-
-// Columns [k0, k0 + K) of a row-major bf16 [R x ld] matrix into the canonical
-// K-major image the tensor cores read from shared memory: core matrices of
-// 8 rows x 8 elements (128 bytes), K-adjacent ones 128 bytes apart, 8-row
-// groups K * 16 bytes apart.
-__global__ void pack_canonical_kernel(const __nv_bfloat16* __restrict__ src, int R, int ld, int k0,
-                                      int K, __nv_bfloat16* __restrict__ dst) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;  // one 8-element vector
-  const int vecs = K / 8;
-  if (i >= R * vecs) return;
-  const int r = i / vecs, c = i % vecs;
-  const uint4 v = *reinterpret_cast<const uint4*>(src + (size_t)r * ld + k0 + c * 8);
-  *reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(dst) + (size_t)(r >> 3) * (K * 16) + c * 128 +
-                            (r & 7) * 16) = v;
+__global__ void refresh_bf16_kernel(const float* __restrict__ w, uint32_t count, Bf16Views b) {
+  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < count) write_bf16(b, i, w[i]);
 }
 
-// dY = (sigmoid(l) - t) / B for the first n columns (0 beyond), bf16, both
-// layouts.
-__device__ __forceinline__ float bce_grad(float l, float t, int B) {
-  return (1.f / (1.f + __expf(-l)) - t) / (float)B;
-}
-__global__ void bce_grad_kernel(const float* __restrict__ logits, const float* __restrict__ target,
-                                int B, int n, int npad, __nv_bfloat16* __restrict__ dY,
-                                __nv_bfloat16* __restrict__ dYt) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= B * npad) return;
-  const int r = i / npad, c = i % npad;
-  const float g = c < n ? bce_grad(logits[(size_t)r * npad + c], target[(size_t)r * n + c], B) : 0.f;
-  const __nv_bfloat16 gb = __float2bfloat16(g);
-  dY[(size_t)r * npad + c] = gb;
-  dYt[(size_t)c * B + r] = gb;
+// The weight gradients of one backward pass in one launch: tiles of gW2, gW1
+// and gW3 (each a sum over the rows, K = rows), then the bias gradients (one
+// warp per row of dZ2t / dZ1t), the n columns of db3 and the loss.  Every sum
+// is taken in a fixed order, so that a training run is reproducible bit for
+// bit.
+struct GradArgs {
+  GemmArgs w[3];        // gW2, gW1, gW3
+  int tiles[3], mt[3];  // tiles of each, tiles along M
+  const __nv_bfloat16 *dZ2t, *dZ1t;
+  float *db2, *db1, *db3, *loss;
+  const float *logits, *target, *terms;
+  int H, B, n, npad;
+};
+constexpr int kGradStages = 4;
+constexpr int kGradTm = 64, kGradBn = 32;  // 24 KB a stage
+
+// out[j] = sum_b M[j][b] (bf16 rows, fp32 sums), one warp per row.
+__device__ __forceinline__ void rowsum_bf16(const __nv_bfloat16* __restrict__ row, int C, int lane,
+                                            float* __restrict__ out) {
+  float s = 0.f;
+#pragma unroll 8
+  for (int c = lane; c < C; c += 32) s += __bfloat162float(row[c]);
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  if (lane == 0) *out = s;
 }
 
-// Block c < n: db3[c] = sum over the rows of the fp32 gradient of column c;
-// block n: loss = the mean BCE, -[t log s(l) + (1-t) log s(-l)] =
-// softplus(l) - t l, computed stably.  Each sum is taken in a fixed order
-// (per-thread strided partial sums, then a tree), so that a training run is
-// reproducible bit for bit.
-__global__ void __launch_bounds__(256) bce_sums_kernel(const float* __restrict__ logits,
-                                                       const float* __restrict__ target, int B,
-                                                       int n, int npad, float* __restrict__ db3,
-                                                       float* __restrict__ loss) {
+__global__ void __launch_bounds__(128) grads_kernel(GradArgs a) {
+  extern __shared__ __align__(1024) uint8_t sm[];
+  __shared__ uint64_t mbar[kGradStages];
+  __shared__ uint32_t tmem_base;
   __shared__ float part[256];
-  const int c = blockIdx.x, tid = threadIdx.x;
-  float acc = 0.f;
-  if (c < n) {
-    for (int r = tid; r < B; r += 256)
-      acc += bce_grad(logits[(size_t)r * npad + c], target[(size_t)r * n + c], B);
-  } else {
-    for (int i = tid; i < B * n; i += 256) {
-      const int r = i / n, q = i % n;
-      const float l = logits[(size_t)r * npad + q], t = target[(size_t)r * n + q];
-      acc += (fmaxf(l, 0.f) + log1pf(__expf(-fabsf(l))) - t * l) / (float)B;
+  int b = blockIdx.x;
+  const int tid = threadIdx.x;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    if (b < a.tiles[k]) {
+      gemm_tile<kGradStages>(a.w[k], (b % a.mt[k]) * kGradTm, (b / a.mt[k]) * a.w[k].bn, sm, mbar,
+                             &tmem_base);
+      return;
     }
+    b -= a.tiles[k];
   }
-  part[tid] = acc;
+  const int rs = (a.H + 3) / 4;  // bias rows, four warps a CTA
+  if (b < 2 * rs) {
+    const int row = (b < rs ? b : b - rs) * 4 + (tid >> 5);
+    if (row < a.H)
+      rowsum_bf16((b < rs ? a.dZ2t : a.dZ1t) + (size_t)row * a.B, a.B, tid & 31,
+                  (b < rs ? a.db2 : a.db1) + row);
+    return;
+  }
+  // 256 strided partial sums and a tree: db3[c] (fp32 gradients), or the loss
+  const int c = b - 2 * rs;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int p = tid + 128 * h;
+    float acc = 0.f;
+    if (c < a.n) {
+#pragma unroll 4
+      for (int r = p; r < a.B; r += 256)
+        acc += bce_grad(a.logits[(size_t)r * a.npad + c], a.target[(size_t)r * a.n + c], a.B);
+    } else {
+#pragma unroll 8
+      for (int i = p; i < a.B * a.n; i += 256) acc += a.terms[i];
+    }
+    part[p] = acc;
+  }
   __syncthreads();
   for (int s = 128; s > 0; s >>= 1) {
     if (tid < s) part[tid] += part[tid + s];
     __syncthreads();
   }
-  if (tid == 0) {
-    if (c < n) db3[c] = part[0];
-    else if (loss) *loss = part[0];
-  }
+  if (tid == 0) *(c < a.n ? a.db3 + c : a.loss) = part[0];
+}
+cudaError_t grads_prepare() {
+  return cudaFuncSetAttribute(grads_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)(kGradStages * gemm_stage_bytes(kGradTm, kGradBn)));
 }
 
-// out[j] = sum_b M[j][b] (bf16 rows, fp32 sums), one warp per row.
-__global__ void rowsum_bf16_kernel(const __nv_bfloat16* __restrict__ Mt, int R, int C,
-                                   float* __restrict__ out) {
-  const int row = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-  const int lane = threadIdx.x & 31;
-  if (row >= R) return;
-  float s = 0.f;
-  for (int c = lane; c < C; c += 32) s += __bfloat162float(Mt[(size_t)row * C + c]);
-  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-  if (lane == 0) out[row] = s;
-}
-
+// One Adam step, the bf16 copies with it; the padded rows of W3 / b3 (flat
+// indices in [z0, z1) and [z2, z3)) stay zero.
 __global__ void adam_kernel(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m,
-                            float* __restrict__ v, size_t count, float lr, float b1, float b2,
-                            float eps, float c1, float c2) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+                            float* __restrict__ v, uint32_t count, float lr, float b1, float b2,
+                            float eps, float c1, float c2, uint32_t z0, uint32_t z1, uint32_t z2,
+                            uint32_t z3, Bf16Views b) {
+  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const float gi = g[i];
   const float mi = b1 * m[i] + (1.f - b1) * gi;
   const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
   m[i] = mi;
   v[i] = vi;
-  w[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  float x = w[i];
+  x -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  if ((i >= z0 && i < z1) || (i >= z2 && i < z3)) x = 0.f;
+  w[i] = x;
+  write_bf16(b, i, x);
 }
 
 }  // namespace pb
@@ -379,7 +552,7 @@ namespace {
 
 struct MlpLayout {
   size_t w, m, v, g, W1, W2, W3, W2t, W3t, W1p, W2p, W3p, X, Xt, H1, H1t, H2, H2t, dY, dYt, dZ2,
-      dZ2t, dZ1, dZ1t, logits, target, loss, status, total;
+      dZ2t, dZ1t, logits, target, terms, loss, status, total;
 };
 
 MlpLayout mlp_layout(int kin, int H, int npad, int B) {
@@ -414,10 +587,10 @@ MlpLayout mlp_layout(int kin, int H, int npad, int B) {
   L.dYt = take((size_t)B * npad * 2);
   L.dZ2 = take((size_t)B * H * 2);
   L.dZ2t = take((size_t)B * H * 2);
-  L.dZ1 = take((size_t)B * H * 2);
   L.dZ1t = take((size_t)B * H * 2);
   L.logits = take((size_t)B * npad * 4);
   L.target = take((size_t)B * npad * 4);
+  L.terms = take((size_t)B * npad * 4);
   L.loss = take(256);
   L.status = take(16);
   L.total = (p + 255) & ~(size_t)255;
@@ -433,10 +606,11 @@ int mlp_dims(int n, int d, int hidden, int batch, int* kin, int* npad) {
   return PB_OK;
 }
 
-// GEMM helper: D = epi(A[M x K] B[N x K]^T)
-cudaError_t mm(const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, void* D, int ldd,
-               int M, int N, int K, int flags, const float* bias, const __nv_bfloat16* mask,
-               int ldm, cudaStream_t st, uint32_t* status) {
+// D = epi(A[M x K] B[N x K]^T) of this network (and its transpose, bf16
+// [N x M], when Dt is set).
+pb::GemmArgs mm(const pb_mlp* p, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb,
+                void* D, int ldd, int M, int N, int K, int flags, const float* bias = nullptr,
+                const __nv_bfloat16* mask = nullptr, __nv_bfloat16* Dt = nullptr) {
   pb::GemmArgs g{};
   g.A = A;
   g.B = B;
@@ -446,111 +620,115 @@ cudaError_t mm(const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb,
   g.lda = lda;
   g.ldb = ldb;
   g.ldd = ldd;
-  g.ldm = ldm;
+  g.ldm = ldd;
   g.M = M;
   g.N = N;
   g.K = K;
   g.flags = flags;
   g.alpha = 1.f;
-  g.status = status;
-  return pb::launch_gemm_bf16(g, st);
+  g.status = p->status;
+  g.Dt = Dt;
+  g.ldt = M;
+  return g;
 }
 
-// bf16 copies of the fp32 master weights (W2t, W3t transposed for the backward).
+pb::Bf16Views bf16_views(const pb_mlp* p) {
+  return {p->W1, p->W2, p->W3, p->W2t, p->W3t, p->W1p, p->W2p, p->W3p, p->kin, p->H, p->npad, p->n};
+}
+
+// bf16 copies of the fp32 master weights.
 cudaError_t refresh_bf16(pb_mlp* p) {
-  const int T = 256;
-  const float* w = p->w;
-  size_t c = (size_t)p->H * p->kin;
-  pb::to_bf16_kernel<<<(unsigned)((c + T - 1) / T), T, 0, p->st>>>(w + p->off_W1, p->H, p->kin, p->W1, nullptr);
-  c = (size_t)p->H * p->H;
-  pb::to_bf16_kernel<<<(unsigned)((c + T - 1) / T), T, 0, p->st>>>(w + p->off_W2, p->H, p->H, p->W2, p->W2t);
-  c = (size_t)p->npad * p->H;
-  pb::to_bf16_kernel<<<(unsigned)((c + T - 1) / T), T, 0, p->st>>>(w + p->off_W3, p->npad, p->H, p->W3, p->W3t);
-  // canonical images for the fused kernel (W2 in K-chunks of 64)
-  auto pack = [&](const __nv_bfloat16* src, int R, int ld, int k0, int K, __nv_bfloat16* dst) {
-    const int v = R * (K / 8);
-    pb::pack_canonical_kernel<<<(v + T - 1) / T, T, 0, p->st>>>(src, R, ld, k0, K, dst);
-  };
-  pack(p->W1, p->H, p->kin, 0, p->kin, p->W1p);
-  for (int k0 = 0; k0 < p->H; k0 += 64)
-    pack(p->W2, p->H, p->H, k0, std::min(64, p->H - k0), p->W2p + (size_t)p->H * k0);
-  pack(p->W3, p->npad, p->H, 0, p->H, p->W3p);
+  const unsigned c = (unsigned)p->n_params;
+  pb::refresh_bf16_kernel<<<(c + 255) / 256, 256, 0, p->st>>>(p->w, c, bf16_views(p));
   return cudaGetLastError();
 }
 
 // Forward of `rows` inputs already in p->X: H1, H2 (bf16), logits (fp32).
-cudaError_t mlp_fwd(pb_mlp* p, int rows) {
+// train: also what the backward pass needs -- the transposes of H1 and H2,
+// the gradient of the logits against p->target and the loss terms.
+cudaError_t mlp_fwd(pb_mlp* p, int rows, bool train) {
   cudaError_t e;
-  const int flags = pb::kEpiRelu | pb::kEpiOutBf16;
-  if ((e = mm(p->X, p->kin, p->W1, p->kin, p->H1, p->H, rows, p->H, p->kin, flags,
-              p->w + p->off_b1, nullptr, 0, p->st, p->status)) != cudaSuccess)
+  const int flags = pb::kEpiRelu | pb::kEpiOutBf16, H = p->H;
+  if ((e = pb::launch_gemm_bf16(mm(p, p->X, p->kin, p->W1, p->kin, p->H1, H, rows, H, p->kin, flags,
+                                   p->w + p->off_b1, nullptr, train ? p->H1t : nullptr),
+                                p->st)) != cudaSuccess)
     return e;
-  if ((e = mm(p->H1, p->H, p->W2, p->H, p->H2, p->H, rows, p->H, p->H, flags, p->w + p->off_b2,
-              nullptr, 0, p->st, p->status)) != cudaSuccess)
+  if ((e = pb::launch_gemm_bf16(mm(p, p->H1, H, p->W2, H, p->H2, H, rows, H, H, flags,
+                                   p->w + p->off_b2, nullptr, train ? p->H2t : nullptr),
+                                p->st)) != cudaSuccess)
     return e;
-  return mm(p->H2, p->H, p->W3, p->H, p->logits, p->npad, rows, p->npad, p->H, 0,
-            p->w + p->off_b3, nullptr, 0, p->st, p->status);
+  pb::GemmArgs g = mm(p, p->H2, H, p->W3, H, p->logits, p->npad, rows, p->npad, H,
+                      train ? pb::kEpiBce : 0, p->w + p->off_b3, nullptr, p->dYt);
+  g.target = p->target;
+  g.D2 = p->dY;
+  g.terms = p->terms;
+  g.n = p->n;
+  return pb::launch_gemm_bf16(g, p->st);
 }
 
-// Backward of the mean BCE over `rows` (targets in p->target): gradients
-// into p->g, loss into p->loss[0].
+// Backward of the mean BCE over `rows` after mlp_fwd(.., train): gradients
+// into p->g, loss into p->loss[0].  p->Xt holds the inputs' transpose.
 cudaError_t mlp_bwd(pb_mlp* p, int rows) {
   cudaError_t e;
-  const int B = rows, H = p->H, T = 256;
-  cudaMemsetAsync(p->g, 0, p->n_params * 4, p->st);
-  cudaMemsetAsync(p->loss, 0, 4, p->st);
-  pb::bce_grad_kernel<<<(B * p->npad + T - 1) / T, T, 0, p->st>>>(p->logits, p->target, B, p->n,
-                                                                   p->npad, p->dY, p->dYt);
-  pb::bce_sums_kernel<<<p->n + 1, 256, 0, p->st>>>(p->logits, p->target, B, p->n, p->npad,
-                                                   p->g + p->off_b3, p->loss);
-  if ((e = pb::transpose_bf16(p->H2, B, H, p->H2t, p->st)) != cudaSuccess) return e;
-  if ((e = pb::transpose_bf16(p->H1, B, H, p->H1t, p->st)) != cudaSuccess) return e;
-  if ((e = pb::transpose_bf16(p->X, B, p->kin, p->Xt, p->st)) != cudaSuccess) return e;
-  // gW3 = dY^T H2
-  if ((e = mm(p->dYt, B, p->H2t, B, p->g + p->off_W3, H, p->npad, H, B, 0, nullptr, nullptr, 0,
-              p->st, p->status)) != cudaSuccess)
+  const int B = rows, H = p->H;
+  const int flags = pb::kEpiMask | pb::kEpiOutBf16;
+  // dZ2 = (dY W3) * [H2 > 0], dZ1 = (dZ2 W2) * [H1 > 0] (its transpose only)
+  if ((e = pb::launch_gemm_bf16(mm(p, p->dY, p->npad, p->W3t, p->npad, p->dZ2, H, B, H, p->npad, flags,
+                                   nullptr, p->H2, p->dZ2t), p->st)) != cudaSuccess ||
+      (e = pb::launch_gemm_bf16(mm(p, p->dZ2, H, p->W2t, H, nullptr, H, B, H, H, flags, nullptr, p->H1,
+                                   p->dZ1t), p->st)) != cudaSuccess)
     return e;
-  // dZ2 = (dY W3) * [H2 > 0]
-  if ((e = mm(p->dY, p->npad, p->W3t, p->npad, p->dZ2, H, B, H, p->npad,
-              pb::kEpiMask | pb::kEpiOutBf16, nullptr, p->H2, H, p->st, p->status)) != cudaSuccess)
-    return e;
-  if ((e = pb::transpose_bf16(p->dZ2, B, H, p->dZ2t, p->st)) != cudaSuccess) return e;
-  // gW2 = dZ2^T H1, gb2 = column sums of dZ2
-  if ((e = mm(p->dZ2t, B, p->H1t, B, p->g + p->off_W2, H, H, H, B, 0, nullptr, nullptr, 0,
-              p->st, p->status)) != cudaSuccess)
-    return e;
-  pb::rowsum_bf16_kernel<<<(H + 7) / 8, 256, 0, p->st>>>(p->dZ2t, H, B, p->g + p->off_b2);
-  // dZ1 = (dZ2 W2) * [H1 > 0]
-  if ((e = mm(p->dZ2, H, p->W2t, H, p->dZ1, H, B, H, H, pb::kEpiMask | pb::kEpiOutBf16, nullptr,
-              p->H1, H, p->st, p->status)) != cudaSuccess)
-    return e;
-  if ((e = pb::transpose_bf16(p->dZ1, B, H, p->dZ1t, p->st)) != cudaSuccess) return e;
-  // gW1 = dZ1^T X, gb1 = column sums of dZ1
-  if ((e = mm(p->dZ1t, B, p->Xt, B, p->g + p->off_W1, p->kin, H, p->kin, B, 0, nullptr, nullptr,
-              0, p->st, p->status)) != cudaSuccess)
-    return e;
-  pb::rowsum_bf16_kernel<<<(H + 7) / 8, 256, 0, p->st>>>(p->dZ1t, H, B, p->g + p->off_b1);
+  // gW2 = dZ2^T H1, gW1 = dZ1^T X, gW3 = dY^T H2, the bias gradients, the loss
+  pb::GradArgs a{};
+  a.w[0] = mm(p, p->dZ2t, B, p->H1t, B, p->g + p->off_W2, H, H, H, B, 0);
+  a.w[1] = mm(p, p->dZ1t, B, p->Xt, B, p->g + p->off_W1, p->kin, H, p->kin, B, 0);
+  a.w[2] = mm(p, p->dYt, B, p->H2t, B, p->g + p->off_W3, H, p->npad, H, B, 0);
+  int total = 0;
+  for (int k = 0; k < 3; ++k) {
+    pb::GemmArgs& g = a.w[k];
+    g.tm = pb::kGradTm;
+    g.bn = std::min(pb::kGradBn, (g.N + 15) / 16 * 16);
+    a.mt[k] = (g.M + g.tm - 1) / g.tm;
+    a.tiles[k] = a.mt[k] * ((g.N + g.bn - 1) / g.bn);
+    total += a.tiles[k];
+  }
+  a.dZ2t = p->dZ2t;
+  a.dZ1t = p->dZ1t;
+  a.db2 = p->g + p->off_b2;
+  a.db1 = p->g + p->off_b1;
+  a.db3 = p->g + p->off_b3;
+  a.loss = p->loss;
+  a.logits = p->logits;
+  a.target = p->target;
+  a.terms = p->terms;
+  a.H = H;
+  a.B = B;
+  a.n = p->n;
+  a.npad = p->npad;
+  total += 2 * ((H + 3) / 4) + p->n + 1;
+  pb::grads_kernel<<<total, 128, pb::kGradStages * pb::gemm_stage_bytes(pb::kGradTm, pb::kGradBn),
+                     p->st>>>(a);
   return cudaGetLastError();
 }
 
 }  // namespace
 
 namespace pb {
-cudaError_t mlp_forward_rows(pb_mlp* p, int rows) { return mlp_fwd(p, rows); }
-cudaError_t mlp_backward_rows(pb_mlp* p, int rows) { return mlp_bwd(p, rows); }
+cudaError_t mlp_forward_rows(pb_mlp* p, int rows) { return mlp_fwd(p, rows, false); }
+cudaError_t mlp_gradient_rows(pb_mlp* p, int rows) {
+  const cudaError_t e = mlp_fwd(p, rows, true);
+  return e == cudaSuccess ? mlp_bwd(p, rows) : e;
+}
 cudaError_t mlp_adam_step(pb_mlp* p, float lr) {
   p->step += 1;
   const float b1 = 0.9f, b2 = 0.999f;
   const float c1 = 1.f - std::pow(b1, (float)p->step), c2 = 1.f - std::pow(b2, (float)p->step);
-  const size_t c = p->n_params;
-  adam_kernel<<<(unsigned)((c + 255) / 256), 256, 0, p->st>>>(p->w, p->g, p->m, p->v, c, lr, b1, b2,
-                                                             1e-8f, c1, c2);
-  // keep the padded rows of W3 / b3 at zero
-  if (p->npad > p->n) {
-    cudaMemsetAsync(p->w + p->off_W3 + (size_t)p->n * p->H, 0, (size_t)(p->npad - p->n) * p->H * 4, p->st);
-    cudaMemsetAsync(p->w + p->off_b3 + p->n, 0, (size_t)(p->npad - p->n) * 4, p->st);
-  }
-  return refresh_bf16(p);
+  const uint32_t c = (uint32_t)p->n_params, H = (uint32_t)p->H;
+  const uint32_t w3 = (uint32_t)p->off_W3, b3 = (uint32_t)p->off_b3, n = (uint32_t)p->n, np = (uint32_t)p->npad;
+  adam_kernel<<<(c + 255) / 256, 256, 0, p->st>>>(p->w, p->g, p->m, p->v, c, lr, b1, b2, 1e-8f, c1, c2,
+                                                 w3 + n * H, w3 + np * H, b3 + n, b3 + np,
+                                                 bf16_views(p));
+  return cudaGetLastError();
 }
 }  // namespace pb
 
@@ -597,8 +775,9 @@ PB_API int pb_mlp_create(int n, int d, int hidden, int batch, uint64_t seed, voi
   p->H2 = (__nv_bfloat16*)(b + L.H2); p->H2t = (__nv_bfloat16*)(b + L.H2t);
   p->dY = (__nv_bfloat16*)(b + L.dY); p->dYt = (__nv_bfloat16*)(b + L.dYt);
   p->dZ2 = (__nv_bfloat16*)(b + L.dZ2); p->dZ2t = (__nv_bfloat16*)(b + L.dZ2t);
-  p->dZ1 = (__nv_bfloat16*)(b + L.dZ1); p->dZ1t = (__nv_bfloat16*)(b + L.dZ1t);
+  p->dZ1t = (__nv_bfloat16*)(b + L.dZ1t);
   p->logits = (float*)(b + L.logits); p->target = (float*)(b + L.target); p->loss = (float*)(b + L.loss);
+  p->terms = (float*)(b + L.terms);
   p->status = (uint32_t*)(b + L.status);
   // Initial weights: uniform(-1/sqrt(fan_in), 1/sqrt(fan_in)) from SplitMix64(seed), biases 0.
   std::vector<float> w(p->n_params, 0.f);
@@ -686,7 +865,7 @@ PB_API int pb_mlp_forward(pb_mlp* p, const void* d_x, int rows, float* d_logits)
   if (!p || !d_x || !d_logits || rows <= 0 || rows > p->batch) return PB_EINVAL;
   if (cudaMemcpyAsync(p->X, d_x, (size_t)rows * p->kin * 2, cudaMemcpyDeviceToDevice, p->st) != cudaSuccess)
     return PB_ECUDA;
-  if (mlp_fwd(p, rows) != cudaSuccess) return PB_ECUDA;
+  if (mlp_fwd(p, rows, false) != cudaSuccess) return PB_ECUDA;
   if (cudaMemcpy2DAsync(d_logits, (size_t)p->n * 4, p->logits, (size_t)p->npad * 4, (size_t)p->n * 4,
                         rows, cudaMemcpyDeviceToDevice, p->st) != cudaSuccess)
     return PB_ECUDA;
@@ -700,10 +879,11 @@ PB_API int pb_mlp_forward(pb_mlp* p, const void* d_x, int rows, float* d_logits)
 PB_API int pb_mlp_backward(pb_mlp* p, const void* d_x, const float* d_target, int rows, float* d_loss) {
   if (!p || !d_x || !d_target || rows <= 0 || rows > p->batch || rows % 8) return PB_EINVAL;
   if (cudaMemcpyAsync(p->X, d_x, (size_t)rows * p->kin * 2, cudaMemcpyDeviceToDevice, p->st) != cudaSuccess ||
-      cudaMemcpy2DAsync(p->target, (size_t)p->n * 4, d_target, (size_t)p->n * 4, (size_t)p->n * 4, rows,
-                        cudaMemcpyDeviceToDevice, p->st) != cudaSuccess)
+      cudaMemcpyAsync(p->target, d_target, (size_t)rows * p->n * 4, cudaMemcpyDeviceToDevice, p->st) != cudaSuccess)
     return PB_ECUDA;
-  if (mlp_fwd(p, rows) != cudaSuccess || mlp_bwd(p, rows) != cudaSuccess) return PB_ECUDA;
+  if (pb::transpose_bf16(p->X, rows, p->kin, p->Xt, p->st) != cudaSuccess ||
+      pb::mlp_gradient_rows(p, rows) != cudaSuccess)
+    return PB_ECUDA;
   if (d_loss && cudaMemcpyAsync(d_loss, p->loss, 4, cudaMemcpyDeviceToDevice, p->st) != cudaSuccess)
     return PB_ECUDA;
   return PB_OK;

@@ -295,8 +295,8 @@ struct pb_mlp {
   __nv_bfloat16 *W1p = nullptr, *W2p = nullptr, *W3p = nullptr;
   __nv_bfloat16 *X = nullptr, *Xt = nullptr, *H1 = nullptr, *H1t = nullptr, *H2 = nullptr,
                 *H2t = nullptr, *dY = nullptr, *dYt = nullptr, *dZ2 = nullptr, *dZ2t = nullptr,
-                *dZ1 = nullptr, *dZ1t = nullptr;
-  float *logits = nullptr, *target = nullptr, *loss = nullptr;
+                *dZ1t = nullptr;
+  float *logits = nullptr, *target = nullptr, *terms = nullptr, *loss = nullptr;
   // PB_ETIMEOUT once a bounded wait in one of this network's kernels expired
   // (a word of the workspace, zeroed at creation)
   uint32_t* status = nullptr;
@@ -304,10 +304,12 @@ struct pb_mlp {
 };
 
 namespace pb {
-// Forward / backward of `rows` rows already staged in mlp->X (and
-// mlp->target): logits in mlp->logits [rows x npad], gradients in mlp->g.
+// Forward of `rows` rows already staged in mlp->X: logits in mlp->logits
+// [rows x npad].  Gradients (forward and backward) of the rows staged in
+// mlp->X, mlp->Xt (their transpose, [kin x rows]) and mlp->target: mlp->g and
+// mlp->loss.
 cudaError_t mlp_forward_rows(pb_mlp* p, int rows);
-cudaError_t mlp_backward_rows(pb_mlp* p, int rows);
+cudaError_t mlp_gradient_rows(pb_mlp* p, int rows);
 cudaError_t mlp_adam_step(pb_mlp* p, float lr);
 cudaError_t mlp_prepare();
 cudaError_t mlp_forward_fused(pb_mlp* p, int rows);
