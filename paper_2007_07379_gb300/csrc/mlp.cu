@@ -3,7 +3,7 @@
 //
 // gemm_tile: D[M x N] = epilogue(alpha * A[M x K] * B[N x K]^T), A and B bf16
 // row-major with K contiguous ("TN"), accumulation in fp32 in TMEM.  One CTA
-// of 4 warps computes a TM x BN tile (TM 64 or 128, BN <= 256): K passes
+// computes a TM x BN tile (TM 64 or 128, BN <= 256): K passes
 // through shared memory in chunks of 128 (canonical K-major layout) in up to
 // four stages filled by cp.async while earlier chunks multiply; one thread
 // issues the MMAs of a chunk and commits them to the stage's mbarrier, all
@@ -59,7 +59,7 @@ struct GemmArgs {
   int tm, bn;  // tile (gemm_tiles)
 };
 
-constexpr int kGemmK = 128;          // K elements of a stage
+constexpr int kGemmK = 128;  // K elements of a stage (the copies in gemm_tile cover 16 columns of 8)
 constexpr size_t kGemmSmemMax = 200 * 1024;
 __host__ __device__ inline size_t gemm_stage_bytes(int tm, int bn) {
   return (size_t)(tm + bn) * kGemmK * 2;
@@ -94,15 +94,20 @@ __device__ __forceinline__ float bce_term(float l, float t, int B) {
   return (fmaxf(l, 0.f) + log1pf(__expf(-fabsf(l))) - t * l) / (float)B;
 }
 
-// One tile (m0, n0) by the CTA's 128 threads; S stages of dynamic shared
-// memory at sm.
-template <int S>
+// One tile (m0, n0) by a CTA of nine warps: eight copy and do the epilogue (two
+// to a quadrant of TMEM lanes, each with half of the columns), the ninth
+// issues the MMAs; S stages of dynamic shared memory at sm.  F: the flags, or
+// -1 to read them from g; CTM, CBN: the tile, or 0 to read it from g.
+constexpr int kGemmThreads = 288;
+template <int S, int F, int CTM = 0, int CBN = 0>
 __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int m0, int n0, uint8_t* sm,
                                           uint64_t* mbar, uint32_t* tmem_base) {
-  const int TM = g.tm, BN = g.bn;
+  const int TM = CTM ? CTM : g.tm, BN = CBN ? CBN : g.bn;
   const uint32_t a_bytes = (uint32_t)TM * kGemmK * 2, stage = (uint32_t)gemm_stage_bytes(TM, BN);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const uint32_t ncols = tmem_cols(BN);
+  const int flags = F >= 0 ? F : g.flags;
 
   if (warp == 0) tc::tmem_alloc(tmem_base, ncols);
   if (tid == 0) {
@@ -110,108 +115,149 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int m0, int n0, uin
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   // chunk c (K elements 128 c ..) into its stage: two 64-wide halves, each in
-  // the canonical layout; one 16-byte vector = 8 K elements
+  // the canonical layout.  A thread copies one 8-element column of every
+  // second 8-row group, so that its addresses only advance by constants (a
+  // copy costs a handful of instructions, which is what paces a tile with few
+  // warps); a warp copies 8 rows x 4 columns: 64-byte pieces of the rows, and
+  // in shared memory 128-byte core matrices without bank conflicts.
   const int nch = (g.K + kGemmK - 1) / kGemmK;
+  const int lr = (warp >> 2) * 8 + (lane & 7), lk = ((warp & 3) * 4 + (lane >> 3)) * 8;
+  const uint32_t lo = tc::smem_u32(sm) + tc::chunk_offset(lr, lk & 63);
+  const __nv_bfloat16* pa = g.A + (size_t)(m0 + lr) * g.lda + lk;
+  const __nv_bfloat16* pb = g.B + (size_t)(n0 + lr) * g.ldb + lk;
+  const bool whole = m0 + TM <= g.M && n0 + BN <= g.N;
   auto load = [&](int c) {
     if (c < nch) {
-      uint8_t* base = sm + (uint32_t)(c % S) * stage;
-      for (int v = tid; v < (TM + BN) * 16; v += 128) {
-        const bool isA = v < TM * 16;
-        const int u = isA ? v : v - TM * 16;
-        const int r = u >> 4, kk = (u & 15) * 8, k = c * kGemmK + kk;
-        const int row = (isA ? m0 : n0) + r;
-        const bool in = row < (isA ? g.M : g.N) && k < g.K;
-        const __nv_bfloat16* p = isA ? g.A : g.B;
-        uint8_t* dst = base + (isA ? 0u : a_bytes) + (uint32_t)(kk >> 6) * (isA ? TM : BN) * 128u +
-                       tc::chunk_offset(r, kk & 63);
-        tc::cp_async16(dst, in ? (const void*)(p + (size_t)row * (isA ? g.lda : g.ldb) + k) : (const void*)p,
-                       in ? 16u : 0u);
+      uint32_t d = lo + (uint32_t)(c % S) * stage + (uint32_t)(lk >> 6) * (uint32_t)TM * 128u;
+      uint32_t e = lo + (uint32_t)(c % S) * stage + a_bytes + (uint32_t)(lk >> 6) * (uint32_t)BN * 128u;
+      const __nv_bfloat16 *q = pa, *w = pb;
+      if (whole && (c + 1) * kGemmK <= g.K) {
+#pragma unroll 4
+        for (int r = 0; r < TM; r += 16, d += 2048u, q += (size_t)16 * g.lda) tc::cp_async16(d, q, 16u);
+#pragma unroll 4
+        for (int r = 0; r < BN; r += 16, e += 2048u, w += (size_t)16 * g.ldb)
+          tc::cp_async16(e, w, 16u);
+      } else {
+        const bool kin = c * kGemmK + lk < g.K;
+        const int ra = kin ? g.M - m0 - lr : 0, rb = kin ? g.N - n0 - lr : 0;  // rows left
+#pragma unroll 1
+        for (int r = 0; r < TM; r += 16, d += 2048u, q += (size_t)16 * g.lda)
+          tc::cp_async16(d, r < ra ? (const void*)q : (const void*)g.A, r < ra ? 16u : 0u);
+#pragma unroll 1
+        for (int r = 0; r < BN; r += 16, e += 2048u, w += (size_t)16 * g.ldb)
+          tc::cp_async16(e, r < rb ? (const void*)w : (const void*)g.B, r < rb ? 16u : 0u);
       }
+      pa += kGemmK;
+      pb += kGemmK;
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
+  // chunks loaded ahead; with four stages the MMAs of the previous chunk may
+  // still run while the next ones are issued
+  constexpr int A = S >= 4 ? S - 2 : S - 1;
+  const bool copier = warp < 8;
+  if (copier) {
 #pragma unroll
-  for (int c = 0; c < S - 1; ++c) load(c);
+    for (int c = 0; c < A; ++c) load(c);
+  }
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tbase = *tmem_base;
   const uint32_t idesc = tc::idesc_bf16_f32(TM, BN);
   bool ok = true;
+  auto done = [&](int c) { return tc::mbar_wait(&mbar[c % S], (uint32_t)(c / S) & 1u); };
 
   for (int c = 0; c < nch; ++c) {
-    // the stage of chunk c - 1 is filled again: its MMAs must be done
-    if (c > 0) ok = tc::mbar_wait(&mbar[(c - 1) % S], (uint32_t)((c - 1) / S) & 1u);
-    load(c + S - 1);
-    asm volatile("cp.async.wait_group %0;" ::"n"(S - 1) : "memory");
-    tc::fence_proxy_async_smem();
-    // one decision for the whole CTA: a thread that gave up and one that saw
-    // the commit must take the same branch (the loop has barriers)
-    ok = __syncthreads_and(ok) != 0;
-    if (!ok) {
-      if (tid == 0 && g.status) atomicCAS(g.status, 0u, (uint32_t)PB_ETIMEOUT);
-      if (tid == 0) tc::mbar_wait(&mbar[(c - 1) % S], (uint32_t)((c - 1) / S) & 1u);  // drain (bounded)
-      break;
+    if (copier) {
+      asm volatile("cp.async.wait_group %0;" ::"n"(A - 1) : "memory");
+      tc::fence_proxy_async_smem();
     }
-    if (tid == 0) {
+    // publishes chunk c, and that the MMAs of chunk c + A - S are done; one
+    // decision for the whole CTA (the loop has barriers)
+    ok = __syncthreads_and(ok) != 0;
+    if (!ok) break;
+    if (copier) {
+      load(c + A);  // into the stage of chunk c + A - S
+    } else if (lane == 0) {
       tc::fence_after_sync();
-      const uint32_t a0 = tc::smem_u32(sm + (uint32_t)(c % S) * stage), b0 = a0 + a_bytes;
+      const uint32_t a0 = tc::smem_u32(sm) + (uint32_t)(c % S) * stage;
+      // descriptors advance by constants (16-byte units): a K-step covers two
+      // 8-wide K columns (LBO apart), four steps a 64-wide half
+      uint64_t ad = tc::smem_desc(a0, tc::kLBO, tc::kSBO);
+      uint64_t bd = tc::smem_desc(a0 + a_bytes, tc::kLBO, tc::kSBO);
+      const int steps = min(kGemmK / 16, (g.K - c * kGemmK + 15) / 16);
+      if (steps == kGemmK / 16) {
 #pragma unroll
-      for (int s = 0; s < kGemmK / 16; ++s) {
-        if (c * kGemmK + 16 * s >= g.K) break;
-        // K-step s covers two 8-wide K columns (LBO apart) of half s / 4
-        const uint32_t ao = (uint32_t)(s >> 2) * TM * 128u + (uint32_t)(s & 3) * 2u * tc::kLBO;
-        const uint32_t bo = (uint32_t)(s >> 2) * BN * 128u + (uint32_t)(s & 3) * 2u * tc::kLBO;
-        const uint64_t ad = tc::smem_desc(a0 + ao, tc::kLBO, tc::kSBO);
-        const uint64_t bd = tc::smem_desc(b0 + bo, tc::kLBO, tc::kSBO);
-        tc::mma_bf16(tbase, ad, bd, idesc, (c > 0) || (s > 0));
+        for (int s = 0; s < kGemmK / 16; ++s)
+          tc::mma_bf16(tbase, ad + (uint32_t)((s >> 2) * TM * 8 + (s & 3) * 16),
+                       bd + (uint32_t)((s >> 2) * BN * 8 + (s & 3) * 16), idesc, (c > 0) || (s > 0));
+      } else {
+#pragma unroll 1
+        for (int s = 0; s < steps; ++s)
+          tc::mma_bf16(tbase, ad + (uint32_t)((s >> 2) * TM * 8 + (s & 3) * 16),
+                       bd + (uint32_t)((s >> 2) * BN * 8 + (s & 3) * 16), idesc, (c > 0) || (s > 0));
       }
       tc::mma_commit(&mbar[c % S]);
+      // before the next barrier: the stage that the copies after it fill
+      const int p = c + 1 + A - S;
+      if (p >= 0) ok = done(p);
     }
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
-  if (ok) {
-    const bool done = tc::mbar_wait(&mbar[(nch - 1) % S], (uint32_t)((nch - 1) / S) & 1u);
-    ok = __syncthreads_and(done) != 0;
-    if (!ok && tid == 0) {
-      if (g.status) atomicCAS(g.status, 0u, (uint32_t)PB_ETIMEOUT);
-      tc::mbar_wait(&mbar[(nch - 1) % S], (uint32_t)((nch - 1) / S) & 1u);
-    }
+  if (ok) ok = done(nch - 1);
+  ok = __syncthreads_and(ok) != 0;
+  if (!ok && tid == kGemmThreads - 32) {
+    if (g.status) atomicCAS(g.status, 0u, (uint32_t)PB_ETIMEOUT);
+    done(nch - 1);  // let MMAs in flight drain (bounded)
   }
   tc::fence_after_sync();
 
-  if (ok) {
+  if (ok && copier) {
     // accumulator rows: TM = 128: TMEM lane = row; TM = 64: row r at lane
     // 32 (r / 16) + r % 16
-    const int row = m0 + (TM == 128 ? warp * 32 + lane : warp * 16 + lane);
+    const int quad = warp & 3;
+    const int row = m0 + (TM == 128 ? quad * 32 + lane : quad * 16 + lane);
     const bool live = row < g.M && (TM == 128 || lane < 16);
-    for (int c0 = 0; c0 < BN; c0 += 16) {
+    for (int c0 = (warp >> 2) * 16; c0 < BN; c0 += 32) {
       float v[16];
-      tc::tmem_ld16(tbase + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
+      tc::tmem_ld16(tbase + ((uint32_t)(quad * 32) << 16) + (uint32_t)c0, v);
       if (!live) continue;
       const int col0 = n0 + c0;
       const bool full = col0 + 16 <= g.N;
       __align__(16) __nv_bfloat16 mk[16];
-      if ((g.flags & kEpiMask) && full && (g.ldm & 7) == 0 && ((uintptr_t)g.mask & 15) == 0) {
+      if ((flags & kEpiMask) && full && (g.ldm & 7) == 0 && ((uintptr_t)g.mask & 15) == 0) {
         const uint4* src = reinterpret_cast<const uint4*>(g.mask + (size_t)row * g.ldm + col0);
         reinterpret_cast<uint4*>(mk)[0] = src[0];
         reinterpret_cast<uint4*>(mk)[1] = src[1];
-      } else if (g.flags & kEpiMask) {
+      } else if (flags & kEpiMask) {
 #pragma unroll
         for (int i = 0; i < 16; ++i)
           mk[i] = col0 + i < g.N ? g.mask[(size_t)row * g.ldm + col0 + i] : __float2bfloat16(0.f);
+      }
+      float bs[16];
+      const bool bias = g.bias != nullptr;
+      if (bias && full && ((uintptr_t)(g.bias + col0) & 15) == 0) {
+#pragma unroll
+        for (int i = 0; i < 16; i += 4) {
+          const float4 x = *reinterpret_cast<const float4*>(g.bias + col0 + i);
+          bs[i] = x.x; bs[i + 1] = x.y; bs[i + 2] = x.z; bs[i + 3] = x.w;
+        }
+      } else if (bias) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) bs[i] = col0 + i < g.N ? g.bias[col0 + i] : 0.f;
       }
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
         const int col = col0 + i;
         if (col >= g.N) continue;
         float x = g.alpha * v[i];
-        if (g.bias) x += g.bias[col];
-        if (g.flags & kEpiRelu) x = fmaxf(x, 0.f);
-        if (g.flags & kEpiMask) x = (__bfloat162float(mk[i]) > 0.f) ? x : 0.f;
+        if (bias) x += bs[i];
+        if (flags & kEpiRelu) x = fmaxf(x, 0.f);
+        if (flags & kEpiMask) x = (__bfloat162float(mk[i]) > 0.f) ? x : 0.f;
         v[i] = x;
       }
-      if (g.flags & kEpiBce) {
+      if (flags & kEpiBce) {
         __align__(16) __nv_bfloat16 gb[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
@@ -230,7 +276,7 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int m0, int n0, uin
         dst[0] = reinterpret_cast<const uint4*>(gb)[0];
         dst[1] = reinterpret_cast<const uint4*>(gb)[1];
       }
-      if (g.flags & kEpiOutBf16) {
+      if (flags & kEpiOutBf16) {
         __align__(16) __nv_bfloat16 o[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) o[i] = __float2bfloat16(v[i]);
@@ -253,14 +299,14 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int m0, int n0, uin
         }
       } else {
         float* d = reinterpret_cast<float*>(g.D) + (size_t)row * g.ldd + col0;
-        if (full && !(g.flags & kEpiAccum) && (g.ldd & 3) == 0 && ((uintptr_t)g.D & 15) == 0) {
+        if (full && !(flags & kEpiAccum) && (g.ldd & 3) == 0 && ((uintptr_t)g.D & 15) == 0) {
 #pragma unroll
           for (int i = 0; i < 16; i += 4)
             *reinterpret_cast<float4*>(d + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
         } else {
 #pragma unroll
           for (int i = 0; i < 16; ++i)
-            if (col0 + i < g.N) d[i] = (g.flags & kEpiAccum) ? d[i] + v[i] : v[i];
+            if (col0 + i < g.N) d[i] = (flags & kEpiAccum) ? d[i] + v[i] : v[i];
         }
       }
     }
@@ -270,12 +316,25 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int m0, int n0, uin
   if (warp == 0) tc::tmem_dealloc(tbase, ncols);
 }
 
-template <int S>
-__global__ void __launch_bounds__(128) gemm_bf16_tn_kernel(GemmArgs g) {
+template <int S, int F>
+__global__ void __launch_bounds__(kGemmThreads) gemm_bf16_tn_kernel(GemmArgs g) {
   extern __shared__ __align__(1024) uint8_t sm[];
   __shared__ uint64_t mbar[S];
   __shared__ uint32_t tmem_base;
-  gemm_tile<S>(g, blockIdx.x * g.tm, blockIdx.y * g.bn, sm, mbar, &tmem_base);
+  gemm_tile<S, F>(g, blockIdx.x * g.tm, blockIdx.y * g.bn, sm, mbar, &tmem_base);
+}
+
+// The kernel for a tile and flags: four stages where they fit (the network's
+// own layers, by their flags), else two.
+typedef void (*GemmKernel)(GemmArgs);
+inline GemmKernel gemm_kernel(const GemmArgs& g) {
+  if (gemm_stages(g.tm, g.bn) != 4) return gemm_bf16_tn_kernel<2, -1>;
+  switch (g.flags) {
+    case kEpiRelu | kEpiOutBf16: return gemm_bf16_tn_kernel<4, kEpiRelu | kEpiOutBf16>;
+    case kEpiMask | kEpiOutBf16: return gemm_bf16_tn_kernel<4, kEpiMask | kEpiOutBf16>;
+    case kEpiBce: return gemm_bf16_tn_kernel<4, kEpiBce>;
+    default: return gemm_bf16_tn_kernel<4, -1>;
+  }
 }
 
 // One-time set-up outside any stream capture (shared-memory opt-in).
@@ -283,8 +342,12 @@ cudaError_t mlp_fused_prepare();
 cudaError_t grads_prepare();
 cudaError_t mlp_prepare() {
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t e = cudaFuncSetAttribute(gemm_bf16_tn_kernel<2>, a, (int)kGemmSmemMax);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_bf16_tn_kernel<4>, a, (int)kGemmSmemMax);
+  cudaError_t e = cudaSuccess;
+  for (GemmKernel k : {(GemmKernel)gemm_bf16_tn_kernel<2, -1>, (GemmKernel)gemm_bf16_tn_kernel<4, -1>,
+                       (GemmKernel)gemm_bf16_tn_kernel<4, kEpiRelu | kEpiOutBf16>,
+                       (GemmKernel)gemm_bf16_tn_kernel<4, kEpiMask | kEpiOutBf16>,
+                       (GemmKernel)gemm_bf16_tn_kernel<4, kEpiBce>})
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, a, (int)kGemmSmemMax);
   if (e == cudaSuccess) e = grads_prepare();
   return e == cudaSuccess ? mlp_fused_prepare() : e;
 }
@@ -292,10 +355,8 @@ cudaError_t mlp_prepare() {
 cudaError_t launch_gemm_bf16(GemmArgs g, cudaStream_t st) {
   gemm_tiles(g);
   dim3 grid((g.M + g.tm - 1) / g.tm, (g.N + g.bn - 1) / g.bn);
-  const int S = gemm_stages(g.tm, g.bn);
-  const size_t smem = (size_t)S * gemm_stage_bytes(g.tm, g.bn);
-  if (S == 4) gemm_bf16_tn_kernel<4><<<grid, 128, smem, st>>>(g);
-  else gemm_bf16_tn_kernel<2><<<grid, 128, smem, st>>>(g);
+  const size_t smem = (size_t)gemm_stages(g.tm, g.bn) * gemm_stage_bytes(g.tm, g.bn);
+  gemm_kernel(g)<<<grid, kGemmThreads, smem, st>>>(g);
   return cudaGetLastError();
 }
 
@@ -462,7 +523,7 @@ struct GradArgs {
   int H, B, n, npad;
 };
 constexpr int kGradStages = 4;
-constexpr int kGradTm = 64, kGradBn = 32;  // 24 KB a stage
+constexpr int kGradTm = 64, kGradBn = 16;  // 20 KB a stage
 
 // out[j] = sum_b M[j][b] (bf16 rows, fp32 sums), one warp per row.
 __device__ __forceinline__ void rowsum_bf16(const __nv_bfloat16* __restrict__ row, int C, int lane,
@@ -474,7 +535,7 @@ __device__ __forceinline__ void rowsum_bf16(const __nv_bfloat16* __restrict__ ro
   if (lane == 0) *out = s;
 }
 
-__global__ void __launch_bounds__(128) grads_kernel(GradArgs a) {
+__global__ void __launch_bounds__(kGemmThreads) grads_kernel(GradArgs a) {
   extern __shared__ __align__(1024) uint8_t sm[];
   __shared__ uint64_t mbar[kGradStages];
   __shared__ uint32_t tmem_base;
@@ -484,15 +545,17 @@ __global__ void __launch_bounds__(128) grads_kernel(GradArgs a) {
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     if (b < a.tiles[k]) {
-      gemm_tile<kGradStages>(a.w[k], (b % a.mt[k]) * kGradTm, (b / a.mt[k]) * a.w[k].bn, sm, mbar,
-                             &tmem_base);
+      gemm_tile<kGradStages, 0, kGradTm, kGradBn>(a.w[k], (b % a.mt[k]) * kGradTm,
+                                                  (b / a.mt[k]) * kGradBn, sm, mbar, &tmem_base);
       return;
     }
     b -= a.tiles[k];
   }
-  const int rs = (a.H + 3) / 4;  // bias rows, four warps a CTA
+  constexpr int kRows = 8;
+  if (tid >= 256) return;  // (the ninth warp: MMAs only)
+  const int rs = (a.H + kRows - 1) / kRows;  // bias rows, one warp each
   if (b < 2 * rs) {
-    const int row = (b < rs ? b : b - rs) * 4 + (tid >> 5);
+    const int row = (b < rs ? b : b - rs) * kRows + (tid >> 5);
     if (row < a.H)
       rowsum_bf16((b < rs ? a.dZ2t : a.dZ1t) + (size_t)row * a.B, a.B, tid & 31,
                   (b < rs ? a.db2 : a.db1) + row);
@@ -500,20 +563,16 @@ __global__ void __launch_bounds__(128) grads_kernel(GradArgs a) {
   }
   // 256 strided partial sums and a tree: db3[c] (fp32 gradients), or the loss
   const int c = b - 2 * rs;
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int p = tid + 128 * h;
-    float acc = 0.f;
-    if (c < a.n) {
+  float acc = 0.f;
+  if (c < a.n) {
 #pragma unroll 4
-      for (int r = p; r < a.B; r += 256)
-        acc += bce_grad(a.logits[(size_t)r * a.npad + c], a.target[(size_t)r * a.n + c], a.B);
-    } else {
+    for (int r = tid; r < a.B; r += 256)
+      acc += bce_grad(a.logits[(size_t)r * a.npad + c], a.target[(size_t)r * a.n + c], a.B);
+  } else {
 #pragma unroll 8
-      for (int i = p; i < a.B * a.n; i += 256) acc += a.terms[i];
-    }
-    part[p] = acc;
+    for (int i = tid; i < a.B * a.n; i += 256) acc += a.terms[i];
   }
+  part[tid] = acc;
   __syncthreads();
   for (int s = 128; s > 0; s >>= 1) {
     if (tid < s) part[tid] += part[tid + s];
@@ -687,7 +746,7 @@ cudaError_t mlp_bwd(pb_mlp* p, int rows) {
   for (int k = 0; k < 3; ++k) {
     pb::GemmArgs& g = a.w[k];
     g.tm = pb::kGradTm;
-    g.bn = std::min(pb::kGradBn, (g.N + 15) / 16 * 16);
+    g.bn = pb::kGradBn;
     a.mt[k] = (g.M + g.tm - 1) / g.tm;
     a.tiles[k] = a.mt[k] * ((g.N + g.bn - 1) / g.bn);
     total += a.tiles[k];
@@ -705,8 +764,8 @@ cudaError_t mlp_bwd(pb_mlp* p, int rows) {
   a.B = B;
   a.n = p->n;
   a.npad = p->npad;
-  total += 2 * ((H + 3) / 4) + p->n + 1;
-  pb::grads_kernel<<<total, 128, pb::kGradStages * pb::gemm_stage_bytes(pb::kGradTm, pb::kGradBn),
+  total += 2 * ((H + 7) / 8) + p->n + 1;
+  pb::grads_kernel<<<total, pb::kGemmThreads, pb::kGradStages * pb::gemm_stage_bytes(pb::kGradTm, pb::kGradBn),
                      p->st>>>(a);
   return cudaGetLastError();
 }
