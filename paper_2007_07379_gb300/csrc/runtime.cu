@@ -36,6 +36,11 @@ cudaError_t launch_elim(const RunModelDev* d_rm, int n_models, uint32_t total_gr
                         const uint32_t* const* d_init_tabs, uint32_t n_sweeps, size_t smem_bytes,
                         WsHeader* hdr, cudaStream_t st, bool wgt, int warps);
 size_t elim_smem_bytes(int n, int d, int zwords, int warps);
+size_t elim_plain_smem_bytes(int n, int d, uint32_t hist_bins, int warps);
+cudaError_t launch_elim_plain(const RunModelDev* d_rm, int n_models, uint32_t total_groups,
+                              const uint32_t* const* d_init_tabs, uint32_t n_sweeps,
+                              size_t smem_bytes, int warps, WsHeader* hdr, cudaStream_t st);
+cudaError_t elim_plain_prepare();
 cudaError_t launch_amplitudes(const RunModelDev* d_rm, int model, uint32_t bins, int l2,
                               cudaStream_t st);
 cudaError_t launch_philox_fill(const uint32_t* ctr, uint32_t k0, uint32_t k1, uint32_t count,
@@ -919,7 +924,9 @@ struct pb_run {
   int nc = 2;              // colour steps per sweep (largest over the models)
   bool elim = false;       // exact-sampler run: i.i.d. paths instead of sweeps
   size_t elim_smem = 0;
-  int elim_warps = 8;      // exact samplers: warps per CTA (8, 16 or 32)
+  int elim_warps = 8;      // exact samplers: warps per CTA
+  bool elim_plain = false; // exact-sampler run of plain models, no clamped output
+  std::vector<char> elim_hist;  // elim_plain: models that count in shared memory
   std::vector<std::vector<uint32_t>> clamp_keep;
   int grid = 0;
   uint64_t sweeps_done = 0;
@@ -953,6 +960,10 @@ __global__ void periods_init_kernel(WsHeader* hdr, uint32_t periods) { hdr->peri
 
 // The launches of n sweeps of every model (no moves), in stream order.
 cudaError_t enqueue_sweeps(pb_run* r, uint32_t n_sweeps, cudaStream_t st) {
+  if (r->elim_plain)
+    return launch_elim_plain(r->d_rm(), r->nm, r->total_groups,
+                             reinterpret_cast<const uint32_t* const*>(r->ws + r->L.init_ptrs),
+                             n_sweeps, r->elim_smem, r->elim_warps, r->hdr(), st);
   if (r->elim)
     return launch_elim(r->d_rm(), r->nm, r->total_groups,
                        reinterpret_cast<const uint32_t* const*>(r->ws + r->L.init_ptrs), n_sweeps,
@@ -1064,6 +1075,7 @@ void apply_shape(pb_run* r, int cons, int prod, int blocks_per_sm) {
   r->threads = cons + prod + 32;
   std::vector<char> use;
   r->smem = plan_smem(r, r->units, &use);
+  if (r->elim_plain) use = r->elim_hist;  // (their launches have a shape of their own)
   for (int i = 0; i < r->nm; ++i) r->rm[i].hist_smem = use[i] ? 1u : 0u;
   r->persistent = r->nm > 1;
   if (const char* e = std::getenv("PB_PERSISTENT")) r->persistent = std::atoi(e) != 0;
@@ -1304,22 +1316,46 @@ PB_API int pb_run_create(pb_model* const* models, const pb_run_cfg* cfgs, int n_
     x.ws = ws + r->L.ms[i].mh;
   }
   // Exact samplers: warps per CTA.  Samples are independent, so a CTA with
-  // more warps hides more latency; 32 while the groups leave SMs free, 16 up
-  // to two groups per SM, else 8 (several CTAs per SM do the same), and
-  // fewer when the per-warp images do not fit.
+  // more warps hides more latency: as many as fit while the groups leave SMs
+  // free, fewer when several CTAs share one.
   if (r->elim) {
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int ew = r->total_groups <= (uint32_t)sms ? 32 : (r->total_groups <= 2u * (uint32_t)sms ? 16 : 8);
-    auto smem_for = [&](int w) {
-      size_t b = 0;
-      for (auto& m : r->models) b = std::max(b, elim_smem_bytes(m->n, m->d, (m->h + 3) & ~3, w));
-      return b;
-    };
-    while (ew > 8 && smem_for(ew) > kSweepSmemMax) ew /= 2;
-    r->elim_warps = ew;
-    r->elim_smem = smem_for(ew);
+    r->elim_plain = !r->wgt;
+    for (auto& c : r->cfgs) r->elim_plain = r->elim_plain && c.sampler == PB_ELIM;
+    if (r->elim_plain) {
+      // histograms in shared memory by the rule of the sweeps (4096 bins, 1024
+      // in a batch) where 8 warps' images still fit beside them
+      const size_t cap_bins = n_models == 1 ? 4096u : 1024u;
+      auto bytes = [&](int i, int w) {
+        return elim_plain_smem_bytes(r->models[i]->n, r->models[i]->d,
+                                     r->elim_hist[i] ? r->L.ms[i].bins : 0, w);
+      };
+      r->elim_hist.assign(n_models, 1);
+      for (int i = 0; i < n_models; ++i)
+        r->elim_hist[i] = r->L.ms[i].bins <= cap_bins && bytes(i, 8) <= kSweepSmemMax;
+      auto smem_for = [&](int w) {
+        size_t b = 0;
+        for (int i = 0; i < n_models; ++i) b = std::max(b, bytes(i, w));
+        return b;
+      };
+      int ew = r->total_groups <= (uint32_t)sms ? 16 : 8;
+      while (ew > 1 && smem_for(ew) > kSweepSmemMax) --ew;
+      r->elim_warps = ew;
+      r->elim_smem = smem_for(ew);
+    } else {
+      // 32 while the groups leave SMs free, 16 up to two groups per SM, else 8
+      int ew = r->total_groups <= (uint32_t)sms ? 32 : (r->total_groups <= 2u * (uint32_t)sms ? 16 : 8);
+      auto smem_for = [&](int w) {
+        size_t b = 0;
+        for (auto& m : r->models) b = std::max(b, elim_smem_bytes(m->n, m->d, (m->h + 3) & ~3, w));
+        return b;
+      };
+      while (ew > 8 && smem_for(ew) > kSweepSmemMax) ew /= 2;
+      r->elim_warps = ew;
+      r->elim_smem = smem_for(ew);
+    }
   }
   // Work list for the persistent launch: longest first (LPT order).
   std::stable_sort(cost.begin(), cost.end(),
@@ -1327,7 +1363,9 @@ PB_API int pb_run_create(pb_model* const* models, const pb_run_cfg* cfgs, int n_
                      return a.first > b.first;
                    });
   for (auto& c : cost) work.push_back(c.second);
-  if (sweep_prepare() != cudaSuccess || sweep_plain_prepare() != cudaSuccess) return PB_ECUDA;
+  if (sweep_prepare() != cudaSuccess || sweep_plain_prepare() != cudaSuccess ||
+      elim_plain_prepare() != cudaSuccess)
+    return PB_ECUDA;
   choose_shape(r.get());
   if (r->smem > kSweepSmemMax || r->elim_smem > kSweepSmemMax) return PB_ERANGE;
   if ((e = cudaMemcpyAsync(ws + r->L.rm, r->rm.data(), sizeof(RunModelDev) * n_models,

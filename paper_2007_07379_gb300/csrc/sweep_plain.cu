@@ -46,26 +46,6 @@ struct PlainShape {
   int cons, work, units;  // consumer threads, worker warps, units of a period (plain_period)
 };
 
-__device__ __forceinline__ uint32_t lds(uint32_t a) {
-  uint32_t x;
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(x) : "r"(a));
-  return x;
-}
-__device__ __forceinline__ uint2 lds2(uint32_t a) {
-  uint2 x;
-  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(x.x), "=r"(x.y) : "r"(a));
-  return x;
-}
-__device__ __forceinline__ uint4 lds4(uint32_t a) {
-  uint4 x;
-  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w) : "r"(a));
-  return x;
-}
-__device__ __forceinline__ void sts(uint32_t a, uint32_t v) {
-  asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-}
-
 // Four planes (Philox output grp) of [u < t], most significant first.
 __device__ __forceinline__ void compare_planes(uint32_t& lt, uint32_t& eq, uint32_t t, uint4 r,
                                                uint32_t grp) {
@@ -151,28 +131,6 @@ __device__ __forceinline__ uint32_t redraw(uint32_t r0, uint32_t r1, uint32_t r2
   const uint32_t sel = ~(r0 ^ r1) & (~(r1 ^ r2) | M2);
   return neg ^ ((sel & ab.x) | (~sel & ab.y));
 }
-
-// 32 x 32 bit transpose with the lane's masks held in registers: a step is
-// one shuffle, one rotation and one select.
-struct Transpose {
-  uint32_t m[5];
-  __device__ explicit Transpose(int lane) {
-    const uint32_t masks[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
-#pragma unroll
-    for (int k = 0; k < 5; ++k) m[k] = (lane & (16 >> k)) ? ~masks[k] : masks[k];
-  }
-  // lane r holds row r; returns column `lane` (bit r = bit `lane` of row r)
-  __device__ uint32_t operator()(uint32_t x, int lane) const {
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      const int j = 16 >> k;
-      const uint32_t y = __shfl_xor_sync(0xffffffffu, x, j);
-      const uint32_t r = __funnelshift_l(y, y, (lane & j) ? 32 - j : j);
-      x = (x & m[k]) | (r & ~m[k]);
-    }
-    return x;
-  }
-};
 
 // A launch is one kernel: the CTA that is the last to have read the sweep
 // index (counted in ctas_done) advances it for the next launch.
