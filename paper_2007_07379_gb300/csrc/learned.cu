@@ -214,7 +214,7 @@ __global__ void sample_kernel(const float* __restrict__ logits, int npad, int n,
 // words meet in shared memory, and warp w transposes layers k + w, k + w +
 // 32, ...  The last CTA counts the move.
 constexpr int kMaxLayers = 64;
-__global__ void __launch_bounds__(1024) accept_slice_kernel(
+__global__ void __launch_bounds__(1024, 2) accept_slice_kernel(
     const uint32_t* __restrict__ P, const uint32_t* __restrict__ Pn,
     const LayerTab* __restrict__ tab, uint32_t beta, uint32_t nmask, int n, int d, float J,
     const float* __restrict__ lq, const float* __restrict__ lqf, uint32_t chains, uint32_t k0,
