@@ -124,6 +124,16 @@ __device__ __forceinline__ void philox_pair(const PhiloxPair& P, uint32_t sw, ui
   rb = o[1];
 }
 
+// A value the compiler keeps in a register: addresses that depend on the
+// model's sizes are otherwise recomputed from them at every use, on the
+// uniform datapath, which takes issue slots like any other instruction (a
+// quarter of the kernel's).
+__device__ __forceinline__ uint32_t keep(uint32_t x) {
+  uint32_t y;
+  asm volatile("mov.u32 %0, %1;" : "=r"(y) : "r"(x));
+  return y;
+}
+
 // New word of a p-bit from its links' demands and its two comparison words.
 __device__ __forceinline__ uint32_t redraw(uint32_t r0, uint32_t r1, uint32_t r2, uint32_t M2,
                                            uint2 ab) {
@@ -288,8 +298,8 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
     return left < (uint32_t)ps ? left : (uint32_t)ps;
   };
   // The launch's Philox words of outputs j, j + 1.
-  const uint32_t sphx_addr = (uint32_t)__cvta_generic_to_shared(sphx);
-  const uint32_t stm_addr = (uint32_t)__cvta_generic_to_shared(stm);
+  const uint32_t sphx_addr = keep((uint32_t)__cvta_generic_to_shared(sphx));
+  const uint32_t stm_addr = keep((uint32_t)__cvta_generic_to_shared(stm));
   auto load_keys = [&](PhiloxPair& P, uint32_t j) {
     const uint4 ab = lds4(sphx_addr + 8u * j);
     P.a[0] = ab.x; P.a[1] = ab.y; P.b[0] = ab.z; P.b[1] = ab.w;
@@ -311,6 +321,10 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
     Tm[4] = y.x; Tm[5] = y.y; Tm[6] = y.z; Tm[7] = y.w;
   };
 
+  const uint32_t ring_addr = keep((uint32_t)__cvta_generic_to_shared(ring));
+  const uint32_t sent_addr = keep((uint32_t)__cvta_generic_to_shared(sent));
+  const uint32_t sinfo_addr = keep((uint32_t)__cvta_generic_to_shared(sinfo) + 4u * (uint32_t)lane);
+
   // Words of the 64 units from 64 c on of a period whose first sweep is sw0,
   // from planes 0..7 (unit idx: p-bit idx mod npb, in colour order, of the
   // period's sweep idx / npb), two units a lane so that four Philox chains
@@ -318,10 +332,12 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
   // the equal lanes are those that drew eight zeros and no lane is below:
   // the word itself holds the equal lanes.  Otherwise the partial comparison
   // is stored and redone by finish_units.
-  auto start_units = [&](const PhiloxPair& P, uint32_t sw0, uint32_t c, uint2* words,
-                         uint32_t* masks) {
-    const uint32_t idx0 = 64u * c + (uint32_t)lane;
-    const uint32_t X[2] = {sinfo[idx0], sinfo[idx0 + 32u]};
+  // (words: shared address of the period's words; masks: of its masks)
+  auto start_units = [&](const PhiloxPair& P, uint32_t sw0, uint32_t c, uint32_t words,
+                         uint32_t masks) {
+    const uint32_t xa = sinfo_addr + 256u * c;
+    const uint32_t X[2] = {lds(xa), lds(xa + 128u)};
+    words += 512u * c + 8u * (uint32_t)lane;
     uint4 RR[2][2];
 #pragma unroll
     for (int h = 0; h < 2; ++h)
@@ -349,9 +365,10 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
         // (t0 = 2^31 is decided by plane 0)
         open = (linked & eqA) | (odd & eqB);
       }
-      words[idx0 + 32u * h] = ab;
+      asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(words + 256u * h), "r"(ab.x), "r"(ab.y)
+                   : "memory");
       const unsigned mask = __ballot_sync(0xffffffffu, open != 0u);
-      if (lane == 0) masks[2u * c + h] = mask;
+      if (lane == 0) sts(masks + 8u * c + 4u * h, mask);
     }
   };
   // The undecided units among the 256 from 256 f on of period q (ns: its
@@ -428,8 +445,6 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
     }
   };
 
-  const uint32_t ring_addr = (uint32_t)__cvta_generic_to_shared(ring);
-  const uint32_t sent_addr = (uint32_t)__cvta_generic_to_shared(sent);
   int col_lo[NC + 1];
 #pragma unroll
   for (int c = 0; c <= NC; ++c) col_lo[c] = uni(md.col_off[c]);
@@ -439,8 +454,10 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
   // of its samples)
   const uint32_t a_lo = rm.n_alphas ? rm.alpha_sorted[0] : 0u;
   const uint32_t a_hi = rm.n_alphas ? rm.alpha_sorted[rm.n_alphas - 1] : ~0u;
-  const uint32_t svio_addr = (uint32_t)__cvta_generic_to_shared(svio);
-  const uint32_t sph_addr = (uint32_t)__cvta_generic_to_shared(sph);
+  const uint32_t svio_addr = keep((uint32_t)__cvta_generic_to_shared(svio) + 8u * (uint32_t)lane);
+  const uint32_t sph_addr = keep((uint32_t)__cvta_generic_to_shared(sph) + 4u * (uint32_t)lane);
+  const uint32_t last_off = keep(8u * (uint32_t)(d * n));
+  const uint32_t iw4 = keep(4u * (uint32_t)iw);
 
   // Records (Fig. 2 Step 3) of the pair of sweeps sw, sw + 1 whose snapshots
   // start at shared address S (ns: the sweeps that exist).  The lanes take
@@ -456,7 +473,7 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
       v[1] = x.y;
     };
     const uint32_t SS = S | (S << 16);  // offsets are added in pairs (no carry: below 64 KB)
-    uint32_t ea = svio_addr + 8u * (uint32_t)lane;
+    uint32_t ea = svio_addr;
 #pragma unroll 2
     for (int k = 0; k < n_vio; k += 32, ea += 256u) {
       const uint2 e = lds2(ea);
@@ -468,7 +485,7 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
 #pragma unroll
       for (int s = 0; s < 2; ++s) viol[s] |= x[s] ^ y[s] ^ z[s];
     }
-    ea = sph_addr + 4u * (uint32_t)lane;
+    ea = sph_addr;
     auto terms = [&](uint32_t (&x)[2]) {  // the next entries' products
       const uint32_t e = lds(ea) + SS;
       uint32_t y[2];
@@ -533,7 +550,7 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
     uint32_t row[2];
     const bool one = n <= 29;  // one transpose: rows 0..2 the planes, then the layer
     const int q = one ? lane - 3 : lane;
-    ldv(S + 8u * (uint32_t)(d * n + (q >= 0 && q < n ? q : 0)), row);
+    ldv(S + last_off + 8u * (uint32_t)(q >= 0 && q < n ? q : 0), row);
     const bool active = g * 32u + (uint32_t)lane < rm.chains;
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
@@ -595,8 +612,8 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
       const uint32_t ss = sq < n_periods ? (sweeps_of(sq) * (uint32_t)npb + 63u) >> 6 : 0u;
       const uint32_t nf = (fs + 7u) >> 3, nr = rq < n_periods ? (sweeps_of(rq) + 1u) >> 1 : 0u;
       uint32_t* counter = cnt + it % 3u;
-      uint2* words = ring + (sq % 3u) * (uint32_t)punits;
-      uint32_t* masks = smask + (sq & 1u) * (uint32_t)(punits >> 5);
+      const uint32_t words = keep(ring_addr + 8u * (sq % 3u) * (uint32_t)punits);
+      const uint32_t masks = keep((uint32_t)__cvta_generic_to_shared(smask) + 4u * (sq & 1u) * (uint32_t)(punits >> 5));
       PhiloxPair P;
       load_keys(P, 0u);
       if (w == 0u && lane == 0) cnt[(it + 1u) % 3u] = 0u;  // last used in iteration it - 2
@@ -608,7 +625,7 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
           finish_units(fq, k, fs);
         } else if (k < nf + nr) {
           const uint32_t i = (k - nf) << 1, sw = sweep0 + rq * (uint32_t)ps + i;
-          const uint32_t S = w_addr + 4u * (uint32_t)(iw * (1 + (int)(rq & 1u) * psp + (int)i));
+          const uint32_t S = w_addr + iw4 * (1u + (rq & 1u) * (uint32_t)psp + i);
           record(S, sw, sweeps_of(rq) - i);
         } else {
           start_units(P, sweep0 + sq * (uint32_t)ps, k - nf - nr, words, masks);
@@ -641,16 +658,24 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
         uint32_t ab_addr = ring_addr + 8u * ((t % 3u) * (uint32_t)punits + (uint32_t)tid);
         // snapshot of word address a: 2 a + so
         const uint32_t sbase = w_addr + 4u * (uint32_t)(iw * (1 + (int)(t & 1u) * psp)) - 2u * w_addr;
+        // classes in which this warp has p-bits, and its units' words
+        uint32_t act = 0u, abo[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          act |= warp * 32 < col_lo[c + 1] - col_lo[c] ? 1u << c : 0u;
+          abo[c] = keep(8u * (uint32_t)col_lo[c]);
+        }
+        act = keep(act);
+        const uint32_t npb8 = keep(8u * (uint32_t)npb);
         uint2 ab = make_uint2(0u, 0u);
-        if (warp * 32 < col_lo[1]) ab = lds2(ab_addr);
+        if (act & 1u) ab = lds2(ab_addr);
 #pragma unroll 1
         for (uint32_t i = 0; i < cnt_t; ++i) {
-          const uint32_t next = i + 1u < cnt_t ? 8u * (uint32_t)npb : 0u;
-          const uint32_t so = sbase + 4u * ((i & ~1u) * (uint32_t)iw + (i & 1u));
+          const uint32_t next = i + 1u < cnt_t ? npb8 : 0u;
+          const uint32_t so = sbase + (i & ~1u) * iw4 + 4u * (i & 1u);
           auto step = [&](auto cc) {
             constexpr int C = decltype(cc)::value;
-            const int lo = col_lo[C], K = col_lo[C + 1] - lo;
-            if (warp * 32 < K) {
+            if (act & (1u << C)) {
               const uint32_t r0 = lds(la[C][0]) ^ lds(lb[C][0]);
               const uint32_t r1 = lds(la[C][1]) ^ lds(lb[C][1]);
               const uint32_t r2 = lds(la[C][2]) ^ lds(lb[C][2]);
@@ -659,7 +684,7 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
               sts(2u * da[C] + so, v);
               if constexpr (MULTI) {  // further p-bits of a class larger than the consumers
 #pragma unroll 1
-                for (int k = tid + sh.cons; k < K; k += sh.cons) {
+                for (int lo = col_lo[C], K = col_lo[C + 1] - lo, k = tid + sh.cons; k < K; k += sh.cons) {
                   const uint32_t ea = sent_addr + 16u * (uint32_t)(lo + k);
                   const uint4 x = lds4(ea), y = lds4(ea + 16u * (uint32_t)npb);
                   const uint2 ab2 = lds2(ab_addr + 8u * (uint32_t)(lo + k - tid));
@@ -676,8 +701,7 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
             // its class reads another unit's: unused; the allocation has room
             // for the 31 words past the last)
             constexpr int CN = (C + 1) % NC;
-            if (warp * 32 < col_lo[CN + 1] - col_lo[CN])
-              ab = lds2(ab_addr + (CN ? 8u * (uint32_t)col_lo[CN] : next));
+            if (act & (1u << CN)) ab = lds2(ab_addr + (CN ? abo[CN] : next));
             if (cw > 1) bar_sync_first(1u, (uint32_t)sh.cons);
             else __syncwarp();
           };
@@ -685,7 +709,7 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
           step(std::integral_constant<int, 1>{});
           if constexpr (NC > 2) step(std::integral_constant<int, 2>{});
           if constexpr (NC > 3) step(std::integral_constant<int, 3>{});
-          ab_addr += 8u * (uint32_t)npb;
+          ab_addr += npb8;
         }
       }
     }
