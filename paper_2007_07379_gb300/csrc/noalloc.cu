@@ -93,6 +93,8 @@ extern "C" PB_API int pb_gibbs_run_noalloc(const pb_model* m, const pb_run_cfg* 
   const size_t o_rec = off; off = align256(off + npb * sizeof(Rec));
   const size_t o_init = off; off = align256(off + npb * 4);
   const size_t o_state = off; off = align256(off + (size_t)groups * npb * 4);
+  // counters: the run keeps them in the caller's buffers; the scratch has
+  // room for them where those are not aligned for 64-bit atomics
   const size_t o_hist = off; off = align256(off + (size_t)bins * 8 * 8);
   const size_t o_cnt = off; off = align256(off + 2 * 8);
   if (off > kScratchBytes) return PB_ERANGE;
@@ -143,9 +145,12 @@ extern "C" PB_API int pb_gibbs_run_noalloc(const pb_model* m, const pb_run_cfg* 
   r.desc = reinterpret_cast<const Desc*>(base + o_desc);
   r.rec = reinterpret_cast<const Rec*>(base + o_rec);
   r.state = reinterpret_cast<uint32_t*>(base + o_state);
-  r.hist = reinterpret_cast<unsigned long long*>(base + o_hist);
-  r.valid = reinterpret_cast<unsigned long long*>(base + o_cnt);
-  r.samples = reinterpret_cast<unsigned long long*>(base + o_cnt + 8);
+  const bool direct = (((uintptr_t)d_counts | (uintptr_t)d_totals) & 7u) == 0;
+  unsigned long long* counts = direct ? d_counts : reinterpret_cast<unsigned long long*>(base + o_hist);
+  unsigned long long* totals = direct ? d_totals : reinterpret_cast<unsigned long long*>(base + o_cnt);
+  r.hist = counts;
+  r.valid = totals;
+  r.samples = totals + 1;
   r.alpha_sorted = nullptr;
   r.alpha_slot = nullptr;
   r.amp = nullptr;
@@ -163,30 +168,36 @@ extern "C" PB_API int pb_gibbs_run_noalloc(const pb_model* m, const pb_run_cfg* 
   r.hist_smem = hist_smem ? 1u : 0u;
   const uint32_t* init_tab = reinterpret_cast<const uint32_t*>(base + o_init);
 
-  // Every call starts from a cleared header (sweep index 0, status 0) and
-  // cleared counters; the rest of the scratch is overwritten below.
-  cudaError_t e;
-  if ((e = cudaMemsetAsync(base, 0, o_desc, st)) != cudaSuccess ||
-      (e = cudaMemsetAsync(base + o_hist, 0, off - o_hist, st)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(base + o_md, &md, sizeof md, cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(base + o_rm, &r, sizeof r, cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(base + o_iptr, &init_tab, sizeof init_tab, cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(base + o_desc, m->desc.data(), npb * sizeof(Desc), cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(base + o_rec, m->rec.data(), npb * sizeof(Rec), cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(base + o_init, m->init.data(), npb * 4, cudaMemcpyHostToDevice, st)) != cudaSuccess)
+  // Everything below the chain words -- a cleared header (sweep index 0,
+  // status 0), the run entry and the tables -- goes up as one block from the
+  // stack, and the kernels count in the caller's buffers: two clears, one
+  // copy and two kernels (eleven operations, each a few microseconds of a
+  // short call, when every table had its own copy and the counters theirs).
+  constexpr size_t kUpMax = 40 * 1024;  // n <= 16, d <= 64: at most 1024 p-bits
+  alignas(16) char up[kUpMax];
+  if (o_state > kUpMax) return PB_ERANGE;
+  std::memset(up, 0, o_state);
+  std::memcpy(up + o_md, &md, sizeof md);
+  std::memcpy(up + o_rm, &r, sizeof r);
+  std::memcpy(up + o_iptr, &init_tab, sizeof init_tab);
+  std::memcpy(up + o_desc, m->desc.data(), npb * sizeof(Desc));
+  std::memcpy(up + o_rec, m->rec.data(), npb * sizeof(Rec));
+  std::memcpy(up + o_init, m->init.data(), npb * 4);
+  if (cudaMemcpyAsync(base, up, o_init + npb * 4, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+      cudaMemsetAsync(counts, 0, (size_t)bins * 8 * 8, st) != cudaSuccess ||
+      cudaMemsetAsync(totals, 0, 2 * 8, st) != cudaSuccess)
     return PB_ECUDA;
   const RunModelDev* d_rm = reinterpret_cast<const RunModelDev*>(base + o_rm);
   WsHeader* hdr = reinterpret_cast<WsHeader*>(base + o_hdr);
-  if ((e = launch_init(d_rm, 1, groups, reinterpret_cast<const uint32_t* const*>(base + o_iptr),
-                       (size_t)n_words(n, d) * 4, hdr, st)) != cudaSuccess)
+  if (launch_init(d_rm, 1, groups, reinterpret_cast<const uint32_t* const*>(base + o_iptr),
+                  (size_t)n_words(n, d) * 4, hdr, st) != cudaSuccess)
     return PB_ECUDA;
-  if (n_sweeps > 0 &&
-      (e = launch_sweeps_plain(d_rm, 1, groups, n_sweeps, ps.cons, ps.prod, ps.units,
-                               maxcol, nc, smem, hdr, st)) != cudaSuccess)
+  if (n_sweeps > 0 && launch_sweeps_plain(d_rm, 1, groups, n_sweeps, ps.cons, ps.prod, ps.units, maxcol,
+                                          nc, smem, hdr, st) != cudaSuccess)
     return PB_ECUDA;
-  if ((e = cudaMemcpyAsync(d_counts, base + o_hist, (size_t)bins * 8 * 8, cudaMemcpyDeviceToDevice, st)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(d_totals, base + o_cnt, 2 * 8, cudaMemcpyDeviceToDevice, st)) != cudaSuccess)
+  if (!direct && (cudaMemcpyAsync(d_counts, counts, (size_t)bins * 8 * 8, cudaMemcpyDeviceToDevice, st) !=
+                      cudaSuccess ||
+                  cudaMemcpyAsync(d_totals, totals, 2 * 8, cudaMemcpyDeviceToDevice, st) != cudaSuccess))
     return PB_ECUDA;
-  (void)e;
   return PB_OK;
 }
