@@ -20,7 +20,7 @@ cudaError_t launch_init(const RunModelDev* d_rm, int n_models, uint32_t total_gr
                         cudaStream_t st);
 cudaError_t launch_sweeps_plain(const RunModelDev* d_rm, int n_models, uint32_t total_groups,
                                 uint32_t n_sweeps, int cons, int prod, int units, int max_col, int nc,
-                                size_t smem_bytes, WsHeader* hdr, cudaStream_t st);
+                                bool wgt, size_t smem_bytes, WsHeader* hdr, cudaStream_t st);
 cudaError_t sweep_plain_prepare();
 }  // namespace pb
 
@@ -193,7 +193,7 @@ extern "C" PB_API int pb_gibbs_run_noalloc(const pb_model* m, const pb_run_cfg* 
                   (size_t)n_words(n, d) * 4, hdr, st) != cudaSuccess)
     return PB_ECUDA;
   if (n_sweeps > 0 && launch_sweeps_plain(d_rm, 1, groups, n_sweeps, ps.cons, ps.prod, ps.units, maxcol,
-                                          nc, smem, hdr, st) != cudaSuccess)
+                                          nc, false, smem, hdr, st) != cudaSuccess)
     return PB_ECUDA;
   if (!direct && (cudaMemcpyAsync(d_counts, counts, (size_t)bins * 8 * 8, cudaMemcpyDeviceToDevice, st) !=
                       cudaSuccess ||

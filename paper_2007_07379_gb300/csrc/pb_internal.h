@@ -55,7 +55,8 @@ static_assert(sizeof(Rec) == 16, "Rec must be 16 bytes");
 // word where it has no such neighbour): a proposed flip is accepted always
 // (amask bit c) or when the tag-6 uniform is below A[c].  B: the exact
 // sampler's threshold of a coupled output.  flags bit 0: the p-bit has a
-// coupling; bit 1: it is the output of a coupled gate.
+// coupling; bit 1: it is the output of a coupled gate; bits 8-31: its index
+// among the coupled p-bits.
 struct Cpl {
   uint16_t win, wout;
   uint32_t amask;
@@ -123,6 +124,7 @@ struct ModelDev {
   int32_t n_tr;            // two-qubit table gates (TRec entries)
   double log2z;            // log2 of the estimator scale
   int32_t n_rec[4];        // record terms: own links, phases of weight 1, 2, 4
+  int32_t n_cp;            // coupled p-bits (Cpl::flags bit 0)
 };
 
 // Per-model run entry (device), one per model of a run.
@@ -206,6 +208,18 @@ inline size_t plain_smem_bytes(int n, int d, uint32_t hist_bins, int period_unit
          (npad + 96 + units) * 4 + (28 + 144 + 4) * 4 + 2 * (units >> 5) * 4 + (size_t)hist_bins * 32;
 }
 
+// The same for a model of a general-gate run: 40 bytes a bin where it has
+// general gates, and the coupled p-bits' thresholds and entries, the gate
+// phases and two periods of acceptance words.
+inline size_t general_smem_bytes(int n, int d, bool wgt, int n_cp, int n_ug, uint32_t hist_bins,
+                                 int period_units) {
+  const size_t npb = (size_t)n * d, ps = (size_t)plain_period((int)npb, period_units);
+  const size_t words = wgt ? ((size_t)hist_bins * 10 + 3) & ~(size_t)3 : (size_t)hist_bins * 8;
+  return plain_smem_bytes(n, d, 0, period_units) + words * 4 + (size_t)n_cp * 16 +
+         (((size_t)n_cp + 1) & ~(size_t)1) * 8 + npb * 16 + (size_t)n_ug * 16 +
+         (((size_t)n_ug + 3) & ~(size_t)3) * 4 + 2 * ps * ((size_t)n_cp + 1) * 16;
+}
+
 constexpr uint32_t kTagSweep = 0;
 constexpr uint32_t kTagInit = 1;
 constexpr uint32_t kTagMH = 2;
@@ -235,6 +249,7 @@ struct pb_model {
   int n_u = 0, n_coupled = 0;
   double log2z = 0.0;
   std::vector<pb::Cpl> cpl;           // by p (wgt only)
+  int n_cp = 0;                       // coupled p-bits
   std::vector<pb::UPh> uph;           // one per PB_U gate
   int n_ccx = 0;                      // Toffoli gates
   std::vector<pb::GLink> glk;         // by p (Toffoli models only)

@@ -21,10 +21,10 @@ cudaError_t launch_init(const RunModelDev* d_rm, int n_models, uint32_t total_gr
                         cudaStream_t st);
 cudaError_t launch_sweeps(const RunModelDev* d_rm, int n_models, uint32_t total_groups,
                           uint32_t n_sweeps, int cons, int prod, int max_col, int nc,
-                          size_t smem_bytes, WsHeader* hdr, cudaStream_t st, bool ext);
+                          size_t smem_bytes, WsHeader* hdr, cudaStream_t st);
 cudaError_t launch_sweeps_plain(const RunModelDev* d_rm, int n_models, uint32_t total_groups,
                                 uint32_t n_sweeps, int cons, int prod, int units, int max_col, int nc,
-                                size_t smem_bytes, WsHeader* hdr, cudaStream_t st);
+                                bool wgt, size_t smem_bytes, WsHeader* hdr, cudaStream_t st);
 cudaError_t launch_sweeps_plain_persistent(const RunModelDev* d_rm, int n_models,
                                            const uint32_t* d_work, uint32_t n_work,
                                            uint32_t n_sweeps, int cons, int prod, int units,
@@ -433,6 +433,7 @@ PB_API int pb_compile_g(int n, int d, const pb_gate* gates, int n_gates, const d
           else C.A[c] = u32_threshold(std::exp(-dk));
         }
         if (C.flags & 1u) D.mflag |= 8;
+        if (C.flags & 1u) C.flags |= (uint32_t)m->n_cp++ << 8;
         m->cpl.push_back(C);
       }
       const bool tin = table(prod), tout = k < d && table(at(k, q));
@@ -920,7 +921,8 @@ struct pb_run {
   size_t smem = 0;
   bool persistent = false;
   bool wgt = false;        // some model has PB_U gates (the general-gate kernels)
-  bool ext = false;        // some model has Toffoli links or two-qubit tables
+  bool ext = false;        // some model has Toffoli links or two-qubit tables, or the general
+                           // gates' tables do not fit: sweep_kernel instead of the word kernels
   int nc = 2;              // colour steps per sweep (largest over the models)
   bool elim = false;       // exact-sampler run: i.i.d. paths instead of sweeps
   size_t elim_smem = 0;
@@ -968,15 +970,15 @@ cudaError_t enqueue_sweeps(pb_run* r, uint32_t n_sweeps, cudaStream_t st) {
     return launch_elim(r->d_rm(), r->nm, r->total_groups,
                        reinterpret_cast<const uint32_t* const*>(r->ws + r->L.init_ptrs), n_sweeps,
                        r->elim_smem, r->hdr(), st, r->wgt, r->elim_warps);
-  if (r->wgt)
+  if (r->ext)
     return launch_sweeps(r->d_rm(), r->nm, r->total_groups, n_sweeps, r->cons, r->prod, r->max_col,
-                         r->nc, r->smem, r->hdr(), st, r->ext);
+                         r->nc, r->smem, r->hdr(), st);
   if (r->persistent)
     return launch_sweeps_plain_persistent(
         r->d_rm(), r->nm, reinterpret_cast<const uint32_t*>(r->ws + r->L.work), r->total_groups,
         n_sweeps, r->cons, r->prod, r->units, r->max_col, r->nc, r->grid, r->smem, r->hdr(), st);
   return launch_sweeps_plain(r->d_rm(), r->nm, r->total_groups, n_sweeps, r->cons, r->prod, r->units,
-                             r->max_col, r->nc, r->smem, r->hdr(), st);
+                             r->max_col, r->nc, r->wgt, r->smem, r->hdr(), st);
 }
 
 // Graph of n sweeps of a learned run (Fig. 2 Step 1 with the network as the
@@ -1052,7 +1054,8 @@ size_t plan_smem(const pb_run* r, int units, std::vector<char>* use) {
   for (int i = 0; i < r->nm; ++i) {
     const pb_model& m = *r->models[i];
     auto bytes = [&](uint32_t bins) {
-      return r->wgt ? sweep_smem_bytes(m.n, m.d, r->cons, r->max_col, bins)
+      if (r->ext) return sweep_smem_bytes(m.n, m.d, r->cons, r->max_col, bins);
+      return r->wgt ? general_smem_bytes(m.n, m.d, m.wgt, m.n_cp, (int)m.uph.size(), bins, units)
                     : plain_smem_bytes(m.n, m.d, bins, units);
     };
     const uint32_t bins = r->L.ms[i].bins;
@@ -1093,6 +1096,20 @@ void apply_shape(pb_run* r, int cons, int prod, int blocks_per_sm) {
   r->blocks_per_sm = blocks_per_sm;
 }
 
+// General-gate runs count FP64 phase sums (an add returns the old value), which
+// global memory makes slow: the longest period, up to `units`, that keeps as
+// many models' sums in shared memory as the shortest one does.
+int general_units(const pb_run* r, int units) {
+  auto in_smem = [&](int u) {
+    std::vector<char> use;
+    if (plan_smem(r, u, &use) > kSweepSmemMax) return -1;
+    return (int)std::count(use.begin(), use.end(), (char)1);
+  };
+  const int most = in_smem(1);
+  while (units > 1 && in_smem(units) < most) units /= 2;
+  return units;
+}
+
 // Default launch shape.  Plain runs: plain_shape.  General-gate runs:
 // consumers = the largest colour class rounded up to a warp (one p-bit per
 // consumer per class), capped at 224; producers = one per Philox call of a
@@ -1108,7 +1125,10 @@ void choose_shape(pb_run* r) {
   auto up32 = [](int x) { return ((x + 31) / 32) * 32; };
   int cons = std::max(32, std::min(224, up32(maxcol)));
   int prod = std::min(kProducersMax, up32(want));
-  if (!r->wgt) {
+  // general-gate models too large for the word tables (n d near 2048) take
+  // the kernel of the Toffoli and table runs
+  if (r->wgt && !r->ext && plan_smem(r, 1, nullptr) > kSweepSmemMax) r->ext = true;
+  if (!r->ext) {
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1117,6 +1137,7 @@ void choose_shape(pb_run* r) {
     cons = ps.cons;
     prod = ps.prod;
     r->units = ps.units;
+    if (r->wgt) r->units = general_units(r, ps.units);
   }
   if (const char* e = std::getenv("PB_CONS")) {
     int v = std::atoi(e);
@@ -1208,6 +1229,7 @@ PB_API int pb_run_create(pb_model* const* models, const pb_run_cfg* cfgs, int n_
     for (int k = 0; k < 4; ++k) md.max_col = std::max(md.max_col, m.col_off[k + 1] - m.col_off[k]);
     md.wgt = m.wgt ? 1 : 0;
     for (int k = 0; k < 4; ++k) md.n_rec[k] = m.n_rec[k];
+    md.n_cp = m.n_cp;
     md.n_ug = (int32_t)m.uph.size();
     md.n_tr = (int32_t)m.trec.size();
     md.log2z = m.n_tab ? 0.0 : m.log2z;  // tables: unit scale, read L2-normalised

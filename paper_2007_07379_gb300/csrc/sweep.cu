@@ -1,5 +1,6 @@
-// General-gate Gibbs sweeps, initial paths, exact sampler and amplitude kernels
-// (sm_103a); sweep_plain.cu holds the plain (Clifford+T) sweeps.
+// Gibbs sweeps of runs with Toffoli or two-qubit table gates, initial paths, the
+// general and clamped exact samplers and the amplitude kernels (sm_103a);
+// sweep_plain.cu holds the other sweeps.
 //
 // Layout: 32 chains are bit-sliced into one 32-bit word per p-bit (bit c =
 // chain 32 g + c of group g).  A CTA owns one group at a time and keeps the
@@ -281,19 +282,6 @@ __device__ __noinline__ uint32_t table_accept(const uint32_t* W, const TAcc* tp,
   return old ^ (flip & acc);
 }
 
-// Compensated FP64 accumulation of the phase sums: *s += x by an atomic add,
-// whose old value gives the exact rounding error of fl(old + x) (Knuth's
-// two-sum), and that error (plus `carry`, a compensation brought along) is
-// added to the compensation word *c.  The sum is *s + *c; the rounding of the
-// big partial sums no longer accumulates over the samples.
-__device__ __forceinline__ void atomic_add_comp(double* s, double* c, double x, double carry = 0.0) {
-  const double old = atomicAdd(s, x);
-  const double nw = old + x;
-  const double bp = nw - old;
-  const double err = (old - (nw - bp)) + (x - bp) + carry;
-  if (err != 0.0) atomicAdd(c, err);
-}
-
 // CTA roles: `cons` consumer threads redraw the p-bits of the current colour
 // class; `prod` producer threads compute the Philox planes of the next class,
 // compared group by group with each p-bit's two thresholds,
@@ -323,210 +311,6 @@ __host__ __device__ inline size_t group_smem_bytes(int n, int d, int cons, int m
          (size_t)4 * cons * sizeof(ClassEnt) +
          (size_t)2 * ((size_t)kPre * max_col + (size_t)kPreC * cons) * sizeof(uint4);
 }
-
-// Record of one sweep (Fig. 2 Step 3), computed by the recorder warp from a
-// snapshot of the sweep's final state while the stage warps run the next
-// sweep, pipelined over the colour stages: read() gathers, for a range of
-// p-bits, the violation word and the phase (three bit planes, mod 8);
-// reduce() combines the lanes and takes the last layer; bin() adds one count
-// per valid chain to (end state alpha, phase class).
-struct Recorder {
-  uint32_t viol = 0u, f0 = 0u, f1 = 0u, f2 = 0u, lastw = 0u;
-  uint32_t phi = 0u;  // general gates: this lane's chain's phase, 2^-32 turn
-
-  __device__ void clear() { viol = f0 = f1 = f2 = phi = 0u; }
-
-  // Two-qubit tables lo..hi-1: each adds its entry's phase for the lane's
-  // chain, and a zero entry marks the chain's path invalid.
-  __device__ void read_t(const uint32_t* S, const TRec* tr, int lo, int hi, int lane) {
-    bool bad = false;
-#pragma unroll 1
-    for (int i = lo; i < hi; ++i) {
-      const TRec& R = tr[i];
-      const uint32_t idx = ((S[R.wx0] >> lane) & 1u) | (((S[R.wx1] >> lane) & 1u) << 1) |
-                           (((S[R.wy0] >> lane) & 1u) << 2) | (((S[R.wy1] >> lane) & 1u) << 3);
-      phi += R.ph[idx];
-      bad = bad || ((R.zmask >> idx) & 1u);
-    }
-    viol |= __ballot_sync(0xffffffffu, bad);
-  }
-
-  // Phases of general gates lo..hi-1 for the lane's own chain, eight gates
-  // per batch with every load of a batch issued before the first use.
-  __device__ void read_u(const uint32_t* S, const UPh* uph, int lo, int hi, int lane) {
-    int i = lo;
-#pragma unroll 1
-    for (; i + 8 <= hi; i += 8) {
-      uint4 ph[8];
-      uint32_t ww[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        ph[j] = *reinterpret_cast<const uint4*>(uph[i + j].ph);
-        ww[j] = *reinterpret_cast<const uint32_t*>(&uph[i + j].wout);  // wout | win << 16
-      }
-      uint32_t y[8], x[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        y[j] = (S[ww[j] & 0xFFFFu] >> lane) & 1u;
-        x[j] = (S[ww[j] >> 16] >> lane) & 1u;
-      }
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const uint32_t a0 = y[j] ? ph[j].z : ph[j].x, a1 = y[j] ? ph[j].w : ph[j].y;
-        phi += x[j] ? a1 : a0;
-      }
-    }
-#pragma unroll 1
-    for (; i < hi; ++i) {
-      const UPh U = uph[i];
-      const uint32_t y = (S[U.wout] >> lane) & 1u, x = (S[U.win] >> lane) & 1u;
-      const uint32_t a0 = y ? U.ph[2] : U.ph[0], a1 = y ? U.ph[3] : U.ph[1];
-      phi += x ? a1 : a0;
-    }
-  }
-
-  // ANDV: general-gate runs, where a Toffoli target's term is
-  // W[vd] ^ W[va] ^ (W[vb] & W[vc]) (vc = ONES elsewhere).
-  template <bool ANDV = false>
-  __device__ void read(const uint32_t* S, const Rec* srec, int lo, int hi, int lane) {
-#pragma unroll 2
-    for (int i = lo + lane; i < hi; i += 32) {
-      const Rec R = srec[i];
-      if constexpr (ANDV) viol |= S[R.vd] ^ S[R.va] ^ (S[R.vb] & S[R.vc]);
-      else viol |= S[R.vd] ^ S[R.va] ^ S[R.vb];
-      const uint32_t x = S[R.pa] & S[R.pb];
-      add3(f0, f1, f2, (R.w & 1) ? x : 0u, (R.w & 2) ? x : 0u, (R.w & 4) ? x : 0u);
-    }
-  }
-
-  __device__ void reduce(const uint32_t* S, int n, int d, int lane) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      const uint32_t ov = __shfl_xor_sync(0xffffffffu, viol, off);
-      const uint32_t o0 = __shfl_xor_sync(0xffffffffu, f0, off);
-      const uint32_t o1 = __shfl_xor_sync(0xffffffffu, f1, off);
-      const uint32_t o2 = __shfl_xor_sync(0xffffffffu, f2, off);
-      viol |= ov;
-      add3(f0, f1, f2, o0, o1, o2);
-    }
-    lastw = lane < n ? S[d * n + lane] : 0u;
-  }
-
-  // The phasor of this lane's record: the general gates' phases plus the
-  // phase class (2^29 per pi/4), in FP32 (FP64 issues far slower on this
-  // part): the angle rounds to 24 bits (<= pi 2^-24 rad) and sincospif adds
-  // about one ulp, so each term is within 3e-7 of e^{i angle}.
-  __device__ void phasor(uint32_t phase, double& cs, double& sn) const {
-    const uint32_t ang = phi + (phase << 29);
-    float snf, csf;
-    sincospif((float)(int32_t)ang * 0x1p-31f, &snf, &csf);
-    cs = (double)csf;
-    sn = (double)snf;
-  }
-
-  // Few bins (<= 8): all lanes would hit a handful of FP64 counters, so the
-  // warp sums each distinct bin's terms with shuffles and one lane adds them
-  // (whole warp, convergent).
-  __device__ void bin_few(const RunModelDev& rm, uint32_t batch, int lane, uint32_t* shist,
-                          int bin) {
-    const uint32_t phase = ((f0 >> lane) & 1u) | (((f1 >> lane) & 1u) << 1) |
-                           (((f2 >> lane) & 1u) << 2);
-    double cs, sn;
-    phasor(phase, cs, sn);
-    const bool has = bin >= 0;
-    unsigned pending = __ballot_sync(0xffffffffu, has);
-    while (pending) {
-      const int leader = __ffs((int)pending) - 1;
-      const int b = __shfl_sync(0xffffffffu, bin, leader);
-      const bool mine = has && bin == b;
-      const unsigned m = __ballot_sync(0xffffffffu, mine);
-      double r = mine ? cs : 0.0, q = mine ? sn : 0.0;
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        r += __shfl_xor_sync(0xffffffffu, r, off);
-        q += __shfl_xor_sync(0xffffffffu, q, off);
-      }
-      if (lane == leader) {
-        if (shist) {
-          double* sd = reinterpret_cast<double*>(shist) + 4u * (uint32_t)b;
-          atomic_add_comp(&sd[0], &sd[2], r);
-          atomic_add_comp(&sd[1], &sd[3], q);
-          atomicAdd(&shist[8u * rm.bins + (uint32_t)b], (uint32_t)__popc(m));
-        } else {
-          unsigned long long* c = rm.hist + ((size_t)batch * rm.bins + (uint32_t)b) * 8u;
-          double* cd = reinterpret_cast<double*>(c);
-          atomic_add_comp(&cd[0], &cd[3], r);
-          atomic_add_comp(&cd[1], &cd[4], q);
-          atomicAdd(c + 2, (unsigned long long)__popc(m));
-        }
-      }
-      pending &= ~m;
-    }
-  }
-
-  // WGT: models with general gates (rm.cpl set) add e^{i 2 pi phase} in FP64
-  // (re, im, count per bin) instead of one count per phase class.
-  template <bool WGT>
-  __device__ void bin(const RunModelDev& rm, uint32_t g, uint32_t batch, int lane, uint32_t* shist,
-                      unsigned long long& n_valid, unsigned long long& n_samples) {
-    // lane = chain within the group; alpha bit q = bit `lane` of layer-d word q
-    const uint32_t chain = g * 32u + (uint32_t)lane;
-    const bool active = chain < rm.chains;
-    const bool valid = active && !((viol >> lane) & 1u);
-    const uint32_t alpha = warp_transpose32(lastw, lane);
-    const uint32_t phase = ((f0 >> lane) & 1u) | (((f1 >> lane) & 1u) << 1) |
-                           (((f2 >> lane) & 1u) << 2);
-    int bin = -1;
-    if (valid) {
-      const int na = rm.n_alphas;
-      if (na == 0) {
-        bin = (int)alpha;
-      } else {
-        int lo = 0, hi = na - 1;
-        while (lo <= hi) {
-          const int mid = (lo + hi) >> 1;
-          const uint32_t v = rm.alpha_sorted[mid];
-          if (v == alpha) { bin = rm.alpha_slot[mid]; break; }
-          if (v < alpha) lo = mid + 1; else hi = mid - 1;
-        }
-      }
-    }
-    if constexpr (WGT) {
-      if (rm.cpl != nullptr && rm.bins <= 8u) {  // whole warp here: see bin_few
-        bin_few(rm, batch, lane, shist, bin);
-        bin = -1;
-      }
-    }
-    if (bin >= 0) {
-      bool done = false;
-      if constexpr (WGT) {
-        if (rm.cpl != nullptr) {
-          double cs, sn;
-          phasor(phase, cs, sn);
-          if (shist) {
-            double* sd = reinterpret_cast<double*>(shist) + 4u * (uint32_t)bin;
-            atomic_add_comp(&sd[0], &sd[2], cs);
-            atomic_add_comp(&sd[1], &sd[3], sn);
-            atomicAdd(&shist[8u * rm.bins + (uint32_t)bin], 1u);
-          } else {
-            unsigned long long* c = rm.hist + ((size_t)batch * rm.bins + (uint32_t)bin) * 8u;
-            double* cd = reinterpret_cast<double*>(c);
-            atomic_add_comp(&cd[0], &cd[3], cs);
-            atomic_add_comp(&cd[1], &cd[4], sn);
-            atomicAdd(c + 2, 1ull);
-          }
-          done = true;
-        }
-      }
-      if (!done) {
-        if (shist) atomicAdd(&shist[(uint32_t)bin * 8u + phase], 1u);
-        else atomicAdd(&rm.hist[((size_t)batch * rm.bins + (uint32_t)bin) * 8u + phase], 1ull);
-      }
-    }
-    n_valid += __popc(__ballot_sync(0xffffffffu, valid));
-    n_samples += __popc(__ballot_sync(0xffffffffu, active));
-  }
-};
 
 // p-bits lo + first, lo + first + stride, ... < hi of a colour class from
 // their descriptors (a class larger than the consumers; rare).  Output j of
@@ -572,13 +356,12 @@ __device__ __noinline__ void redraw_extra_coupled(uint32_t* W, uint32_t* S, cons
 
 // Runs `n_sweeps` sweeps (absolute indices sweep0...) of one chain group.
 // NC = colour steps per sweep (2..4; the model's classes NC.. are empty).
-// The kernel of runs with general-gate models (coupled p-bits
+// The kernel of runs in which some model has Toffoli links or two-qubit tables
+// (the other general-gate runs take sweep_plain.cu's; coupled p-bits
 // get the Metropolis acceptance, records add FP64 phases); plain models run
-// through it unchanged.  EXT: some model also has Toffoli links or two-qubit
-// tables; without them those paths are compiled out, so the coupled-gate
-// consumers and the recorder keep their shorter code.  12 planes are computed
-// ahead per p-bit, each class's during the step before.
-template <int NC, bool EXT>
+// through it unchanged.  12 planes are computed ahead per p-bit, each class's
+// during the step before.
+template <int NC>
 __device__ void run_group(const RunModelDev& rm_g, uint32_t g, uint32_t sweep0, uint32_t n_sweeps,
                           Shape sh, int max_col_all, uint32_t* smem, WsHeader* hdr) {
   // run and model constants held in registers for the whole launch
@@ -631,7 +414,6 @@ __device__ void run_group(const RunModelDev& rm_g, uint32_t g, uint32_t sweep0, 
     bool ok = D.dst < nw;
 #pragma unroll
     for (int l = 0; l < 3; ++l) ok = ok && D.a[l] < nw && D.b[l] < nw;
-    if (!EXT && (D.mflag & 0x30)) ok = false;  // Toffoli / table p-bit: needs EXT
     if (!ok) {  // never write through a bad index: the entry is skipped
       set_status(hdr, PB_EINVAL);
       D.mflag = 0x80;
@@ -715,8 +497,8 @@ __device__ void run_group(const RunModelDev& rm_g, uint32_t g, uint32_t sweep0, 
       E.dst = 4u * D.dst;
       E.m = (uint32_t)m;
       if (D.mflag & 8) E.m |= 0x100u;     // coupled: Metropolis acceptance
-      if (EXT && (D.mflag & 0x10)) E.m |= 0x200u;  // general links (Toffoli)
-      if (EXT && (D.mflag & 0x20)) E.m |= 0x400u;  // table acceptance
+      if ((D.mflag & 0x10)) E.m |= 0x200u;  // general links (Toffoli)
+      if ((D.mflag & 0x20)) E.m |= 0x400u;  // table acceptance
       E.M0 = m == 0 ? ~0u : 0u;
       E.M1 = m == 1 ? ~0u : 0u;
       E.M2 = m == 2 ? ~0u : 0u;
@@ -793,7 +575,7 @@ __device__ void run_group(const RunModelDev& rm_g, uint32_t g, uint32_t sweep0, 
           wout_w = W[Cp.wout];
         }
         uint32_t v;
-        if (EXT && (E.m & 0x200u))
+        if ((E.m & 0x200u))
           v = glink_heat_bath(W, rm.glk + (E.dst / 4u - (uint32_t)n), rp, thr0, thr1, thr2, thr3,
                               gglob, sweep, pidx, k0, k1);
         else
@@ -804,7 +586,7 @@ __device__ void run_group(const RunModelDev& rm_g, uint32_t g, uint32_t sweep0, 
           v = couple_accept_body(Cp, win_w, wout_w, old_w, v, cur + acc_off + tid * kPreC, gglob,
                                  sweep, p, k0, k1);
         }
-        if (EXT && (E.m & 0x400u)) {  // a second acceptance factor: the tables' energy
+        if ((E.m & 0x400u)) {  // a second acceptance factor: the tables' energy
           const uint32_t p = E.dst / 4u - (uint32_t)n;
           v = table_accept(W, rm.tacc + p, word(E.dst), v, gglob, sweep, p, k0, k1);
         }
@@ -814,8 +596,8 @@ __device__ void run_group(const RunModelDev& rm_g, uint32_t g, uint32_t sweep0, 
       // further p-bits (a class larger than the consumers) from the descriptors
       if (K > sh.cons) {
         redraw_extra_coupled(W, S, sdesc, cur, lo, tid + sh.cons, hi, sh.cons, n, fast, thr0, thr1,
-                             thr2, thr3, gglob, sweep, k0, k1, rm.cpl, EXT ? rm.glk : nullptr,
-                             EXT ? rm.tacc : nullptr);
+                             thr2, thr3, gglob, sweep, k0, k1, rm.cpl, rm.glk,
+                             rm.tacc);
       }
     } else if (producer) {
       // the next step: class C + 1 of this sweep, or class 0 of the next one
@@ -840,9 +622,9 @@ __device__ void run_group(const RunModelDev& rm_g, uint32_t g, uint32_t sweep0, 
           // part C of the records: one share in step 0 (the largest class,
           // the most consumer warps), two in each later step
           constexpr int D = 2 * (NC - 1) - 1, B0 = C == 0 ? 0 : 2 * C - 1, B1 = 2 * C + 1;
-          rec.read<EXT>(Sp, srec, B0 * npb / D, B1 * npb / D, lane);
+          rec.read<true>(Sp, srec, B0 * npb / D, B1 * npb / D, lane);
           if (wgt_m) rec.read_u(Sp, rm.uph, B0 * nug / D, B1 * nug / D, lane);
-          if (EXT && rm.trec) rec.read_t(Sp, rm.trec, B0 * md.n_tr / D, B1 * md.n_tr / D, lane);
+          if (rm.trec) rec.read_t(Sp, rm.trec, B0 * md.n_tr / D, B1 * md.n_tr / D, lane);
         } else {
           rec.reduce(Sp, n, d, lane);
           rec.bin<true>(rm_g, g, batch, lane, shist, n_valid, n_samples);
@@ -867,9 +649,9 @@ __device__ void run_group(const RunModelDev& rm_g, uint32_t g, uint32_t sweep0, 
     if (n_sweeps > 0 && recorded(sweep0 + n_sweeps - 1)) {
       const uint32_t* Sl = smem + iw * (1 + ((n_sweeps - 1u) & 1u));
       rec.clear();
-      rec.read<EXT>(Sl, srec, 0, npb, lane);
+      rec.read<true>(Sl, srec, 0, npb, lane);
       if (wgt_m) rec.read_u(Sl, rm.uph, 0, nug, lane);
-      if (EXT && rm.trec) rec.read_t(Sl, rm.trec, 0, md.n_tr, lane);
+      if (rm.trec) rec.read_t(Sl, rm.trec, 0, md.n_tr, lane);
       rec.reduce(Sl, n, d, lane);
       rec.bin<true>(rm_g, g, batch, lane, shist, n_valid, n_samples);
     }
@@ -906,7 +688,7 @@ __device__ void run_group(const RunModelDev& rm_g, uint32_t g, uint32_t sweep0, 
 }
 
 // One CTA per chain group of every model of the run (flat group index).
-template <int NC, bool EXT>
+template <int NC>
 __global__ void __launch_bounds__(kSweepThreadsWgt) sweep_kernel(const RunModelDev* __restrict__ rm,
                                                      int n_models, uint32_t total_groups,
                                                      uint32_t n_sweeps, Shape sh, int max_col,
@@ -919,7 +701,7 @@ __global__ void __launch_bounds__(kSweepThreadsWgt) sweep_kernel(const RunModelD
   const RunModelDev& r = rm[mi];
   const uint32_t g = flat - r.group_base;
   if (g >= r.groups) return;
-  run_group<NC, EXT>(r, g, sweep0, n_sweeps, sh, max_col, smem, hdr);
+  run_group<NC>(r, g, sweep0, n_sweeps, sh, max_col, smem, hdr);
 }
 
 // ---------------------------------------------------------------------------
@@ -1314,26 +1096,18 @@ cudaError_t launch_init(const RunModelDev* d_rm, int n_models, uint32_t total_gr
 __global__ void advance_kernel(WsHeader* hdr, uint32_t n_sweeps) { hdr->sweep0 += n_sweeps; }
 
 // nc: colour steps per sweep (the largest over the launch's models; 2..4).
-// ext: some model
-// has Toffoli links or two-qubit tables (EXT).
 cudaError_t launch_sweeps(const RunModelDev* d_rm, int n_models, uint32_t total_groups,
                           uint32_t n_sweeps, int cons, int prod, int max_col, int nc,
-                          size_t smem_bytes, WsHeader* hdr, cudaStream_t st, bool ext) {
+                          size_t smem_bytes, WsHeader* hdr, cudaStream_t st) {
   const int threads = cons + prod + 32;
   const Shape sh{cons, prod};
   auto go = [&](auto kern) {
     kern<<<total_groups, threads, smem_bytes, st>>>(d_rm, n_models, total_groups, n_sweeps, sh,
                                                     max_col, hdr);
   };
-  if (ext) {
-    if (nc <= 2) go(sweep_kernel<2, true>);
-    else if (nc == 3) go(sweep_kernel<3, true>);
-    else go(sweep_kernel<4, true>);
-  } else {
-    if (nc <= 2) go(sweep_kernel<2, false>);
-    else if (nc == 3) go(sweep_kernel<3, false>);
-    else go(sweep_kernel<4, false>);
-  }
+  if (nc <= 2) go(sweep_kernel<2>);
+  else if (nc == 3) go(sweep_kernel<3>);
+  else go(sweep_kernel<4>);
   advance_kernel<<<1, 1, 0, st>>>(hdr, n_sweeps);
   return cudaGetLastError();
 }
@@ -1393,12 +1167,9 @@ cudaError_t sweep_prepare() {
   const int big = (int)kSweepSmemMax;
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(sweep_kernel<2, false>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_kernel<3, false>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_kernel<4, false>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_kernel<2, true>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_kernel<3, true>, a, big)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(sweep_kernel<4, true>, a, big)) != cudaSuccess)
+  if ((e = cudaFuncSetAttribute(sweep_kernel<2>, a, big)) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(sweep_kernel<3>, a, big)) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(sweep_kernel<4>, a, big)) != cudaSuccess)
     return e;
   if ((e = cudaFuncSetAttribute(elim_kernel<false, 8>, a, big)) != cudaSuccess ||
       (e = cudaFuncSetAttribute(elim_kernel<false, 16>, a, big)) != cudaSuccess ||

@@ -113,4 +113,221 @@ struct Transpose {
   }
 };
 
+// Compensated FP64 accumulation of the phase sums: *s += x by an atomic add,
+// whose old value gives the exact rounding error of fl(old + x) (Knuth's
+// two-sum), and that error (plus `carry`, a compensation brought along) is
+// added to the compensation word *c.  The sum is *s + *c; the rounding of the
+// big partial sums no longer accumulates over the samples.
+__device__ __forceinline__ void atomic_add_comp(double* s, double* c, double x, double carry = 0.0) {
+  const double old = atomicAdd(s, x);
+  const double nw = old + x;
+  const double bp = nw - old;
+  const double err = (old - (nw - bp)) + (x - bp) + carry;
+  if (err != 0.0) atomicAdd(c, err);
+}
+
+// Record of one sweep (Fig. 2 Step 3), computed by the recorder warp from a
+// snapshot of the sweep's final state while the stage warps run the next
+// sweep, pipelined over the colour stages: read() gathers, for a range of
+// p-bits, the violation word and the phase (three bit planes, mod 8);
+// reduce() combines the lanes and takes the last layer; bin() adds one count
+// per valid chain to (end state alpha, phase class).
+struct Recorder {
+  uint32_t viol = 0u, f0 = 0u, f1 = 0u, f2 = 0u, lastw = 0u;
+  uint32_t phi = 0u;  // general gates: this lane's chain's phase, 2^-32 turn
+
+  __device__ void clear() { viol = f0 = f1 = f2 = phi = 0u; }
+
+  // Two-qubit tables lo..hi-1: each adds its entry's phase for the lane's
+  // chain, and a zero entry marks the chain's path invalid.
+  __device__ void read_t(const uint32_t* S, const TRec* tr, int lo, int hi, int lane) {
+    bool bad = false;
+#pragma unroll 1
+    for (int i = lo; i < hi; ++i) {
+      const TRec& R = tr[i];
+      const uint32_t idx = ((S[R.wx0] >> lane) & 1u) | (((S[R.wx1] >> lane) & 1u) << 1) |
+                           (((S[R.wy0] >> lane) & 1u) << 2) | (((S[R.wy1] >> lane) & 1u) << 3);
+      phi += R.ph[idx];
+      bad = bad || ((R.zmask >> idx) & 1u);
+    }
+    viol |= __ballot_sync(0xffffffffu, bad);
+  }
+
+  // Phases of general gates lo..hi-1 for the lane's own chain, eight gates
+  // per batch with every load of a batch issued before the first use.
+  __device__ void read_u(const uint32_t* S, const UPh* uph, int lo, int hi, int lane) {
+    int i = lo;
+#pragma unroll 1
+    for (; i + 8 <= hi; i += 8) {
+      uint4 ph[8];
+      uint32_t ww[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        ph[j] = *reinterpret_cast<const uint4*>(uph[i + j].ph);
+        ww[j] = *reinterpret_cast<const uint32_t*>(&uph[i + j].wout);  // wout | win << 16
+      }
+      uint32_t y[8], x[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        y[j] = (S[ww[j] & 0xFFFFu] >> lane) & 1u;
+        x[j] = (S[ww[j] >> 16] >> lane) & 1u;
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const uint32_t a0 = y[j] ? ph[j].z : ph[j].x, a1 = y[j] ? ph[j].w : ph[j].y;
+        phi += x[j] ? a1 : a0;
+      }
+    }
+#pragma unroll 1
+    for (; i < hi; ++i) {
+      const UPh U = uph[i];
+      const uint32_t y = (S[U.wout] >> lane) & 1u, x = (S[U.win] >> lane) & 1u;
+      const uint32_t a0 = y ? U.ph[2] : U.ph[0], a1 = y ? U.ph[3] : U.ph[1];
+      phi += x ? a1 : a0;
+    }
+  }
+
+  // ANDV: general-gate runs, where a Toffoli target's term is
+  // W[vd] ^ W[va] ^ (W[vb] & W[vc]) (vc = ONES elsewhere).
+  template <bool ANDV = false>
+  __device__ void read(const uint32_t* S, const Rec* srec, int lo, int hi, int lane) {
+#pragma unroll 2
+    for (int i = lo + lane; i < hi; i += 32) {
+      const Rec R = srec[i];
+      if constexpr (ANDV) viol |= S[R.vd] ^ S[R.va] ^ (S[R.vb] & S[R.vc]);
+      else viol |= S[R.vd] ^ S[R.va] ^ S[R.vb];
+      const uint32_t x = S[R.pa] & S[R.pb];
+      add3(f0, f1, f2, (R.w & 1) ? x : 0u, (R.w & 2) ? x : 0u, (R.w & 4) ? x : 0u);
+    }
+  }
+
+  __device__ void reduce(const uint32_t* S, int n, int d, int lane) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      const uint32_t ov = __shfl_xor_sync(0xffffffffu, viol, off);
+      const uint32_t o0 = __shfl_xor_sync(0xffffffffu, f0, off);
+      const uint32_t o1 = __shfl_xor_sync(0xffffffffu, f1, off);
+      const uint32_t o2 = __shfl_xor_sync(0xffffffffu, f2, off);
+      viol |= ov;
+      add3(f0, f1, f2, o0, o1, o2);
+    }
+    lastw = lane < n ? S[d * n + lane] : 0u;
+  }
+
+  // The phasor of this lane's record: the general gates' phases plus the
+  // phase class (2^29 per pi/4), in FP32 (FP64 issues far slower on this
+  // part): the angle rounds to 24 bits (<= pi 2^-24 rad) and sincospif adds
+  // about one ulp, so each term is within 3e-7 of e^{i angle}.
+  __device__ void phasor(uint32_t phase, double& cs, double& sn) const {
+    const uint32_t ang = phi + (phase << 29);
+    float snf, csf;
+    sincospif((float)(int32_t)ang * 0x1p-31f, &snf, &csf);
+    cs = (double)csf;
+    sn = (double)snf;
+  }
+
+  // Few bins (<= 8): all lanes would hit a handful of FP64 counters, so the
+  // warp sums each distinct bin's terms with shuffles and one lane adds them
+  // (whole warp, convergent).
+  __device__ void bin_few(const RunModelDev& rm, uint32_t batch, int lane, uint32_t* shist,
+                          int bin) {
+    const uint32_t phase = ((f0 >> lane) & 1u) | (((f1 >> lane) & 1u) << 1) |
+                           (((f2 >> lane) & 1u) << 2);
+    double cs, sn;
+    phasor(phase, cs, sn);
+    const bool has = bin >= 0;
+    unsigned pending = __ballot_sync(0xffffffffu, has);
+    while (pending) {
+      const int leader = __ffs((int)pending) - 1;
+      const int b = __shfl_sync(0xffffffffu, bin, leader);
+      const bool mine = has && bin == b;
+      const unsigned m = __ballot_sync(0xffffffffu, mine);
+      double r = mine ? cs : 0.0, q = mine ? sn : 0.0;
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) {
+        r += __shfl_xor_sync(0xffffffffu, r, off);
+        q += __shfl_xor_sync(0xffffffffu, q, off);
+      }
+      if (lane == leader) {
+        if (shist) {
+          double* sd = reinterpret_cast<double*>(shist) + 4u * (uint32_t)b;
+          atomic_add_comp(&sd[0], &sd[2], r);
+          atomic_add_comp(&sd[1], &sd[3], q);
+          atomicAdd(&shist[8u * rm.bins + (uint32_t)b], (uint32_t)__popc(m));
+        } else {
+          unsigned long long* c = rm.hist + ((size_t)batch * rm.bins + (uint32_t)b) * 8u;
+          double* cd = reinterpret_cast<double*>(c);
+          atomic_add_comp(&cd[0], &cd[3], r);
+          atomic_add_comp(&cd[1], &cd[4], q);
+          atomicAdd(c + 2, (unsigned long long)__popc(m));
+        }
+      }
+      pending &= ~m;
+    }
+  }
+
+  // WGT: models with general gates (rm.cpl set) add e^{i 2 pi phase} in FP64
+  // (re, im, count per bin) instead of one count per phase class.
+  template <bool WGT>
+  __device__ void bin(const RunModelDev& rm, uint32_t g, uint32_t batch, int lane, uint32_t* shist,
+                      unsigned long long& n_valid, unsigned long long& n_samples) {
+    // lane = chain within the group; alpha bit q = bit `lane` of layer-d word q
+    const uint32_t chain = g * 32u + (uint32_t)lane;
+    const bool active = chain < rm.chains;
+    const bool valid = active && !((viol >> lane) & 1u);
+    const uint32_t alpha = warp_transpose32(lastw, lane);
+    const uint32_t phase = ((f0 >> lane) & 1u) | (((f1 >> lane) & 1u) << 1) |
+                           (((f2 >> lane) & 1u) << 2);
+    int bin = -1;
+    if (valid) {
+      const int na = rm.n_alphas;
+      if (na == 0) {
+        bin = (int)alpha;
+      } else {
+        int lo = 0, hi = na - 1;
+        while (lo <= hi) {
+          const int mid = (lo + hi) >> 1;
+          const uint32_t v = rm.alpha_sorted[mid];
+          if (v == alpha) { bin = rm.alpha_slot[mid]; break; }
+          if (v < alpha) lo = mid + 1; else hi = mid - 1;
+        }
+      }
+    }
+    if constexpr (WGT) {
+      if (rm.cpl != nullptr && rm.bins <= 8u) {  // whole warp here: see bin_few
+        bin_few(rm, batch, lane, shist, bin);
+        bin = -1;
+      }
+    }
+    if (bin >= 0) {
+      bool done = false;
+      if constexpr (WGT) {
+        if (rm.cpl != nullptr) {
+          double cs, sn;
+          phasor(phase, cs, sn);
+          if (shist) {
+            double* sd = reinterpret_cast<double*>(shist) + 4u * (uint32_t)bin;
+            atomic_add_comp(&sd[0], &sd[2], cs);
+            atomic_add_comp(&sd[1], &sd[3], sn);
+            atomicAdd(&shist[8u * rm.bins + (uint32_t)bin], 1u);
+          } else {
+            unsigned long long* c = rm.hist + ((size_t)batch * rm.bins + (uint32_t)bin) * 8u;
+            double* cd = reinterpret_cast<double*>(c);
+            atomic_add_comp(&cd[0], &cd[3], cs);
+            atomic_add_comp(&cd[1], &cd[4], sn);
+            atomicAdd(c + 2, 1ull);
+          }
+          done = true;
+        }
+      }
+      if (!done) {
+        if (shist) atomicAdd(&shist[(uint32_t)bin * 8u + phase], 1u);
+        else atomicAdd(&rm.hist[((size_t)batch * rm.bins + (uint32_t)bin) * 8u + phase], 1ull);
+      }
+    }
+    n_valid += __popc(__ballot_sync(0xffffffffu, valid));
+    n_samples += __popc(__ballot_sync(0xffffffffu, active));
+  }
+};
+
 }  // namespace pb

@@ -153,7 +153,7 @@ __device__ void advance_sweeps(WsHeader* hdr, uint32_t sweep0, uint32_t n_sweeps
 
 // MULTI: some colour class is larger than the consumers.  ADV: the CTA counts
 // itself among those that have read the sweep index.
-template <int NC, bool MULTI, bool ADV>
+template <int NC, bool MULTI, bool ADV, bool WGT>
 __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sweep0,
                                 uint32_t n_sweeps, PlainShape sh, uint32_t* smem, WsHeader* hdr) {
   const RunModelDev rm = rm_g;
@@ -201,7 +201,23 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
   uint32_t* stm = sphx + kPhiloxWords;
   uint32_t* cnt = stm + 144;  // 3 task counters
   uint32_t* smask = cnt + 4;  // 2 periods: the undecided units of each 32
-  uint32_t* shist = rm.hist_smem ? smask + 2 * (punits >> 5) : nullptr;
+  uint32_t* after = smask + 2 * (punits >> 5);
+  // general-gate runs: acceptance thresholds and {p, always-mask} of the
+  // coupled p-bits, per p-bit (colour order) the addresses of its coupled
+  // neighbours and the offset of its acceptance words, gate phases with the
+  // offsets of their words, and two periods of acceptance words (per sweep
+  // one entry a coupled p-bit and a last one that accepts everything)
+  const bool wgt_m = WGT && rm.cpl != nullptr;
+  const int ncp = wgt_m ? uni(md.n_cp) : 0, nug = wgt_m ? uni(md.n_ug) : 0;
+  uint4* sthr = reinterpret_cast<uint4*>(after);
+  uint2* scp = reinterpret_cast<uint2*>(sthr + ncp);
+  uint4* snb = reinterpret_cast<uint4*>(scp + ((ncp + 1) & ~1));
+  uint4* suph = snb + npb;
+  uint32_t* suof = reinterpret_cast<uint32_t*>(suph + nug);
+  uint4* sacc = reinterpret_cast<uint4*>(suof + ((nug + 3) & ~3));
+  if (WGT) after = reinterpret_cast<uint32_t*>(sacc + 2 * ps * (ncp + 1));
+  const uint32_t hist_words = wgt_m ? (rm.bins * 10u + 3u) & ~3u : rm.bins * 8u;
+  uint32_t* shist = rm.hist_smem ? after : nullptr;
 
   // ---- load the group image and the tables
   const uint32_t w_addr = (uint32_t)__cvta_generic_to_shared(W);
@@ -223,7 +239,7 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
   }
   if (shist) {
 #pragma unroll 1
-    for (uint32_t i = tid; i < rm.bins * 8u; i += T) shist[i] = 0u;
+    for (uint32_t i = tid; i < hist_words; i += T) shist[i] = 0u;
   }
   const uint32_t thr0 = md.thr[0], thr1 = md.thr[1], thr2 = md.thr[2], thr3 = md.thr[3];
   const uint32_t k0 = rm.seed_lo, k1 = rm.seed_hi;
@@ -258,7 +274,8 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
     bool ok = D.dst >= n && D.dst < nw;
 #pragma unroll
     for (int l = 0; l < 3; ++l) ok = ok && D.a[l] < nw && D.b[l] < nw;
-    if (D.mflag & 0x38) ok = false;  // coupled, Toffoli and table p-bits: general-gate runs
+    // Toffoli and table p-bits: sweep_kernel; coupled ones: general-gate runs
+    if (D.mflag & (wgt_m ? 0x30 : 0x38)) ok = false;
     if (!ok) {  // never write through a bad index: the entry redraws the scratch word
       set_status(hdr, PB_EINVAL);
       D.dst = (uint16_t)nw;
@@ -272,6 +289,24 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
     auto at = [&](uint32_t w) { return w_addr + 4u * w; };
     sent[i] = make_uint4(at(D.a[0]), at(D.b[0]), at(D.a[1]), at(D.b[1]));
     sent[npb + i] = make_uint4(at(D.a[2]), at(D.b[2]), at(D.dst), m == 2 ? ~0u : 0u);
+    if constexpr (WGT) {
+      uint4 nb = make_uint4(at(D.dst), at(D.dst), 16u * (uint32_t)ncp, 0u);
+      if (ok && wgt_m) {
+        const uint32_t p = (uint32_t)(D.dst - n);
+        const Cpl C = rm.cpl[p];
+        const uint32_t a = C.flags >> 8;
+        if (C.flags & 1u) {
+          if (C.win >= nw || C.wout >= nw || a >= (uint32_t)ncp) {
+            set_status(hdr, PB_EINVAL);
+          } else {
+            nb = make_uint4(at(C.win), at(C.wout), 16u * a, 1u);
+            sthr[a] = make_uint4(C.A[0], C.A[1], C.A[2], C.A[3]);
+            scp[a] = make_uint2(p, C.amask);
+          }
+        }
+      }
+      snb[i] = nb;
+    }
     const uint32_t x = (uint32_t)(D.dst - n) | (uint32_t)m << 12 | (uint32_t)(m & 1) << 30 |
                        (m ? 1u << 31 : 0u);
 #pragma unroll 1
@@ -285,6 +320,18 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
       if (kv != 0xFFFF) svio[kv] = make_uint2(8u * R.vd | (8u * R.va) << 16, 8u * R.vb);
       if (w) sph[(w == 1 ? 0 : w == 2 ? n_ph1 : n_ph1 + n_ph2) + kp] = 8u * R.pa | (8u * R.pb) << 16;
     }
+  }
+  if constexpr (WGT) {
+#pragma unroll 1
+    for (int i = tid; i < nug; i += T) {
+      const UPh U = rm.uph[i];
+      const bool ok = U.wout < nw && U.win < nw;
+      if (!ok) set_status(hdr, PB_EINVAL);
+      suph[i] = ok ? make_uint4(U.ph[0], U.ph[1], U.ph[2], U.ph[3]) : make_uint4(0u, 0u, 0u, 0u);
+      suof[i] = ok ? 8u * U.wout | (8u * U.win) << 16 : zoff | zoff << 16;
+    }
+#pragma unroll 1
+    for (int i = tid; i < 2 * ps; i += T) sacc[i * (ncp + 1) + ncp] = make_uint4(~0u, ~0u, ~0u, ~0u);
   }
   __syncthreads();
   if (ADV) advance_sweeps(hdr, sweep0, n_sweeps);
@@ -445,6 +492,47 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
     }
   };
 
+  // General-gate runs: the acceptance words of 32 units from 32 c on of period
+  // q (unit: coupled p-bit idx mod ncp of the period's sweep idx / ncp).  A
+  // proposed flip of a lane in category e (e_in + 2 e_out, its disagreement
+  // with the coupled neighbours) stands where word e has the lane: always, or
+  // where the tag-6 uniform is below A[e].  Nearly every warp holds a lane
+  // that 8 planes leave undecided, so 16 are compared at once.
+  auto accept_units = [&](const PhiloxPair& P, uint32_t q, uint32_t c, uint32_t units) {
+    const uint32_t idx = 32u * c + (uint32_t)lane;
+    if (WGT && idx < units) {
+      const uint32_t i = idx / (uint32_t)max(ncp, 1), a = idx - i * (uint32_t)ncp;
+      const uint2 cp = scp[a];
+      const uint4 A4 = sthr[a];
+      const uint32_t A[4] = {A4.x, A4.y, A4.z, A4.w};
+      const uint32_t sw = sweep0 + q * (uint32_t)ps + i, p = cp.x | (kTagCouple << 16);
+      uint32_t lt[4], eq[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        lt[e] = (cp.y >> e) & 1u ? ~0u : 0u;
+        eq[e] = ~lt[e];
+      }
+      auto compare = [&](uint4 r, uint32_t grp) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) compare_planes(lt[e], eq[e], A[e], r, grp);
+      };
+      uint4 R0, R1;
+      philox_pair(P, sw, p, R0, R1);
+      compare(R0, 0u);
+      compare(R1, 1u);
+      PhiloxPair P2;
+      load_keys(P2, 2u);
+      philox_pair(P2, sw, p, R0, R1);
+      compare(R0, 2u);
+      compare(R1, 3u);
+#pragma unroll 1
+      for (uint32_t grp = 4; grp < 8u && (eq[0] | eq[1] | eq[2] | eq[3]) != 0u; ++grp)
+        compare(philox_cold(make_uint4(gglob, sw, p, grp), k0, k1), grp);
+      sacc[((q & 1u) * (uint32_t)ps + i) * (uint32_t)(ncp + 1) + a] = make_uint4(lt[0], lt[1], lt[2], lt[3]);
+    }
+    __syncwarp();
+  };
+
   int col_lo[NC + 1];
 #pragma unroll
   for (int c = 0; c <= NC; ++c) col_lo[c] = uni(md.col_off[c]);
@@ -541,6 +629,45 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
       const uint32_t o2 = __shfl_xor_sync(0xffffffffu, f2[0], off);
       add3(f0[0], f1[0], f2[0], o0, o1, o2);
     }
+    auto recorded = [&](uint32_t t) {
+      return t >= rm.burn_in && (rm.record_every == 1u || (t - rm.burn_in) % rm.record_every == 0u);
+    };
+    if constexpr (WGT) {
+      // the general gates' phases (2^-32 turn) of the lane's own chain
+      uint32_t phi[2] = {0u, 0u};
+#pragma unroll 4
+      for (int i = 0; i < nug; ++i) {
+        const uint4 ph = suph[i];
+        const uint32_t e = suof[i] + SS;
+        uint32_t wo[2], wi[2];
+        ldv(e & 0xFFFFu, wo);
+        ldv(e >> 16, wi);
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+          const bool y = (wo[s] >> lane) & 1u, x = (wi[s] >> lane) & 1u;
+          const uint32_t a0 = y ? ph.z : ph.x, a1 = y ? ph.w : ph.y;
+          phi[s] += x ? a1 : a0;
+        }
+      }
+      uint32_t row[2];
+      ldv(S + last_off + 8u * (uint32_t)(lane < n ? lane : 0), row);
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+        if ((uint32_t)s >= ns) break;
+        Recorder rec;
+        rec.viol = viol[s];
+        rec.f0 = __shfl_sync(0xffffffffu, f0[0], 16 * s);
+        rec.f1 = __shfl_sync(0xffffffffu, f1[0], 16 * s);
+        rec.f2 = __shfl_sync(0xffffffffu, f2[0], 16 * s);
+        rec.lastw = lane < n ? row[s] : 0u;
+        rec.phi = phi[s];
+        if (!recorded(sw + (uint32_t)s)) continue;
+        unsigned long long nv = 0ull, nsm = 0ull;
+        rec.bin<true>(rm, g, batch, lane, shist, nv, nsm);
+        n_valid += (uint32_t)nv;
+        n_samples += (uint32_t)nsm;
+      }
+    } else {
     // lanes 16 s + r now hold sweep s; as rows 0..2 of a transpose: the planes
     const int r = lane & 15;
     const uint32_t plane = r == 0 ? f0[0] : (r == 1 ? f1[0] : f2[0]);
@@ -556,8 +683,7 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
     for (int s = 0; s < 2; ++s) {
       if ((uint32_t)s >= ns) break;
       const uint32_t t = sw + (uint32_t)s;
-      if (t < rm.burn_in || (rm.record_every != 1u && (t - rm.burn_in) % rm.record_every != 0u))
-        continue;
+      if (!recorded(t)) continue;
       const uint32_t pl = __shfl_sync(0xffffffffu, plane, 16 * s + (lane & 3));
       uint32_t word = q >= 0 && q < n ? row[s] : 0u;
       uint32_t alpha, phase;
@@ -591,6 +717,7 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
       n_valid += (uint32_t)__popc(__ballot_sync(0xffffffffu, valid));
       n_samples += (uint32_t)__popc(__ballot_sync(0xffffffffu, active));
     }
+    }
   };
 
   // ---- periods: two to fill the pipeline, then period t is redrawn in
@@ -602,7 +729,8 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
     const uint32_t t = it - 2u;
     const bool fill = it < 2u;
     if (fill || warp >= cw) {
-      // tasks of this iteration, longest first: finish period it - 1, record
+      // tasks of this iteration, longest first: finish period it - 1 (after its
+      // acceptance words in a general-gate run), record
       // period it - 3, start period it; the first of a warp is its own, the
       // next come from a counter
       const uint32_t fq = it - 1u, rq = it - 3u, sq = it;
@@ -610,7 +738,8 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
       const uint32_t nw_t = (uint32_t)(fill ? nwarps : nwarps - cw);
       const uint32_t fs = fq < n_periods ? (sweeps_of(fq) * (uint32_t)npb + 31u) >> 5 : 0u;
       const uint32_t ss = sq < n_periods ? (sweeps_of(sq) * (uint32_t)npb + 63u) >> 6 : 0u;
-      const uint32_t nf = (fs + 7u) >> 3, nr = rq < n_periods ? (sweeps_of(rq) + 1u) >> 1 : 0u;
+      const uint32_t au = WGT && fq < n_periods ? sweeps_of(fq) * (uint32_t)ncp : 0u, na = (au + 31u) >> 5;
+      const uint32_t nf = ((fs + 7u) >> 3) + na, nr = rq < n_periods ? (sweeps_of(rq) + 1u) >> 1 : 0u;
       uint32_t* counter = cnt + it % 3u;
       const uint32_t words = keep(ring_addr + 8u * (sq % 3u) * (uint32_t)punits);
       const uint32_t masks = keep((uint32_t)__cvta_generic_to_shared(smask) + 4u * (sq & 1u) * (uint32_t)(punits >> 5));
@@ -621,8 +750,10 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
       for (uint32_t k = w; k < nf + nr + ss;) {
         uint32_t nx = 0u;
         if (lane == 0) nx = atomicAdd(counter, 1u);
-        if (k < nf) {
-          finish_units(fq, k, fs);
+        if (WGT && k < na) {
+          accept_units(P, fq, k, au);
+        } else if (k < nf) {
+          finish_units(fq, k - na, fs);
         } else if (k < nf + nr) {
           const uint32_t i = (k - nf) << 1, sw = sweep0 + rq * (uint32_t)ps + i;
           const uint32_t S = w_addr + iw4 * (1u + (rq & 1u) * (uint32_t)psp + i);
@@ -637,6 +768,7 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
         // the thread's first p-bit of each class: a consumer without one
         // redraws the scratch word from ZERO links
         uint32_t la[NC][3], lb[NC][3], da[NC], M2[NC];
+        [[maybe_unused]] uint32_t wi[NC], wo[NC], ao[NC], cpm = 0u;  // coupled neighbours, words; classes
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
           const int i = col_lo[c] + tid;
@@ -652,9 +784,26 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
           lb[c][2] = has ? y.y : z;
           da[c] = has ? y.z : w_addr + 4u * (uint32_t)nw;
           M2[c] = y.w;
+          if constexpr (WGT) {
+            const uint4 nb = snb[has ? i : 0];
+            wi[c] = has ? nb.x : da[c];
+            wo[c] = has ? nb.y : da[c];
+            ao[c] = has ? nb.z : 16u * (uint32_t)ncp;
+            cpm |= __any_sync(0xffffffffu, has && nb.w) ? 1u << c : 0u;
+          }
         }
         const uint32_t cnt_t = sweeps_of(t);
         // (A, B) of this thread's unit of class 0, sweep 0 of the period
+        [[maybe_unused]] uint32_t acc = (uint32_t)__cvta_generic_to_shared(sacc) +
+                                        16u * (t & 1u) * (uint32_t)(ps * (ncp + 1));
+        // Metropolis acceptance of a coupled p-bit's proposal v: its current
+        // word at d, its neighbours' at i and o, its acceptance words at a
+        auto accept = [&](uint32_t v, uint32_t d, uint32_t i, uint32_t o, uint32_t a) {
+          const uint32_t old = lds(d), e1 = old ^ lds(i), e2 = old ^ lds(o);
+          const uint4 w = lds4(a);
+          const uint32_t lo = (e1 & w.y) | (~e1 & w.x), hi = (e1 & w.w) | (~e1 & w.z);
+          return old ^ ((old ^ v) & ((e2 & hi) | (~e2 & lo)));
+        };
         uint32_t ab_addr = ring_addr + 8u * ((t % 3u) * (uint32_t)punits + (uint32_t)tid);
         // snapshot of word address a: 2 a + so
         const uint32_t sbase = w_addr + 4u * (uint32_t)(iw * (1 + (int)(t & 1u) * psp)) - 2u * w_addr;
@@ -679,7 +828,9 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
               const uint32_t r0 = lds(la[C][0]) ^ lds(lb[C][0]);
               const uint32_t r1 = lds(la[C][1]) ^ lds(lb[C][1]);
               const uint32_t r2 = lds(la[C][2]) ^ lds(lb[C][2]);
-              const uint32_t v = redraw(r0, r1, r2, M2[C], ab);
+              uint32_t v = redraw(r0, r1, r2, M2[C], ab);
+              if constexpr (WGT)
+                if (cpm & (1u << C)) v = accept(v, da[C], wi[C], wo[C], acc + ao[C]);
               sts(da[C], v);
               sts(2u * da[C] + so, v);
               if constexpr (MULTI) {  // further p-bits of a class larger than the consumers
@@ -691,7 +842,11 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
                   const uint32_t s0 = lds(x.x) ^ lds(x.y);
                   const uint32_t s1 = lds(x.z) ^ lds(x.w);
                   const uint32_t s2 = lds(y.x) ^ lds(y.y);
-                  const uint32_t v2 = redraw(s0, s1, s2, y.w, ab2);
+                  uint32_t v2 = redraw(s0, s1, s2, y.w, ab2);
+                  if constexpr (WGT) {
+                    const uint4 nb = snb[lo + k];
+                    if (nb.w) v2 = accept(v2, y.z, nb.x, nb.y, acc + nb.z);
+                  }
                   sts(y.z, v2);
                   sts(2u * y.z + so, v2);
                 }
@@ -710,6 +865,7 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
           if constexpr (NC > 2) step(std::integral_constant<int, 2>{});
           if constexpr (NC > 3) step(std::integral_constant<int, 3>{});
           ab_addr += npb8;
+          if constexpr (WGT) acc += 16u * (uint32_t)(ncp + 1);
         }
       }
     }
@@ -720,7 +876,19 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
   uint32_t* out = rm.state + (size_t)g * npb;
 #pragma unroll 1
   for (int i = tid; i < npb; i += T) out[i] = W[n + i];
-  if (shist) {
+  if (WGT && shist && wgt_m) {  // (re, im, comp re, comp im) doubles per bin, then u32 counts
+    const double* sd = reinterpret_cast<const double*>(shist);
+#pragma unroll 1
+    for (uint32_t i = tid; i < rm.bins; i += T) {
+      const uint32_t cn = shist[8u * rm.bins + i];
+      if (!cn) continue;
+      unsigned long long* c = rm.hist + ((size_t)batch * rm.bins + i) * 8u;
+      double* cd = reinterpret_cast<double*>(c);
+      atomic_add_comp(&cd[0], &cd[3], sd[4u * i], sd[4u * i + 2u]);
+      atomic_add_comp(&cd[1], &cd[4], sd[4u * i + 1u], sd[4u * i + 3u]);
+      atomicAdd(c + 2, (unsigned long long)cn);
+    }
+  } else if (shist) {
     unsigned long long* gh = rm.hist + (size_t)batch * rm.bins * 8u;
 #pragma unroll 1
     for (uint32_t i = tid; i < rm.bins * 8u; i += T)
@@ -734,8 +902,8 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
 }
 
 // One CTA per chain group of every model of the run (flat group index).
-template <int NC, bool MULTI>
-__global__ void __launch_bounds__(kSweepThreadsPlain) sweep_plain_kernel(
+template <int NC, bool MULTI, bool WGT>
+__global__ void __launch_bounds__(WGT ? kSweepThreadsWgt : kSweepThreadsPlain) sweep_plain_kernel(
     const RunModelDev* __restrict__ rm, int n_models, uint32_t n_sweeps, PlainShape sh,
     WsHeader* hdr) {
   extern __shared__ __align__(16) uint32_t smem[];
@@ -744,7 +912,7 @@ __global__ void __launch_bounds__(kSweepThreadsPlain) sweep_plain_kernel(
   const RunModelDev& r = rm[find_model(rm, n_models, flat)];
   const uint32_t g = flat - r.group_base;
   if (g >= r.groups) return;  // (never: the grid is the runs' groups)
-  run_group_plain<NC, MULTI, true>(r, g, sweep0, n_sweeps, sh, smem, hdr);
+  run_group_plain<NC, MULTI, true, WGT>(r, g, sweep0, n_sweeps, sh, smem, hdr);
 }
 
 // Persistent form: a fixed grid pops (model, group) items from a
@@ -765,7 +933,7 @@ __global__ void __launch_bounds__(kSweepThreadsPlain) sweep_plain_persistent_ker
     const uint32_t flat = work[it];
     const RunModelDev& r = rm[find_model(rm, n_models, flat)];
     const uint32_t g = flat - r.group_base;
-    if (g < r.groups) run_group_plain<NC, MULTI, false>(r, g, sweep0, n_sweeps, sh, smem, hdr);
+    if (g < r.groups) run_group_plain<NC, MULTI, false, false>(r, g, sweep0, n_sweeps, sh, smem, hdr);
   }
   // the last CTA to leave also clears the work counter
   if (threadIdx.x == 0 && atomicAdd(&hdr->ctas_done, 1u) == gridDim.x - 1u) {
@@ -792,12 +960,14 @@ static void plain_dispatch(int nc, bool multi, F f) {
 
 cudaError_t launch_sweeps_plain(const RunModelDev* d_rm, int n_models, uint32_t total_groups,
                                 uint32_t n_sweeps, int cons, int prod, int units, int max_col, int nc,
-                                size_t smem_bytes, WsHeader* hdr, cudaStream_t st) {
+                                bool wgt, size_t smem_bytes, WsHeader* hdr, cudaStream_t st) {
   const PlainShape sh{cons, prod / 32 + 1, units};
   const int threads = cons + 32 * sh.work;
   plain_dispatch(nc, max_col > cons, [&](auto c, auto m) {
-    sweep_plain_kernel<decltype(c)::value, decltype(m)::value>
-        <<<total_groups, threads, smem_bytes, st>>>(d_rm, n_models, n_sweeps, sh, hdr);
+    constexpr int NC = decltype(c)::value;
+    constexpr bool M = decltype(m)::value;
+    if (wgt) sweep_plain_kernel<NC, M, true><<<total_groups, threads, smem_bytes, st>>>(d_rm, n_models, n_sweeps, sh, hdr);
+    else sweep_plain_kernel<NC, M, false><<<total_groups, threads, smem_bytes, st>>>(d_rm, n_models, n_sweeps, sh, hdr);
   });
   return cudaGetLastError();
 }
@@ -827,7 +997,8 @@ cudaError_t sweep_plain_prepare() {
   for (int nc = 2; nc <= 4; ++nc)
     for (int multi = 0; multi < 2; ++multi)
       plain_dispatch(nc, multi != 0, [&](auto c, auto m) {
-        opt(sweep_plain_kernel<decltype(c)::value, decltype(m)::value>);
+        opt(sweep_plain_kernel<decltype(c)::value, decltype(m)::value, false>);
+        opt(sweep_plain_kernel<decltype(c)::value, decltype(m)::value, true>);
         opt(sweep_plain_persistent_kernel<decltype(c)::value, decltype(m)::value>);
       });
   return e;
