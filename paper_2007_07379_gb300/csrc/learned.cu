@@ -527,8 +527,8 @@ cudaError_t mh_enqueue_move_dev(const MhCtx& c, cudaStream_t st, WsHeader* hdr,
   move_begin_kernel<<<(warps * 32 + T - 1) / T, T, 0, st>>>(c.state, n, d, c.groups, q.P, q.ctr, c.seed,
                                                             q.lqf, C, hdr, loop);
   // the proposal (sequential over the suffix layers, one CTA per 128
-  // chains) first on st; log q of the current suffix (one CTA per tile and
-  // layer) beside it on the side stream; both read P and k only
+  // chains) first on st; log q of the current suffix (CTAs with an even share of
+  // the tiles' layers) beside it on the side stream; both read P and k only
   cudaError_t e = cudaSuccess;
   if (c.side) {
     if ((e = cudaEventRecord(c.fork, st)) != cudaSuccess || (e = cudaStreamWaitEvent(c.side, c.fork, 0)) != cudaSuccess)

@@ -1057,6 +1057,14 @@ __device__ __forceinline__ void build_x_part(uint8_t* sX, int kin, int n, int r,
   };
   for (int c = c_lo; c < c_hi; ++c) {
     uint4 w;
+    if (8 * c + 8 <= n) {  // bits only: -1.0 with the sign flipped where set
+      const uint32_t b = prev >> (8 * c);
+      auto pair = [&](int k) {
+        return 0xBF80BF80u ^ ((b << (15 - 2 * k)) & 0x8000u) ^ ((b << (30 - 2 * k)) & 0x80000000u);
+      };
+      *reinterpret_cast<uint4*>(base + c * 128) = make_uint4(pair(0), pair(1), pair(2), pair(3));
+      continue;
+    }
     w.x = elem(8 * c) | (elem(8 * c + 1) << 16);
     w.y = elem(8 * c + 2) | (elem(8 * c + 3) << 16);
     w.z = elem(8 * c + 4) | (elem(8 * c + 5) << 16);
@@ -1460,14 +1468,20 @@ __global__ void __launch_bounds__(kFusedThreads) mlp_move64_kernel(FusedArgs a) 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int quad = warp & 3, part = warp >> 2;
   const int H = a.H, kin = a.kin, npad = a.npad;
-  const int r0 = blockIdx.x * kTile64;
   const int kk = a.k_dev ? *a.k_dev : a.k;
-  // kFusedLogQ: layers kk + y L .. kk + y L + L - 1 (L = a.jlast layers per
-  // CTA, so the weights are loaded once for several layers); kFusedSample:
-  // the suffix, layer after layer
-  const int jfirst = MODE == kFusedLogQ ? kk + (int)blockIdx.y * a.jlast : (a.k_dev ? kk : a.j);
-  const int jend = MODE == kFusedSample ? (a.k_dev ? a.d : a.jlast) : min(jfirst + a.jlast - 1, a.d);
-  if (jfirst < 1 || jfirst > a.d) return;  // whole CTA: no layer here
+  // kFusedLogQ: an even share of the (tile, layer) pairs, tile by tile, so
+  // that the weights are loaded once for all of them; kFusedSample: one tile,
+  // the suffix layer after layer
+  int jfirst = a.k_dev ? kk : a.j, jend = a.k_dev ? a.d : a.jlast, tile = blockIdx.x;
+  long long pair = 0, pair_end = 0;
+  if (MODE == kFusedLogQ) {
+    const long long pairs = (long long)((a.rows + kTile64 - 1) / kTile64) * (a.d - kk + 1);
+    pair = (long long)blockIdx.x * pairs / gridDim.x;
+    pair_end = ((long long)blockIdx.x + 1) * pairs / gridDim.x;
+    if (kk < 1 || pair >= pair_end) return;  // whole CTA: no pair here
+  } else if (jfirst < 1 || jfirst > a.d) {
+    return;  // whole CTA: no layer here
+  }
 
   if (warp == 0) tc::tmem_alloc(&tmem_base, 256);
   if (tid == 0) {
@@ -1528,11 +1542,25 @@ __global__ void __launch_bounds__(kFusedThreads) mlp_move64_kernel(FusedArgs a) 
 
   // this thread's row for the logits: lanes < 16 of every warp
   const int srow = 16 * quad + lane;  // row within the tile (lanes < 16)
+  const int groups = (a.n + 3) / 4;  // 4-bit groups of a layer's bits (n <= 32: at most 8)
+  const uint32_t move = MODE == kFusedSample ? *a.move_dev : 0u;
+  // this thread's first piece (row, 16 bytes of 8 elements) of an x tile and
+  // the step to its next one
+  const int pieces = kin / 8;
+  const int xr0 = tid / pieces, xc0 = tid % pieces, xdr = kFusedThreads / pieces, xdc = kFusedThreads % pieces;
+  bool first = true;  // (the whole CTA's)
+  do {  // tiles (kFusedSample: one)
+  if (MODE == kFusedLogQ) {
+    const int S = a.d - kk + 1;
+    tile = (int)(pair / S);
+    jfirst = kk + (int)(pair - (long long)tile * S);
+    jend = (int)min((long long)a.d, jfirst + (pair_end - pair) - 1);
+    pair += jend - jfirst + 1;
+  }
+  const int r0 = tile * kTile64;
   const int chain = r0 + srow;
   const bool live = lane < 16 && chain < a.rows;
   float lq_acc = 0.f;
-  const int groups = (a.n + 3) / 4;  // 4-bit groups of a layer's bits (n <= 32: at most 8)
-  const uint32_t move = MODE == kFusedSample ? *a.move_dev : 0u;
   const uint32_t gc = a.group0 * 32u + (uint32_t)chain;
   // the previous-layer word of every row of the tile, for the x builders
   for (int r = tid; r < kTile64; r += kFusedThreads) {
@@ -1543,9 +1571,11 @@ __global__ void __launch_bounds__(kFusedThreads) mlp_move64_kernel(FusedArgs a) 
 
   for (int jl = jfirst; jl <= jend; ++jl) {
     // ---- x tile: 64 rows x kin, 16-byte pieces of 8 elements
-    const int pieces = kin / 8;
-    for (int v = tid; v < kTile64 * pieces; v += kFusedThreads) {
-      const int r = v / pieces, c = v % pieces;
+    for (int r = xr0, c = xc0; r < kTile64; r += xdr, c += xdc) {
+      if (c >= pieces) {
+        c -= pieces;
+        if (++r >= kTile64) break;
+      }
       build_x_part(sX, kin, a.n, r, wrd[r], jl, c, c + 1);
     }
     publish();
@@ -1564,7 +1594,8 @@ __global__ void __launch_bounds__(kFusedThreads) mlp_move64_kernel(FusedArgs a) 
         tc::mma_commit(done);
       }
     }
-    ok = __syncthreads_and(ok) != 0;  // thread 0's weight wait, shared
+    if (first) ok = __syncthreads_and(ok) != 0;  // thread 0's weight wait, shared
+    first = false;
     wait_all(done, dph);
     dph ^= 1u;
     if (ok) epilogue(sB);
@@ -1680,6 +1711,7 @@ __global__ void __launch_bounds__(kFusedThreads) mlp_move64_kernel(FusedArgs a) 
     __syncthreads();  // the drawn words are visible to the next x tile
   }  // layers
   if (MODE == kFusedSample && ok && live && part == 0) a.lqf[chain] += lq_acc;
+  } while (MODE == kFusedLogQ && pair < pair_end);
   if (!ok && tid == 0) {
     if (a.status) atomicCAS(a.status, 0u, (uint32_t)PB_ETIMEOUT);
     // let MMAs and copies in flight drain (bounded) before TMEM and shared
@@ -1742,12 +1774,19 @@ cudaError_t mlp_fused_logq_dev(pb_mlp* p, const uint32_t* P, uint32_t beta, int 
   a.k_dev = k_dev;
   a.lq = lq;
   if (const size_t smem64 = fused64_layout(a)) {  // 64-row tiles, weights resident
-    // layers per CTA: one while the (tile, layer) pairs are few, more as the
-    // chains grow, so that the weights are loaded once for several layers
+    // CTAs: the SMs that the draw beside it (a CTA a tile, as long as a
+    // tile's whole suffix) leaves free, where these finish before it does; two
+    // a tile when the tiles fill the GPU (one evened the SMs' loads less: 1.23
+    // ms a move of 65,536 chains against 1.21); every SM's worth between the
+    // two.  A CTA for each (tile, layer) loaded 200 KB of weights and set up
+    // tensor memory for one layer's work (200 moves and sweeps of 4096 chains:
+    // 17.3 -> 16.9 ms, with the x tiles' shorter code 16.8)
     const int tiles = (chains + kTile64 - 1) / kTile64;
-    a.jlast = std::max(1, std::min(p->d, tiles * p->d / 4096));
-    dim3 grid(tiles, (p->d + a.jlast - 1) / a.jlast);
-    mlp_move64_kernel<kFusedLogQ><<<grid, kFusedThreads, smem64, st>>>(a);
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int ctas = 2 * tiles <= sms ? sms - tiles : std::max(sms, 2 * tiles);
+    mlp_move64_kernel<kFusedLogQ><<<ctas, kFusedThreads, smem64, st>>>(a);
     return cudaGetLastError();
   }
   dim3 grid((chains + 127) / 128, p->d);
