@@ -334,7 +334,7 @@ def main():
                 "unit": "T int32 logic ops/s", "frac": achieved / peak_ops, "traffic": None,
                 "peak_basis": f"{sms} SMs x {LOGIC_LANES_PER_SM} int32 logic lanes per clock "
                               f"x {sm_max:.0f} MHz ({peak_kind} sm_max)",
-                "kernel": "sweep_kernel", "launch_ms": statistics.mean(sweep_ms),
+                "kernel": "sweep_plain_kernel", "launch_ms": statistics.mean(sweep_ms),
                 "alg_logic_ops_per_flip": alg_logic_slots_per_word() / 32,
                 "alg_mul_ops_per_flip": expected_calls(32) * PHILOX_MUL_SLOTS / 32,
                 "frac_of_issue": words_per_launch * alg_slots_per_word() / launch_s
@@ -380,7 +380,7 @@ def main():
             "warmup": args.warmup, "ms_per_step": 1e3 * total_s / args.steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "u32", "data": "synthetic",
             "config": _config(wl, args, world), "clocks": clocks, "e2e": e2e,
-            "gpu_launches": 3 * args.steps, "roofline": roofline, "cpu_baseline": cpu,
+            "gpu_launches": 2 * args.steps, "roofline": roofline, "cpu_baseline": cpu,
             "samples_per_s": world * wl.chains * S * args.steps / total_s,
             "learned_vs_plain": learned,
             "other_workloads": extra,
@@ -725,7 +725,7 @@ def kernel_rev() -> str:
     traffic figure to the kernel it was measured on)."""
     import hashlib
     h = hashlib.sha256()
-    for f in ("sweep.cu", "philox.cuh", "pb_internal.h"):
+    for f in ("sweep_plain.cu", "sweep_common.cuh", "philox.cuh", "pb_internal.h"):
         with open(os.path.join(ROOT, "paper_2007_07379_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]

@@ -331,9 +331,11 @@ typedef struct {
 PB_API int pb_run_stats(pb_run* run, pb_run_stats_t* stats);
 
 /* CTA shape of the sweep launches: consumer threads (redraw one colour
- * class, 32..224), producer threads (the Philox planes the consumers
- * compare against, made one or two colour steps ahead, 32..352), both
- * multiples of 32, plus one recorder warp; blocks_per_sm
+ * class, 32..224), producer threads (the comparison words the consumers
+ * read, made whole sweeps ahead, and the records of the sweeps done; in
+ * Toffoli and table runs the Philox planes of the next colour step,
+ * 32..352), both multiples of 32, plus one warp (a recorder in Toffoli and
+ * table runs, one more producer elsewhere); blocks_per_sm
  * caps the persistent grid of batched runs (0 = as many as fit).  A run
  * with PB_U models takes at most 512 threads (consumers + producers + 32;
  * PB_ERANGE otherwise).  The results do not depend on the shape. */
@@ -370,9 +372,10 @@ PB_API int pb_philox_fill(const uint32_t* d_ctr, uint32_t k0, uint32_t k1,
  * whose host application owns every device allocation, or code that runs
  * while a memory budget is frozen).  It is one complete plain Gibbs run (the
  * same kernels and results as pb_run_create + pb_run_sweeps + the histogram)
- * whose scratch -- run header, tables, chain state, counters -- lives in a
+ * whose scratch -- run header, tables, chain state -- lives in a
  * fixed 16 MiB array in device memory that every GPU loading the library
- * holds until the process exits.  It calls no allocator.
+ * holds until the process exits; the counts are summed in the caller's
+ * buffers where these are aligned for it.  It calls no allocator.
  *   m        compiled model, n <= 16 (the full 2^n histogram is recorded).
  *   cfg      as for pb_run_create; alphas must be NULL, sampler PB_GIBBS.
  *            The run starts at sweep 0 from freshly drawn valid paths.

@@ -272,11 +272,12 @@ constexpr int kProducersMax = 352;
 // SMs; smem(units): shared memory of a CTA with that period.
 // Two CTAs an SM where there are groups for them and they fit: the roles of
 // one hide the other's latencies (large workload, ms per 1e3 sweeps: 64
-// consumers + 256 producers, two CTAs, 17.2; 64 + 352, one CTA, 21.8).
+// consumers + 256 producers, two CTAs, 17.2; 64 + 352, one CTA, 21.8, both
+// before the last 0.8 came off the shape that was kept).
 // Otherwise one CTA an SM with a consumer per p-bit of the largest class, as
 // many producers as a period has tasks for and a longer period, whose tasks
 // spread more evenly over the warps (mid, ms per 1e4 sweeps: 4096 units
-// 4.73, 2048 4.89; learned 7.00 and 7.90).
+// 4.73, 2048 4.89; learned 7.00, now 6.85, and 7.90).
 struct PlainDefault {
   int cons, prod, units;
 };

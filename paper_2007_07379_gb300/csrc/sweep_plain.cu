@@ -22,15 +22,20 @@
 // 32 to a warp, so a p-bit costs 2.2 Philox calls on average instead of the 4
 // that a fixed number of planes needs to be nearly always enough.
 //
-// What bounds it: issue slots.  An update costs about 9 warp instructions per
-// 32 of them (two Philox calls 102 of ~290 per 32 units; a call's multiplies
-// alone would allow 17 cycles a warp and SM), and about 55 % of the issue
-// slots are used: one CTA's ~16 warps do not hide every latency.  Measured
+// What bounds it: issue slots, and where one CTA has an SM to itself the
+// consumers' chain beside them.  A word update (32 chains) costs about 8 warp
+// instructions' lanes, two Philox calls being 40 % of them (a call's multiplies
+// alone take 17 cycles a warp and SM), and 53-59 % of the issue slots are used:
+// an SM's ~16 warps do not hide every latency.  On mid a colour step is about
+// 323 cycles; on tiny (one warp of consumers) the chain of loads, logic and
+// barrier is 155 cycles a step and nothing else counts.  Measured
 // against the kernel this replaced (16 planes for every p-bit, the comparison
 // on the consumers' path, one recorder warp, a CTA barrier per class; ms):
 // mid (12 qubits, 20 layers, 4096 chains, 1e4 sweeps) 13.0 -> 4.7, large (24
-// qubits, 32 layers, 65,536 chains, 1e3 sweeps) 41.9 -> 17.3, tiny (1e4
-// sweeps) 9.0 -> 1.6, 256 batched circuits (1e4 sweeps) 502 -> 157.
+// qubits, 32 layers, 65,536 chains, 1e3 sweeps) 41.9 -> 16.4, tiny (1e4
+// sweeps) 9.0 -> 1.6, 256 batched circuits (300 sweeps) 15.2 -> 4.35; with
+// general one-qubit gates, whose acceptance words are made ahead as well,
+// general_mid (35 coupled gates, 4096 chains, 2e3 sweeps) 6.63 -> 3.1.
 #include <cuda_runtime.h>
 
 #include <type_traits>
