@@ -34,6 +34,7 @@ enum : int {
   kEpiAccum = 4,    // fp32 output: D += x
   kEpiMask = 8,     // x *= (mask[row, col] > 0)   (ReLU derivative)
   kEpiBce = 16,     // fp32 logits: also the cross-entropy's gradient and terms
+  kEpiPublic = kEpiRelu | kEpiOutBf16 | kEpiAccum | kEpiMask,  // flags of pb_gemm_bf16
 };
 
 struct GemmArgs {
@@ -394,6 +395,7 @@ extern "C" PB_API int pb_gemm_bf16(const void* dA, int lda, const void* dB, int 
   if ((K % 8) || (lda % 8) || (ldb % 8) || lda < K || ldb < K || ldd < N) return PB_EINVAL;
   if (((uintptr_t)dA & 15) || ((uintptr_t)dB & 15)) return PB_EINVAL;
   if ((flags & kEpiMask) && (!dmask || ldm < N)) return PB_EINVAL;
+  flags &= kEpiPublic;  // (kEpiBce would write through pointers that this call does not have)
   GemmArgs g{};
   g.A = static_cast<const __nv_bfloat16*>(dA);
   g.B = static_cast<const __nv_bfloat16*>(dB);
