@@ -493,8 +493,10 @@ PB_API int pb_mlp_train_paths(pb_mlp* mlp, const uint32_t* d_paths, uint64_t n_p
  * 16-byte aligned rows), fp32 accumulation.  flags: 1 ReLU, 2 store bf16
  * (else fp32), 4 accumulate into fp32 D, 8 multiply by [mask(row,col) > 0]
  * (mask bf16, leading dimension ldm); other bits are ignored.  dbias (fp32,
- * N) may be NULL.  All pointers are device pointers; asynchronous on
- * `stream`.  Errors: PB_EINVAL (shapes, alignment), PB_ECUDA. */
+ * N) may be NULL.  D may lie over A, row on row, where N <= 64, and over B
+ * where M <= 128 too; elsewhere it must not overlap them.  All pointers are
+ * device pointers; asynchronous on `stream`.  Errors: PB_EINVAL (shapes,
+ * alignment), PB_ECUDA. */
 PB_API int pb_gemm_bf16(const void* dA, int lda, const void* dB, int ldb, void* dD, int ldd,
                         const float* dbias, const void* dmask, int ldm, int M, int N, int K,
                         int flags, float alpha, uintptr_t stream);

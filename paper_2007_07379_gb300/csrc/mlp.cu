@@ -69,15 +69,18 @@ __host__ __device__ inline int gemm_stages(int tm, int bn) {
   return 4 * gemm_stage_bytes(tm, bn) <= kGemmSmemMax ? 4 : 2;
 }
 // Tile: 128 rows and N rounded up to 16, at most 256, narrowed step by step to
-// 64 x 32 while the tiles would leave most of the 152 SMs idle.
-inline void gemm_tiles(GemmArgs& g) {
+// 64 x 32 while the tiles would leave most of the 152 SMs idle.  A result that
+// lies over an operand (in_place) keeps at least 64 columns a tile: with one
+// tile across N, a CTA has read all it needs of the rows that it writes (M <=
+// 128 too: all of B), which smaller tiles would lose.
+inline void gemm_tiles(GemmArgs& g, bool in_place) {
   int bn = ((g.N + 15) / 16) * 16, tm = 128;
   if (bn > 256) bn = 256;
   auto tiles = [&] { return ((g.M + tm - 1) / tm) * ((g.N + bn - 1) / bn); };
   if (bn > 128 && tiles() < 120) bn = 128;
   if (bn > 64 && tiles() < 120) bn = 64;
-  if (tiles() < 120) tm = 64;
-  if (bn > 32 && tiles() < 120) bn = 32;
+  if (!in_place && tiles() < 120) tm = 64;
+  if (!in_place && bn > 32 && tiles() < 120) bn = 32;
   g.tm = tm;
   g.bn = bn;
 }
@@ -353,8 +356,8 @@ cudaError_t mlp_prepare() {
   return e == cudaSuccess ? mlp_fused_prepare() : e;
 }
 
-cudaError_t launch_gemm_bf16(GemmArgs g, cudaStream_t st) {
-  gemm_tiles(g);
+cudaError_t launch_gemm_bf16(GemmArgs g, cudaStream_t st, bool in_place = false) {
+  gemm_tiles(g, in_place);
   dim3 grid((g.M + g.tm - 1) / g.tm, (g.N + g.bn - 1) / g.bn);
   const size_t smem = (size_t)gemm_stages(g.tm, g.bn) * gemm_stage_bytes(g.tm, g.bn);
   gemm_kernel(g)<<<grid, kGemmThreads, smem, st>>>(g);
@@ -413,8 +416,15 @@ extern "C" PB_API int pb_gemm_bf16(const void* dA, int lda, const void* dB, int 
   g.alpha = alpha;
   g.status = nullptr;
   if (mlp_prepare() != cudaSuccess) return PB_ECUDA;
-  return launch_gemm_bf16(g, reinterpret_cast<cudaStream_t>(stream)) == cudaSuccess ? PB_OK
-                                                                                   : PB_ECUDA;
+  const uintptr_t d0 = (uintptr_t)dD, d1 = d0 + ((size_t)(M - 1) * ldd + N) * (flags & kEpiOutBf16 ? 2 : 4);
+  auto over = [&](const void* p, int rows, int ld) {
+    const uintptr_t x = (uintptr_t)p;
+    return x < d1 && d0 < x + ((size_t)(rows - 1) * ld + K) * 2;
+  };
+  return launch_gemm_bf16(g, reinterpret_cast<cudaStream_t>(stream), over(dA, M, lda) || over(dB, N, ldb)) ==
+                 cudaSuccess
+             ? PB_OK
+             : PB_ECUDA;
 }
 
 // ===========================================================================

@@ -33,3 +33,21 @@ def test_other_flag_bits_are_ignored(flags, extra):
     pbits.gemm_bf16(A, B, want, flags=flags)
     pbits.gemm_bf16(A, B, got, flags=flags | extra)
     assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("M", [1, 100, 128, 300, 5000])
+@pytest.mark.parametrize("N,K", [(64, 64), (33, 72), (17, 256)])
+def test_result_over_an_operand(M, N, K):
+    """D in A's place row by row, and (one row tile) in B's place: each CTA
+    reads the rows that it writes before it writes them."""
+    import torch
+    A, B = _operands(M, N, K, seed=M + N + K)
+    want = (A.double() @ B.double().T).to(torch.bfloat16)
+    X = A.clone()
+    pbits.gemm_bf16(X, B, X[:, :N], flags=pbits.EPI_OUT_BF16)
+    assert torch.equal(X[:, :N], want) and torch.equal(X[:, N:], A[:, N:])
+    if M <= 128:
+        buf = torch.zeros((max(M, N), K), dtype=torch.bfloat16, device="cuda")
+        buf[:N] = B
+        pbits.gemm_bf16(A, buf[:N], buf[:M, :N], flags=pbits.EPI_OUT_BF16)
+        assert torch.equal(buf[:M, :N], want)
