@@ -375,7 +375,8 @@ PB_API int pb_philox_fill(const uint32_t* d_ctr, uint32_t k0, uint32_t k1,
  * whose scratch -- run header, tables, chain state -- lives in a
  * fixed 16 MiB array in device memory that every GPU loading the library
  * holds until the process exits; the counts are summed in the caller's
- * buffers where these are aligned for it.  It calls no allocator.
+ * buffers where these are aligned for it.  It calls no allocator and keeps
+ * less than 4 KB on the caller's stack.
  *   m        compiled model, n <= 16 (the full 2^n histogram is recorded).
  *   cfg      as for pb_run_create; alphas must be NULL, sampler PB_GIBBS.
  *            The run starts at sweep 0 from freshly drawn valid paths.

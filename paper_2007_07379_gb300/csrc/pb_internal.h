@@ -256,9 +256,27 @@ struct pb_model {
   int n_tab = 0;                      // two-qubit table gates
   std::vector<pb::TAcc> tacc;         // by p (table models only)
   std::vector<pb::TRec> trec;         // one per table gate
+  std::vector<char> tables;           // models of the no-allocation run: desc, rec and init in one
+                                      // block (table_offsets), which a call uploads from here
 };
 
 namespace pb {
+// Models that the no-allocation run takes, and their tables' places in one
+// block.
+inline bool noalloc_model(const pb_model& m) { return !m.wgt && m.n <= 16; }
+struct TableOffsets {
+  size_t desc, rec, init, bytes;
+};
+inline TableOffsets table_offsets(size_t npb) {
+  auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
+  TableOffsets t;
+  t.desc = 0;
+  t.rec = up(npb * sizeof(Desc));
+  t.init = up(t.rec + npb * sizeof(Rec));
+  t.bytes = t.init + npb * 4;
+  return t;
+}
+
 // Philox calls the producers of a general-gate launch make in one colour
 // step: 3 per p-bit of the next class (12 planes ahead, two buffers).
 inline int sweep_producers_wanted(const pb_model& m) {

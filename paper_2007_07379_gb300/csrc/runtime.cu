@@ -677,6 +677,13 @@ PB_API int pb_compile_g(int n, int d, const pb_gate* gates, int n_gates, const d
     }
     m->rank = nvar > 0 ? gf2_rank_rows(wire, nvar) : 0;
   }
+  if (noalloc_model(*m)) {
+    const TableOffsets t = table_offsets((size_t)npb);
+    m->tables.assign(t.bytes, 0);
+    std::memcpy(m->tables.data() + t.desc, m->desc.data(), (size_t)npb * sizeof(Desc));
+    std::memcpy(m->tables.data() + t.rec, m->rec.data(), (size_t)npb * sizeof(Rec));
+    std::memcpy(m->tables.data() + t.init, m->init.data(), (size_t)npb * 4);
+  }
   *out = m.release();
   return PB_OK;
 }

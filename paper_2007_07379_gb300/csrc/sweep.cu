@@ -705,8 +705,7 @@ __global__ void __launch_bounds__(kSweepThreadsWgt) sweep_kernel(const RunModelD
 }
 
 // ---------------------------------------------------------------------------
-// Initial chains: a valid path with random H outputs (tag-1 stream), every
-// other bit its deterministic value, layer by layer.
+// Initial chains of every group (init_group).
 __global__ void init_kernel(const RunModelDev* __restrict__ rm, int n_models,
                             uint32_t total_groups, const uint32_t* const* __restrict__ init_tabs,
                             WsHeader* hdr) {
@@ -717,40 +716,7 @@ __global__ void init_kernel(const RunModelDev* __restrict__ rm, int n_models,
   const RunModelDev& r = rm[mi];
   const uint32_t g = flat - r.group_base;
   if (g >= r.groups) return;
-  const ModelDev* mp = r.model;
-  const int n = mp->n, d = mp->d, nw = mp->nw;
-  const uint32_t* itab = init_tabs[mi];  // per p-bit: 0xFFFFFFFF = H, else a | b << 16
-  uint32_t* W = smem;
-  for (int i = threadIdx.x; i < nw; i += blockDim.x) {
-    uint32_t v = 0u;
-    if (i < n) v = ((mp->beta >> i) & 1u) ? ~0u : 0u;
-    else if (i == ones_idx(n, d)) v = ~0u;
-    W[i] = v;
-  }
-  __syncthreads();
-  for (int k = 1; k <= d; ++k) {
-    for (int q = threadIdx.x; q < n; q += blockDim.x) {
-      const int p = (k - 1) * n + q;
-      const uint32_t e = itab[p];
-      uint32_t v;
-      if (e == 0xFFFFFFFFu) {
-        v = philox4x32_10(make_uint4(g + r.group0, 0u, (uint32_t)p | (kTagInit << 16), 0u),
-                          r.seed_lo, r.seed_hi).x;
-      } else if (e == 0xFFFFFFFEu) {  // Toffoli target: its own general link
-        const GLink* G = r.glk ? r.glk + p : nullptr;
-        if (!G || G->a[0] >= nw || G->b[0] >= nw || G->c[0] >= nw) { set_status(hdr, PB_EINVAL); v = 0u; }
-        else v = W[G->a[0]] ^ (W[G->b[0]] & W[G->c[0]]);
-      } else {
-        const uint32_t a = e & 0xFFFFu, b = e >> 16;
-        if ((int)a >= nw || (int)b >= nw) { set_status(hdr, PB_EINVAL); v = 0u; }
-        else v = W[a] ^ W[b];
-      }
-      W[k * n + q] = v;
-    }
-    __syncthreads();
-  }
-  uint32_t* out = r.state + (size_t)g * n * d;
-  for (int i = threadIdx.x; i < n * d; i += blockDim.x) out[i] = W[n + i];
+  init_group(r, *r.model, g, init_tabs[mi], smem, hdr);
 }
 
 // ---------------------------------------------------------------------------

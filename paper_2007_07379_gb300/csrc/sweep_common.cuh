@@ -54,6 +54,44 @@ __device__ __forceinline__ void set_status(WsHeader* hdr, int code) {
 // colour class), rounded up to 16 bytes.
 __host__ __device__ inline int image_words(int n, int d) { return (n_words(n, d) + 1 + 3) & ~3; }
 
+// Initial chains of group g: a valid path with random H outputs (tag-1
+// stream), every other bit its deterministic value, layer by layer.  The whole
+// CTA; W: n_words of shared memory; itab per p-bit: 0xFFFFFFFF = H, else
+// a | b << 16.
+static __device__ void init_group(const RunModelDev& r, const ModelDev& md, uint32_t g,
+                                  const uint32_t* __restrict__ itab, uint32_t* W, WsHeader* hdr) {
+  const int n = md.n, d = md.d, nw = md.nw;
+  for (int i = threadIdx.x; i < nw; i += blockDim.x) {
+    uint32_t v = 0u;
+    if (i < n) v = ((md.beta >> i) & 1u) ? ~0u : 0u;
+    else if (i == ones_idx(n, d)) v = ~0u;
+    W[i] = v;
+  }
+  __syncthreads();
+  for (int k = 1; k <= d; ++k) {
+    for (int q = threadIdx.x; q < n; q += blockDim.x) {
+      const int p = (k - 1) * n + q;
+      const uint32_t e = itab[p];
+      uint32_t v;
+      if (e == 0xFFFFFFFFu) {
+        v = philox4x32_10(make_uint4(g + r.group0, 0u, (uint32_t)p | (kTagInit << 16), 0u),
+                          r.seed_lo, r.seed_hi).x;
+      } else if (e == 0xFFFFFFFEu) {  // Toffoli target: its own general link
+        const GLink* G = r.glk ? r.glk + p : nullptr;
+        if (!G || G->a[0] >= nw || G->b[0] >= nw || G->c[0] >= nw) { set_status(hdr, PB_EINVAL); v = 0u; }
+        else v = W[G->a[0]] ^ (W[G->b[0]] & W[G->c[0]]);
+      } else {
+        const uint32_t a = e & 0xFFFFu, b = e >> 16;
+        if ((int)a >= nw || (int)b >= nw) { set_status(hdr, PB_EINVAL); v = 0u; }
+        else v = W[a] ^ W[b];
+      }
+      W[k * n + q] = v;
+    }
+    __syncthreads();
+  }
+  uint32_t* out = r.state + (size_t)g * n * d;
+  for (int i = threadIdx.x; i < n * d; i += blockDim.x) out[i] = W[n + i];
+}
 
 // 32 x 32 bit transpose across a warp: on entry lane r holds row r; on
 // return lane c holds column c (bit r = bit c of row r).  Five butterfly
