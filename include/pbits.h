@@ -342,9 +342,10 @@ PB_API int pb_run_stats(pb_run* run, pb_run_stats_t* stats);
 PB_API int pb_run_set_shape(pb_run* run, int consumers, int producers, int blocks_per_sm);
 PB_API int pb_run_get_shape(const pb_run* run, int* consumers, int* producers, int* blocks_per_sm,
                             int* grid);
-/* Autotuner: times trial_sweeps sweeps of each candidate shape on the run
- * itself (the run's state, counters and sweep index are restored after
- * every trial, so the run is unchanged) and keeps the fastest.  cache_path
+/* Autotuner: times trial_sweeps sweeps of each candidate shape, the default
+ * one among them, on the run itself (the run's state, counters and sweep
+ * index are restored after every trial, so the run is unchanged) and keeps
+ * the fastest for launches of that length.  cache_path
  * (may be NULL): a text file of earlier results keyed by the run's (n, d,
  * chains) list; a hit applies the cached shape without trials.  *best_ms
  * (may be NULL) receives the time of trial_sweeps sweeps with that shape. */

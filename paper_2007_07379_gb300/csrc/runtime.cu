@@ -924,6 +924,7 @@ struct pb_run {
   uint32_t total_groups = 0;
   int threads = 32;
   int cons = 32, prod = 32, max_col = 1, blocks_per_sm = 0;
+  int cons0 = 32, prod0 = 32;  // the default shape (choose_shape)
   int units = 0;           // plain runs: units of a period
   size_t smem = 0;
   bool persistent = false;
@@ -1396,6 +1397,8 @@ PB_API int pb_run_create(pb_model* const* models, const pb_run_cfg* cfgs, int n_
       elim_plain_prepare() != cudaSuccess)
     return PB_ECUDA;
   choose_shape(r.get());
+  r->cons0 = r->cons;
+  r->prod0 = r->prod;
   if (r->smem > kSweepSmemMax || r->elim_smem > kSweepSmemMax) return PB_ERANGE;
   if ((e = cudaMemcpyAsync(ws + r->L.rm, r->rm.data(), sizeof(RunModelDev) * n_models,
                            cudaMemcpyHostToDevice, st)) ||
@@ -1683,34 +1686,36 @@ PB_API int pb_run_tune(pb_run* r, uint32_t trial_sweeps, const char* cache_path,
   for (auto& m : r->models)
     for (int c = 0; c < 4; ++c) maxcol = std::max(maxcol, m->col_off[c + 1] - m->col_off[c]);
   const int up = ((maxcol + 31) / 32) * 32;
-  std::vector<int> cons_c, prod_c, bpsm_c = {0};
-  for (int c : {64, 128, 224})
-    if (c <= std::max(64, up)) cons_c.push_back(c);
+  // candidates: the default shape first (of equal times the first is kept),
+  // then a grid
+  std::vector<int> bpsm_c = {0};
+  std::vector<std::pair<int, int>> shapes = {{r->cons0, r->prod0}};
   int pw = 352;
   if (r->wgt) {
     pw = 32;
     for (auto& m : r->models) pw = std::max(pw, sweep_producers_wanted(*m));
   }
-  for (int p : {96, 192, 256, 352})
-    if (p <= std::max(96, ((pw + 31) / 32) * 32)) prod_c.push_back(p);
-  if (r->nm > 1) bpsm_c = {1, 2, 0};
+  for (int c : {64, 128, 224})
+    for (int p : {96, 192, 256, 352})
+      if (c <= std::max(64, up) && p <= std::max(96, ((pw + 31) / 32) * 32) && shapes[0] != std::make_pair(c, p))
+        shapes.emplace_back(c, p);
+  if (r->nm > 1) bpsm_c = {0, 1, 2};
   double best = 1e30;
   int bc = r->cons, bp = r->prod, bb = r->blocks_per_sm;
-  for (int c : cons_c)
-    for (int p : prod_c)
-      for (int b : bpsm_c) {
-        rc = pb_run_set_shape(r, c, p, b);
-        if (rc == PB_ERANGE) continue;  // a shape that does not fit in shared memory
-        if (rc != PB_OK) return rc;
-        // first launch builds the graph; time the second
-        if ((rc = pb_run_sweeps(r, trial_sweeps)) != PB_OK) return rc;
-        if ((rc = pb_run_sweeps(r, trial_sweeps)) != PB_OK) return rc;
-        pb_run_stats_t st;
-        if ((rc = pb_run_stats(r, &st)) != PB_OK) return rc;
-        if (st.last_ms < best) { best = st.last_ms; bc = c; bp = p; bb = b; }
-        if ((rc = pb_run_restore(r, blob.data(), blob.size())) != PB_OK) return rc;
-        r->sweeps_done = sweeps_before;
-      }
+  for (auto [c, p] : shapes)
+    for (int b : bpsm_c) {
+      rc = pb_run_set_shape(r, c, p, b);
+      if (rc == PB_ERANGE) continue;  // a shape that does not fit in shared memory
+      if (rc != PB_OK) return rc;
+      // first launch builds the graph; time the second
+      if ((rc = pb_run_sweeps(r, trial_sweeps)) != PB_OK) return rc;
+      if ((rc = pb_run_sweeps(r, trial_sweeps)) != PB_OK) return rc;
+      pb_run_stats_t st;
+      if ((rc = pb_run_stats(r, &st)) != PB_OK) return rc;
+      if (st.last_ms < best) { best = st.last_ms; bc = c; bp = p; bb = b; }
+      if ((rc = pb_run_restore(r, blob.data(), blob.size())) != PB_OK) return rc;
+      r->sweeps_done = sweeps_before;
+    }
   if ((rc = pb_run_set_shape(r, bc, bp, bb)) != PB_OK) return rc;
   if (best_ms) *best_ms = best;
   if (cache_path) {
