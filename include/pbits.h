@@ -347,7 +347,8 @@ PB_API int pb_run_get_shape(const pb_run* run, int* consumers, int* producers, i
  * index are restored after every trial, so the run is unchanged) and keeps
  * the fastest for launches of that length.  cache_path
  * (may be NULL): a text file of earlier results keyed by the run's (n, d,
- * chains) list; a hit applies the cached shape without trials.  *best_ms
+ * chains, bins) list, its kernels and the GPU's SM count; a hit whose shape
+ * the run takes applies it without trials.  *best_ms
  * (may be NULL) receives the time of trial_sweeps sweeps with that shape. */
 PB_API int pb_run_tune(pb_run* run, uint32_t trial_sweeps, const char* cache_path, double* best_ms);
 

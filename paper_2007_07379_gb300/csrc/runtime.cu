@@ -1652,13 +1652,21 @@ PB_API int pb_run_tune(pb_run* r, uint32_t trial_sweeps, const char* cache_path,
     if (best_ms) *best_ms = 0.0;
     return PB_OK;
   }
-  // key: the run's shapes
+  // key: what a shape's meaning and speed depend on (kShapeFormat: another
+  // one where the kernels give the two thread counts another meaning)
+  constexpr uint64_t kShapeFormat = 2;
+  int dev = 0, sms = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   uint64_t key = 1469598103934665603ull;
   auto mix = [&](uint64_t v) { key = (key ^ v) * 1099511628211ull; };
+  for (uint64_t v : {kShapeFormat, (uint64_t)sms, (uint64_t)r->wgt, (uint64_t)r->ext, (uint64_t)r->persistent})
+    mix(v);
   for (int i = 0; i < r->nm; ++i) {
     mix((uint64_t)r->models[i]->n);
     mix((uint64_t)r->models[i]->d);
     mix((uint64_t)r->cfgs[i].chains);
+    mix((uint64_t)r->L.ms[i].bins);
   }
   if (cache_path) {
     if (FILE* f = std::fopen(cache_path, "r")) {
@@ -1671,8 +1679,12 @@ PB_API int pb_run_tune(pb_run* r, uint32_t trial_sweeps, const char* cache_path,
         if (k == key) { found = 1; bc = c; bp = p; bb = b; bms = ms; }
       std::fclose(f);
       if (found) {
-        if (best_ms) *best_ms = bms;
-        return pb_run_set_shape(r, bc, bp, bb);
+        const int rc = pb_run_set_shape(r, bc, bp, bb);
+        // (a shape that this run does not take: the trials, as without an entry)
+        if (rc != PB_EINVAL && rc != PB_ERANGE) {
+          if (best_ms) *best_ms = bms;
+          return rc;
+        }
       }
     }
   }
