@@ -154,7 +154,8 @@ extern "C" PB_API int pb_gibbs_run_noalloc(const pb_model* m, const pb_run_cfg* 
     return PB_ECUDA;
   const PlainDefault ps = plain_shape(n * d, maxcol, groups, sms, smem_for);
   const bool hist_smem = hist_fits(ps.units);
-  const size_t smem = smem_for(ps.units);
+  const int units = plain_launch_units(n * d, ps.units, n_sweeps);
+  const size_t smem = plain_smem_bytes(n, d, hist_smem ? bins : 0, units);
   if (smem > kSweepSmemMax) return PB_ERANGE;
 
   NoallocRun run{};
@@ -213,8 +214,9 @@ extern "C" PB_API int pb_gibbs_run_noalloc(const pb_model* m, const pb_run_cfg* 
   if (cudaGetLastError() != cudaSuccess) return PB_ECUDA;
   const RunModelDev* d_rm = run.d_rm;
   WsHeader* hdr = run.d_hdr;
-  if (n_sweeps > 0 && launch_sweeps_plain(d_rm, 1, groups, n_sweeps, ps.cons, ps.prod, ps.units, maxcol,
-                                          nc, false, smem, hdr, st) != cudaSuccess)
+  const int prod = std::min(ps.prod, plain_launch_producers(n * d, ps.cons, ps.units, n_sweeps));
+  if (n_sweeps > 0 && launch_sweeps_plain(d_rm, 1, groups, n_sweeps, ps.cons, prod, units, maxcol, nc,
+                                          false, smem, hdr, st) != cudaSuccess)
     return PB_ECUDA;
   if (!direct && (cudaMemcpyAsync(d_counts, counts, (size_t)bins * 8 * 8, cudaMemcpyDeviceToDevice, st) !=
                       cudaSuccess ||

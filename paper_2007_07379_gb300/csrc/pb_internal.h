@@ -196,6 +196,19 @@ constexpr __host__ __device__ int plain_period(int npb, int units) {
   const int ps = units / npb;
   return ps < 2 ? 1 : (ps > 16 ? 16 : ps & ~1);
 }
+// The period of a launch: shorter where n_sweeps are few, a quarter of them so
+// that the stages overlap, but no less than (up to eight sweeps of) what 16
+// warps start in one task each.
+constexpr __host__ __device__ int plain_launch_period(int npb, int units, uint32_t n_sweeps) {
+  const int ps = plain_period(npb, units);
+  if (ps < 2 || n_sweeps >= 4u * (uint32_t)ps) return ps;
+  if (n_sweeps < 2u) return 1;
+  const int n = (int)n_sweeps, share = ((n + 3) >> 2) & ~1, all = (n + 1) & ~1;
+  int least = (1024 / npb) & ~1;
+  least = least > 8 ? 8 : (least < 2 ? 2 : least);
+  const int want = share > least ? share : (least < all ? least : all);
+  return want < ps ? want : ps;
+}
 // Shared memory of a CTA: the group image, the snapshots of two periods,
 // consumer entries, three periods of comparison words, record lists, the
 // period's units, Philox and threshold words, undecided masks, an optional
@@ -311,6 +324,20 @@ inline PlainDefault plain_shape(int npb, int maxcol, uint32_t groups, int sms, S
   const int tasks = (ps * npb + 63) / 64 + (ps * npb + 255) / 256 + (ps + 1) / 2;
   s.prod = std::max(32, std::min(two ? 256 : 352, 32 * ((tasks + 1) / 2)));
   return s;
+}
+// A launch of few sweeps needs less than the run's shape: the units of its
+// period, and a producer warp for two tasks of an iteration (with one period,
+// the start of its words, their finish and its records are iterations of
+// their own) or a thread for every p-bit of the tables.
+inline int plain_launch_units(int npb, int units, uint32_t n_sweeps) {
+  return plain_launch_period(npb, units, n_sweeps) * npb;
+}
+inline int plain_launch_producers(int npb, int cons, int units, uint32_t n_sweeps) {
+  if (n_sweeps >= 4u * (uint32_t)plain_period(npb, units)) return kProducersMax;
+  const int ps = std::min<uint32_t>(plain_launch_period(npb, units, n_sweeps), n_sweeps);
+  const int start = (ps * npb + 63) / 64, finish = (ps * npb + 255) / 256, record = (ps + 1) / 2;
+  const int tasks = n_sweeps == (uint32_t)ps ? std::max(start, record) : start + finish + record;
+  return std::max(32, std::max(32 * ((tasks + 1) / 2), (npb + 31) / 32 * 32 - cons - 32));
 }
 }  // namespace pb
 

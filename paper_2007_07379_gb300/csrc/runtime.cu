@@ -923,7 +923,7 @@ struct pb_run {
   std::vector<RunModelDev> rm;
   uint32_t total_groups = 0;
   int threads = 32;
-  int cons = 32, prod = 32, max_col = 1, blocks_per_sm = 0;
+  int cons = 32, prod = 32, max_col = 1, max_npb = 1, blocks_per_sm = 0;
   int cons0 = 32, prod0 = 32;  // the default shape (choose_shape)
   int units = 0;           // plain runs: units of a period
   size_t smem = 0;
@@ -968,6 +968,36 @@ int cuda_status(cudaError_t e) { return e == cudaSuccess ? PB_OK : PB_ECUDA; }
 // the graph's while node whether to run another.
 __global__ void periods_init_kernel(WsHeader* hdr, uint32_t periods) { hdr->periods_left = periods; }
 
+// CTAs of a persistent launch.
+int persistent_grid(const pb_run* r, int threads, size_t smem) {
+  int dev = 0, sms = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  int per_sm = sweep_plain_blocks_per_sm(r->max_col, r->cons, r->nc, threads, smem);
+  if (r->blocks_per_sm > 0) per_sm = std::min(per_sm, r->blocks_per_sm);
+  const int grid = std::max(1, sms * std::max(1, per_sm));
+  return (int)std::min<uint32_t>((uint32_t)grid, r->total_groups);
+}
+
+// Shape of a plain run's launch of n sweeps: the run's, smaller where n is
+// small, so that more CTAs share an SM: their set-up is most of such a launch
+// (3 qubits, 4 layers: one sweep of 65,536 chains 39.7 -> 19.6 us, of 256
+// circuits of 256 chains in one persistent launch 48.5 -> 26.0; eight sweeps
+// 70.3 -> 33.7 and 56.8 -> 34.0).
+struct PlainLaunch {
+  int prod, units, grid;
+  size_t smem;
+};
+PlainLaunch plain_launch(const pb_run* r, uint32_t n_sweeps) {
+  PlainLaunch l{std::min(r->prod, plain_launch_producers(r->max_npb, r->cons, r->units, n_sweeps)), 0, r->grid, 0};
+  for (auto& m : r->models) l.units = std::max(l.units, plain_launch_units(m->n * m->d, r->units, n_sweeps));
+  for (int i = 0; i < r->nm; ++i)  // the histograms where the run has them
+    l.smem = std::max(l.smem, plain_smem_bytes(r->models[i]->n, r->models[i]->d,
+                                               r->rm[i].hist_smem ? r->L.ms[i].bins : 0, l.units));
+  if (r->persistent) l.grid = persistent_grid(r, r->cons + l.prod + 32, l.smem);
+  return l;
+}
+
 // The launches of n sweeps of every model (no moves), in stream order.
 cudaError_t enqueue_sweeps(pb_run* r, uint32_t n_sweeps, cudaStream_t st) {
   if (r->elim_plain)
@@ -981,12 +1011,16 @@ cudaError_t enqueue_sweeps(pb_run* r, uint32_t n_sweeps, cudaStream_t st) {
   if (r->ext)
     return launch_sweeps(r->d_rm(), r->nm, r->total_groups, n_sweeps, r->cons, r->prod, r->max_col,
                          r->nc, r->smem, r->hdr(), st);
+  if (r->wgt)
+    return launch_sweeps_plain(r->d_rm(), r->nm, r->total_groups, n_sweeps, r->cons, r->prod, r->units,
+                               r->max_col, r->nc, true, r->smem, r->hdr(), st);
+  const PlainLaunch l = plain_launch(r, n_sweeps);
   if (r->persistent)
     return launch_sweeps_plain_persistent(
         r->d_rm(), r->nm, reinterpret_cast<const uint32_t*>(r->ws + r->L.work), r->total_groups,
-        n_sweeps, r->cons, r->prod, r->units, r->max_col, r->nc, r->grid, r->smem, r->hdr(), st);
-  return launch_sweeps_plain(r->d_rm(), r->nm, r->total_groups, n_sweeps, r->cons, r->prod, r->units,
-                             r->max_col, r->nc, r->wgt, r->smem, r->hdr(), st);
+        n_sweeps, r->cons, l.prod, l.units, r->max_col, r->nc, l.grid, l.smem, r->hdr(), st);
+  return launch_sweeps_plain(r->d_rm(), r->nm, r->total_groups, n_sweeps, r->cons, l.prod, l.units,
+                             r->max_col, r->nc, false, l.smem, r->hdr(), st);
 }
 
 // Graph of n sweeps of a learned run (Fig. 2 Step 1 with the network as the
@@ -1091,17 +1125,8 @@ void apply_shape(pb_run* r, int cons, int prod, int blocks_per_sm) {
   r->persistent = r->nm > 1;
   if (const char* e = std::getenv("PB_PERSISTENT")) r->persistent = std::atoi(e) != 0;
   if (r->wgt) r->persistent = false;  // general-gate sweeps: one CTA per group
-  r->grid = 0;
-  if (r->persistent) {
-    int dev = 0, sms = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int per_sm = sweep_plain_blocks_per_sm(maxcol, cons, r->nc, r->threads, r->smem);
-    if (blocks_per_sm > 0) per_sm = std::min(per_sm, blocks_per_sm);
-    r->grid = std::max(1, sms * std::max(1, per_sm));
-    r->grid = (int)std::min<uint32_t>((uint32_t)r->grid, r->total_groups);
-  }
   r->blocks_per_sm = blocks_per_sm;
+  r->grid = r->persistent ? persistent_grid(r, r->threads, r->smem) : 0;
 }
 
 // General-gate runs count FP64 phase sums (an add returns the old value), which
@@ -1127,7 +1152,7 @@ void choose_shape(pb_run* r) {
   int maxcol = 1, npb = 1, want = 32;
   for (auto& m : r->models) {
     for (int c = 0; c < 4; ++c) maxcol = std::max(maxcol, m->col_off[c + 1] - m->col_off[c]);
-    npb = std::max(npb, m->n * m->d);
+    npb = r->max_npb = std::max(npb, m->n * m->d);
     want = std::max(want, sweep_producers_wanted(*m));
   }
   auto up32 = [](int x) { return ((x + 31) / 32) * 32; };

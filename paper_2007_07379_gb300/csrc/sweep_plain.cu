@@ -172,11 +172,9 @@ __device__ void run_group_plain(const RunModelDev& rm_g, uint32_t g, uint32_t sw
   const int lane = tid & 31, nwarps = T >> 5, warp = uni(tid >> 5);
   const int cw = sh.cons >> 5;
   const int iw = image_words(n, d);
-  // sweeps of a period: fewer in a short launch, so that its stages overlap
-  // (the sizes in shared memory stay within those of the full period)
-  int ps = plain_period(npb, sh.units);
-  if (n_sweeps < 4u * (uint32_t)ps)
-    ps = n_sweeps < 2u ? 1 : min(ps, max(2, (int)((n_sweeps + 3u) >> 2) & ~1));
+  // sweeps of a period (the sizes in shared memory stay within those of a
+  // long launch's period)
+  const int ps = plain_launch_period(npb, sh.units, n_sweeps);
   // units (p-bit updates) of a full period, padded to whole tasks: the
   // padding's words are made like the others and never read
   const int punits = (ps * npb + 63) & ~63;
