@@ -55,12 +55,13 @@ __global__ void __launch_bounds__(512) elim_plain_kernel(
   auto uni = [](auto x) { return __shfl_sync(0xffffffffu, x, 0); };
   const int n = uni(rm.md.n), d = uni(rm.md.d), nw = n_words(n, d), npb = n * d;
   const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, warp = uni(tid >> 5), nwarps = T >> 5;
-  const ElimLayout L = elim_layout(n, d, rm.hist_smem ? rm.bins : 0u);
+  const bool hist_smem = rm.hist_smem && elim_hist_pays(rm.bins, n_sweeps, rm.record_every);
+  const ElimLayout L = elim_layout(n, d, hist_smem ? rm.bins : 0u);
   uint32_t* lnk = smem + L.lnk;
   uint32_t* hp = smem + L.hp;
   uint32_t* sph = smem + L.sph;
   uint32_t* cnt = smem + L.cnt;
-  uint32_t* shist = rm.hist_smem ? smem + L.hist : nullptr;
+  uint32_t* shist = hist_smem ? smem + L.hist : nullptr;
   uint32_t* img = smem + L.img + (uint32_t)warp * L.img_words;
   const uint32_t img_addr = (uint32_t)__cvta_generic_to_shared(img);
   const uint32_t* itab = init_tabs[mi];  // per p-bit: 0xFFFFFFFF = H, else a | b << 16

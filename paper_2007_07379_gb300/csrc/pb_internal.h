@@ -341,6 +341,16 @@ inline int plain_launch_producers(int npb, int cons, int units, uint32_t n_sweep
 }
 }  // namespace pb
 
+namespace pb {
+// Exact sampler of plain models: a launch counts in shared memory where it adds
+// two counts to every counter on average.  Below that, clearing and flushing
+// the histogram cost more than counting in global memory (12 qubits, 16,384
+// chains, one sample: 58.8 us against 17.6; 2000 samples of 4096 chains: equal).
+constexpr __host__ __device__ bool elim_hist_pays(uint32_t bins, uint32_t n_sweeps, uint32_t record_every) {
+  return 2ull * (n_sweeps / record_every) >= bins;
+}
+}  // namespace pb
+
 // Proposal network (host side of pb_mlp): fp32 master weights, Adam state,
 // bf16 copies for the tensor cores and the batch buffers of one call.
 struct pb_mlp {
