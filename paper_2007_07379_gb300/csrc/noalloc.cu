@@ -214,7 +214,8 @@ extern "C" PB_API int pb_gibbs_run_noalloc(const pb_model* m, const pb_run_cfg* 
   if (cudaGetLastError() != cudaSuccess) return PB_ECUDA;
   const RunModelDev* d_rm = run.d_rm;
   WsHeader* hdr = run.d_hdr;
-  const int prod = std::min(ps.prod, plain_launch_producers(n * d, ps.cons, ps.units, n_sweeps));
+  const int prod = std::min(ps.prod, plain_launch_producers(n * d, 0, hist_smem ? bins : 0, groups > (uint32_t)sms,
+                                                            ps.cons, ps.units, n_sweeps));
   if (n_sweeps > 0 && launch_sweeps_plain(d_rm, 1, groups, n_sweeps, ps.cons, prod, units, maxcol, nc,
                                           false, smem, hdr, st) != cudaSuccess)
     return PB_ECUDA;

@@ -326,18 +326,26 @@ inline PlainDefault plain_shape(int npb, int maxcol, uint32_t groups, int sms, S
   return s;
 }
 // A launch of few sweeps needs less than the run's shape: the units of its
-// period, and a producer warp for two tasks of an iteration (with one period,
-// the start of its words, their finish and its records are iterations of
-// their own) or a thread for every p-bit of the tables.
+// period, and a producer warp for two tasks of an iteration: the start of a
+// period's words, their finish (ncp: coupled p-bits, whose acceptance words
+// are tasks too) and its records, which with one period are iterations of
+// their own, and which more CTAs an SM overlap where the groups fill the GPU
+// (full; with coupled p-bits, whose records take as long as the rest, up to
+// three periods).  At least a thread for every p-bit of the tables and for eight bins
+// of a histogram in shared memory.
 inline int plain_launch_units(int npb, int units, uint32_t n_sweeps) {
   return plain_launch_period(npb, units, n_sweeps) * npb;
 }
-inline int plain_launch_producers(int npb, int cons, int units, uint32_t n_sweeps) {
+inline int plain_launch_producers(int npb, int ncp, uint32_t hist_bins, bool full, int cons, int units,
+                                  uint32_t n_sweeps) {
   if (n_sweeps >= 4u * (uint32_t)plain_period(npb, units)) return kProducersMax;
   const int ps = std::min<uint32_t>(plain_launch_period(npb, units, n_sweeps), n_sweeps);
-  const int start = (ps * npb + 63) / 64, finish = (ps * npb + 255) / 256, record = (ps + 1) / 2;
-  const int tasks = n_sweeps == (uint32_t)ps ? std::max(start, record) : start + finish + record;
-  return std::max(32, std::max(32 * ((tasks + 1) / 2), (npb + 31) / 32 * 32 - cons - 32));
+  const int start = (ps * npb + 63) / 64, record = (ps + 1) / 2;
+  const int finish = (ps * npb + 255) / 256 + (ps * ncp + 31) / 32;
+  const bool apart = n_sweeps == (uint32_t)ps || (full && (ncp == 0 || n_sweeps <= 3u * (uint32_t)ps));
+  const int tasks = apart ? std::max(std::max(start, finish), record) : start + finish + record;
+  const int threads = std::max(npb, (int)hist_bins / 8);
+  return std::max(32, std::max(32 * ((tasks + 1) / 2), (threads + 31) / 32 * 32 - cons - 32));
 }
 }  // namespace pb
 

@@ -922,6 +922,7 @@ struct pb_run {
   Layout L;
   std::vector<RunModelDev> rm;
   uint32_t total_groups = 0;
+  bool full = false;       // more chain groups than SMs
   int threads = 32;
   int cons = 32, prod = 32, max_col = 1, max_npb = 1, blocks_per_sm = 0;
   int cons0 = 32, prod0 = 32;  // the default shape (choose_shape)
@@ -937,7 +938,6 @@ struct pb_run {
   int elim_warps = 8;      // exact samplers: warps per CTA
   bool elim_plain = false; // exact-sampler run of plain models, no clamped output
   std::vector<char> elim_hist;  // elim_plain: models whose counts fit shared memory
-  bool elim_full = false;  // more chain groups than SMs
   std::vector<std::vector<uint32_t>> clamp_keep;
   int grid = 0;
   uint64_t sweeps_done = 0;
@@ -969,6 +969,14 @@ int cuda_status(cudaError_t e) { return e == cudaSuccess ? PB_OK : PB_ECUDA; }
 // the graph's while node whether to run another.
 __global__ void periods_init_kernel(WsHeader* hdr, uint32_t periods) { hdr->periods_left = periods; }
 
+// Shared memory of a sweep CTA for model i of a run on the word kernels
+// (sweep_plain.cu).
+size_t word_smem(const pb_run* r, int i, uint32_t bins, int units) {
+  const pb_model& m = *r->models[i];
+  return r->wgt ? general_smem_bytes(m.n, m.d, m.wgt, m.n_cp, (int)m.uph.size(), bins, units)
+                : plain_smem_bytes(m.n, m.d, bins, units);
+}
+
 // CTAs of a persistent launch.
 int persistent_grid(const pb_run* r, int threads, size_t smem) {
   int dev = 0, sms = 1;
@@ -980,21 +988,26 @@ int persistent_grid(const pb_run* r, int threads, size_t smem) {
   return (int)std::min<uint32_t>((uint32_t)grid, r->total_groups);
 }
 
-// Shape of a plain run's launch of n sweeps: the run's, smaller where n is
+// Shape of a launch of n sweeps on the word kernels: the run's, smaller where n is
 // small, so that more CTAs share an SM: their set-up is most of such a launch
 // (3 qubits, 4 layers: one sweep of 65,536 chains 39.7 -> 19.6 us, of 256
 // circuits of 256 chains in one persistent launch 48.5 -> 26.0; eight sweeps
-// 70.3 -> 33.7 and 56.8 -> 34.0).
+// 70.3 -> 33.7 and 56.8 -> 34.0; with half of the gates general, one sweep of
+// the 65,536 chains 118 -> 58).
 struct PlainLaunch {
   int prod, units, grid;
   size_t smem;
 };
 PlainLaunch plain_launch(const pb_run* r, uint32_t n_sweeps) {
-  PlainLaunch l{std::min(r->prod, plain_launch_producers(r->max_npb, r->cons, r->units, n_sweeps)), 0, r->grid, 0};
-  for (auto& m : r->models) l.units = std::max(l.units, plain_launch_units(m->n * m->d, r->units, n_sweeps));
-  for (int i = 0; i < r->nm; ++i)  // the histograms where the run has them
-    l.smem = std::max(l.smem, plain_smem_bytes(r->models[i]->n, r->models[i]->d,
-                                               r->rm[i].hist_smem ? r->L.ms[i].bins : 0, l.units));
+  PlainLaunch l{0, 0, r->grid, 0};
+  auto hist = [&](int i) { return r->rm[i].hist_smem ? r->L.ms[i].bins : 0u; };
+  for (int i = 0; i < r->nm; ++i) {
+    const pb_model& m = *r->models[i];
+    l.units = std::max(l.units, plain_launch_units(m.n * m.d, r->units, n_sweeps));
+    l.prod = std::max(l.prod, plain_launch_producers(m.n * m.d, m.n_cp, hist(i), r->full, r->cons, r->units, n_sweeps));
+  }
+  l.prod = std::min(l.prod, r->prod);
+  for (int i = 0; i < r->nm; ++i) l.smem = std::max(l.smem, word_smem(r, i, hist(i), l.units));
   if (r->persistent) l.grid = persistent_grid(r, r->cons + l.prod + 32, l.smem);
   return l;
 }
@@ -1004,7 +1017,7 @@ PlainLaunch plain_launch(const pb_run* r, uint32_t n_sweeps) {
 // groups fill the GPU (one sample of 3 qubits, 4 layers, 65,536 chains 29.6 ->
 // 10.4 us, of 24 qubits, 32 layers 84.9 -> 56.4).
 cudaError_t enqueue_elim_plain(pb_run* r, uint32_t n, cudaStream_t st) {
-  const int share = r->elim_full ? 256 : 64;
+  const int share = r->full ? 256 : 64;
   const int warps = (int)std::min<uint32_t>(
       (uint32_t)r->elim_warps, std::max<uint32_t>((uint32_t)(r->max_npb + share - 1) / share, (n + 3u) / 4u));
   size_t smem = 0;
@@ -1028,16 +1041,13 @@ cudaError_t enqueue_sweeps(pb_run* r, uint32_t n_sweeps, cudaStream_t st) {
   if (r->ext)
     return launch_sweeps(r->d_rm(), r->nm, r->total_groups, n_sweeps, r->cons, r->prod, r->max_col,
                          r->nc, r->smem, r->hdr(), st);
-  if (r->wgt)
-    return launch_sweeps_plain(r->d_rm(), r->nm, r->total_groups, n_sweeps, r->cons, r->prod, r->units,
-                               r->max_col, r->nc, true, r->smem, r->hdr(), st);
   const PlainLaunch l = plain_launch(r, n_sweeps);
   if (r->persistent)
     return launch_sweeps_plain_persistent(
         r->d_rm(), r->nm, reinterpret_cast<const uint32_t*>(r->ws + r->L.work), r->total_groups,
         n_sweeps, r->cons, l.prod, l.units, r->max_col, r->nc, l.grid, l.smem, r->hdr(), st);
   return launch_sweeps_plain(r->d_rm(), r->nm, r->total_groups, n_sweeps, r->cons, l.prod, l.units,
-                             r->max_col, r->nc, false, l.smem, r->hdr(), st);
+                             r->max_col, r->nc, r->wgt, l.smem, r->hdr(), st);
 }
 
 // Graph of n sweeps of a learned run (Fig. 2 Step 1 with the network as the
@@ -1113,9 +1123,7 @@ size_t plan_smem(const pb_run* r, int units, std::vector<char>* use) {
   for (int i = 0; i < r->nm; ++i) {
     const pb_model& m = *r->models[i];
     auto bytes = [&](uint32_t bins) {
-      if (r->ext) return sweep_smem_bytes(m.n, m.d, r->cons, r->max_col, bins);
-      return r->wgt ? general_smem_bytes(m.n, m.d, m.wgt, m.n_cp, (int)m.uph.size(), bins, units)
-                    : plain_smem_bytes(m.n, m.d, bins, units);
+      return r->ext ? sweep_smem_bytes(m.n, m.d, r->cons, r->max_col, bins) : word_smem(r, i, bins, units);
     };
     const uint32_t bins = r->L.ms[i].bins;
     const bool in = bins <= cap_bins && bytes(bins) <= kSweepSmemMax;
@@ -1387,13 +1395,14 @@ PB_API int pb_run_create(pb_model* const* models, const pb_run_cfg* cfgs, int n_
     x.seed = c.seed;
     x.ws = ws + r->L.ms[i].mh;
   }
+  int dev = 0, sms = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  r->full = r->total_groups > (uint32_t)sms;
   // Exact samplers: warps per CTA.  Samples are independent, so a CTA with
   // more warps hides more latency: as many as fit while the groups leave SMs
   // free, fewer when several CTAs share one.
   if (r->elim) {
-    int dev = 0, sms = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     r->elim_plain = !r->wgt;
     for (auto& c : r->cfgs) r->elim_plain = r->elim_plain && c.sampler == PB_ELIM;
     if (r->elim_plain) {
@@ -1412,8 +1421,7 @@ PB_API int pb_run_create(pb_model* const* models, const pb_run_cfg* cfgs, int n_
         for (int i = 0; i < n_models; ++i) b = std::max(b, bytes(i, w));
         return b;
       };
-      r->elim_full = r->total_groups > (uint32_t)sms;
-      int ew = r->elim_full ? 8 : 16;
+      int ew = r->full ? 8 : 16;
       while (ew > 1 && smem_for(ew) > kSweepSmemMax) --ew;
       r->elim_warps = ew;
       r->elim_smem = smem_for(ew);

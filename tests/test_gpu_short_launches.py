@@ -55,3 +55,19 @@ def test_uneven_models_in_one_launch(sweeps, monkeypatch):
                   [pbits.RunCfg(seed=s, chains=c) for *_, s, c, _ in what])
     r.sweeps(sweeps)
     _check([(w, r, i) for i, w in enumerate(what)], sweeps)
+
+
+@pytest.mark.parametrize("n,d,chains", [(3, 4, 100), (3, 4, 9760), (8, 16, 100), (12, 20, 64)])
+@pytest.mark.parametrize("lengths", [[1], [2, 3], [5], [8], [13], [24], [33]])
+def test_general_gates(n, d, chains, lengths):
+    g, mats = W.random_general_circuit(n, d, 6, frac_u=0.5)
+    r = pbits.Run([pbits.Model(n, d, g, 3.0, mats=mats)], [pbits.RunCfg(seed=5, chains=chains)])
+    for k in lengths:
+        r.sweeps(k)
+    ref = oracle.u_gibbs(n, d, g, mats, J=3.0, seed=5, chains=chains, sweeps=sum(lengths))
+    sums, cnt, valid, samples = r.phase_sums()
+    assert np.array_equal(pbits.unslice_state(r.get_state(), chains), ref["state"])
+    assert valid == ref["valid"] and samples == ref["samples"] and np.array_equal(cnt, ref["cnt"])
+    # the bound of a term, times the count
+    n_u = int(np.sum(g[:, 0] == W.U))
+    assert np.all(np.abs(sums - ref["sum"]) <= cnt * (3e-7 + n_u * 7.4e-10) + 1e-9)
