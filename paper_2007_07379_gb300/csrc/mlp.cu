@@ -486,7 +486,7 @@ cudaError_t transpose_bf16(const __nv_bfloat16* src, int R, int C, __nv_bfloat16
 // 16 K bytes apart (W2 in K-chunks of 64).
 struct Bf16Views {
   __nv_bfloat16 *W1, *W2, *W3, *W2t, *W3t, *W1p, *W2p, *W3p;
-  int kin, H, npad, n;
+  int kin, H, npad;
 };
 __device__ __forceinline__ uint32_t canonical_index(int r, int c, int K) {
   return (uint32_t)((r >> 3) * (K * 8) + (c >> 3) * 64 + (r & 7) * 8 + (c & 7));
@@ -710,7 +710,7 @@ pb::GemmArgs mm(const pb_mlp* p, const __nv_bfloat16* A, int lda, const __nv_bfl
 }
 
 pb::Bf16Views bf16_views(const pb_mlp* p) {
-  return {p->W1, p->W2, p->W3, p->W2t, p->W3t, p->W1p, p->W2p, p->W3p, p->kin, p->H, p->npad, p->n};
+  return {p->W1, p->W2, p->W3, p->W2t, p->W3t, p->W1p, p->W2p, p->W3p, p->kin, p->H, p->npad};
 }
 
 // bf16 copies of the fp32 master weights.
@@ -990,7 +990,7 @@ namespace pb {
 
 // Modes of the fused kernel:
 //   kFusedLogits  rows of x from global memory -> logits to global memory;
-//   kFusedLogQ    rows (chain c, layer j = k + blockIdx.y) built from the
+//   kFusedLogQ    rows (chain c, layer j of k .. d) built from the
 //                 per-chain words P -> lq[c d + j-1] = log q(P[c][j-1] | x);
 //   kFusedSample  rows (chain c, layer j) built from P (j == k) or Pn (j > k)
 //                 -> s'_j drawn from q into Pn[c][j-1], lqf[c] += log q(s'_j | x).
@@ -1010,8 +1010,9 @@ struct FusedArgs {
   float* lqf;
   const uint32_t* move_dev;
   const int* k_dev;  // per-chain modes: when set, the suffix start k is read here
-                     // (kFusedLogQ: layers k + blockIdx.y; kFusedSample: j = k,
-                     // jlast = d) and CTAs past layer d leave at once
+                     // (kFusedLogQ: layers k .. d, in the 128-row kernel layer
+                     // k + blockIdx.y; kFusedSample: j = k, jlast = d) and CTAs
+                     // without a layer leave at once
   uint32_t beta, k0, k1, group0;
   int n, d, k, j, jlast;  // kFusedSample: layers j .. jlast, one after the other
   // shared-memory layout (byte offsets; fused_layout) and W2 chunk buffers
@@ -1780,9 +1781,10 @@ cudaError_t mlp_fused_logq(pb_mlp* p, const uint32_t* P, uint32_t beta, int chai
   return cudaGetLastError();
 }
 
-// The same with the suffix start read from k_dev on the device (a grid over
-// all d layers; the CTAs of layers before k leave at once), so that one
-// captured graph serves every k.
+// The same with the suffix start read from k_dev on the device, so that one
+// captured graph serves every k: even shares of the suffix's (tile, layer)
+// pairs for the 64-row kernel; for the 128-row kernel a grid over all d layers,
+// whose CTAs past the suffix leave at once.
 cudaError_t mlp_fused_logq_dev(pb_mlp* p, const uint32_t* P, uint32_t beta, int chains,
                                const int* k_dev, float* lq, cudaStream_t st) {
   FusedArgs a = fused_args(p, chains);

@@ -184,9 +184,10 @@ constexpr size_t kSweepSmemMax = 226 * 1024;
 // Threads per sweep CTA in a run with general one-qubit gates (the general
 // instantiation is compiled for at most this many).
 constexpr int kSweepThreadsWgt = 512;
-// Bound on the threads of a plain run's sweep CTA (224 consumers, 352
-// producers and one more warp at most): up to 88 registers a thread, so that
-// two CTAs of the default 352 threads share an SM.
+// Launch bound of the plain sweep kernels: the largest that leaves a thread 88
+// registers (65,536 / 736), so that two CTAs of 352 threads share an SM.
+// Launches have 608 threads at most (224 consumers, 352 producers and one more
+// warp).
 constexpr int kSweepThreadsPlain = 736;
 
 // Plain runs work in periods of plain_period sweeps: about `units` p-bit
@@ -301,10 +302,16 @@ constexpr int kProducersMax = 352;
 // Plain runs: default CTA shape and period for `groups` chain groups of
 // models of up to npb p-bits (largest colour class maxcol) on a GPU of `sms`
 // SMs; smem(units): shared memory of a CTA with that period.
-// Two CTAs an SM where there are groups for them and they fit: the roles of
-// one hide the other's latencies (large workload, ms per 1e3 sweeps: 64
-// consumers + 256 producers, two CTAs, 17.2; 64 + 352, one CTA, 21.8, both
-// before the last 0.8 came off the shape that was kept).
+// Two CTAs an SM where there are groups for them and they fit beside the
+// histogram that smem counts: the roles of one hide the other's latencies
+// (large workload, ms per 1e3 sweeps: 64 consumers + 256 producers, two CTAs,
+// 17.2; 64 + 352, one CTA, 21.8, both before the last 0.8 came off the shape
+// that was kept).  A histogram of 1024 to 4096 bins takes that room (a CTA with
+// one would be alone), so full histograms of 10 to 12 qubits run one CTA an SM
+// although two fit with their counts in global memory (20 layers, 65,536
+// chains, ms per 1e3 sweeps, one CTA / two CTAs with global counts: 10 qubits
+// 6.65 / 5.94, 11 qubits 6.41 / 5.65, 12 qubits, whose counts are in global
+// memory either way, 6.72 / 5.96).
 // Otherwise one CTA an SM with a consumer per p-bit of the largest class, as
 // many producers as a period has tasks for and a longer period, whose tasks
 // spread more evenly over the warps (mid, ms per 1e4 sweeps: 4096 units

@@ -70,7 +70,8 @@ __global__ void bitonic_step_kernel(unsigned long long* __restrict__ keys, uint3
 // The stages with j < nb, for k = k0 .. k1: a CTA sorts or merges its nb keys
 // (nb >= 2, a power of two, at most kSortBlock) in shared memory.  A launch
 // for each stage was a launch's latency and a pass over the keys each: 36 of
-// them for 250 samples (0.1 ms), 231 for 1.4 million (1.6 ms).
+// them for 250 samples (0.1 ms of a 7.4 ms call), 231 for 1.4 million (1.6 ms
+// of 328, where the gain is within the noise of a call).
 __global__ void __launch_bounds__(1024) bitonic_local_kernel(unsigned long long* __restrict__ keys,
                                                              uint32_t nb, uint32_t k0, uint32_t k1) {
   __shared__ unsigned long long s[kSortBlock];
@@ -313,9 +314,8 @@ PB_API int pb_shor_columns(uint64_t N, uint64_t a, int n, const uint32_t* x, uin
   uint8_t* gend = reinterpret_cast<uint8_t*>(ws + L.gend);
   uint32_t* bounds = reinterpret_cast<uint32_t*>(ws + L.bounds);
   const unsigned long long K = 1ull << n;
-  cudaError_t e;
-  if ((e = cudaMemcpyAsync(dx, x, (size_t)T * 4, cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-      (e = cudaMemsetAsync(d_prob, 0, K * 8, st)) != cudaSuccess)
+  if (cudaMemcpyAsync(dx, x, (size_t)T * 4, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+      cudaMemsetAsync(d_prob, 0, K * 8, st) != cudaSuccess)
     return PB_ECUDA;
   const int tpb = 256;
   shor_modexp_kernel<<<(L.Tpad + tpb - 1) / tpb, tpb, 0, st>>>(dx, T, L.Tpad, N, a, keys, ys);

@@ -35,7 +35,9 @@
 // qubits, 32 layers, 65,536 chains, 1e3 sweeps) 41.9 -> 16.4, tiny (1e4
 // sweeps) 9.0 -> 1.6, 256 batched circuits (300 sweeps) 15.2 -> 4.35; with
 // general one-qubit gates, whose acceptance words are made ahead as well,
-// general_mid (35 coupled gates, 4096 chains, 2e3 sweeps) 6.63 -> 3.1.
+// general_mid (35 coupled gates, 4096 chains, 2e3 sweeps) 6.63 -> 3.1: there
+// 35 % of the slots are used, the other warps waiting at a period's end for
+// the last phase records (sincospif and FP64 shared atomics).
 #include <cuda_runtime.h>
 
 #include <type_traits>
