@@ -314,8 +314,9 @@ PB_API int pb_shor_columns(uint64_t N, uint64_t a, int n, const uint32_t* x, uin
   uint8_t* gend = reinterpret_cast<uint8_t*>(ws + L.gend);
   uint32_t* bounds = reinterpret_cast<uint32_t*>(ws + L.bounds);
   const unsigned long long K = 1ull << n;
-  if (cudaMemcpyAsync(dx, x, (size_t)T * 4, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-      cudaMemsetAsync(d_prob, 0, K * 8, st) != cudaSuccess)
+  cudaError_t e;
+  if ((e = cudaMemcpyAsync(dx, x, (size_t)T * 4, cudaMemcpyHostToDevice, st)) != cudaSuccess ||
+      (e = cudaMemsetAsync(d_prob, 0, K * 8, st)) != cudaSuccess)
     return PB_ECUDA;
   const int tpb = 256;
   shor_modexp_kernel<<<(L.Tpad + tpb - 1) / tpb, tpb, 0, st>>>(dx, T, L.Tpad, N, a, keys, ys);
