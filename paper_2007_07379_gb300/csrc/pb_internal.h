@@ -352,7 +352,9 @@ inline int plain_launch_producers(int npb, int ncp, uint32_t hist_bins, bool ful
   const bool apart = n_sweeps == (uint32_t)ps || (full && (ncp == 0 || n_sweeps <= 3u * (uint32_t)ps));
   const int tasks = apart ? std::max(std::max(start, finish), record) : start + finish + record;
   const int threads = std::max(npb, (int)hist_bins / 8);
-  return std::max(32, std::max(32 * ((tasks + 1) / 2), (threads + 31) / 32 * 32 - cons - 32));
+  // (one more warp than producers, which counts where the groups fill the GPU)
+  const int warps = full ? (tasks - 1) / 2 : (tasks + 1) / 2;
+  return std::max(full ? 0 : 32, std::max(32 * warps, (threads + 31) / 32 * 32 - cons - 32));
 }
 }  // namespace pb
 

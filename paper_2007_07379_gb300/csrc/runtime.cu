@@ -990,10 +990,10 @@ int persistent_grid(const pb_run* r, int threads, size_t smem) {
 
 // Shape of a launch of n sweeps on the word kernels: the run's, smaller where n is
 // small, so that more CTAs share an SM: their set-up is most of such a launch
-// (3 qubits, 4 layers: one sweep of 65,536 chains 39.7 -> 19.6 us, of 256
-// circuits of 256 chains in one persistent launch 48.5 -> 26.0; eight sweeps
-// 70.3 -> 33.7 and 56.8 -> 34.0; with half of the gates general, one sweep of
-// the 65,536 chains 118 -> 58).
+// (3 qubits, 4 layers: one sweep of 65,536 chains 39.6 -> 19.2 us, of 256
+// circuits of 256 chains in one persistent launch 48.0 -> 21.7; eight sweeps
+// 70.3 -> 27.3 and 76.8 -> 32.6; with half of the gates general, one sweep of
+// the 65,536 chains 119 -> 50).
 struct PlainLaunch {
   int prod, units, grid;
   size_t smem;
