@@ -338,7 +338,9 @@ PB_API int pb_run_stats(pb_run* run, pb_run_stats_t* stats);
  * table runs, one more producer elsewhere); blocks_per_sm
  * caps the persistent grid of batched runs (0 = as many as fit).  A run
  * with PB_U models takes at most 512 threads (consumers + producers + 32;
- * PB_ERANGE otherwise).  The results do not depend on the shape. */
+ * PB_ERANGE otherwise).  A launch of few sweeps takes fewer producers, and a
+ * persistent one more CTAs, than the shape says.  The results do not depend
+ * on the shape. */
 PB_API int pb_run_set_shape(pb_run* run, int consumers, int producers, int blocks_per_sm);
 PB_API int pb_run_get_shape(const pb_run* run, int* consumers, int* producers, int* blocks_per_sm,
                             int* grid);
